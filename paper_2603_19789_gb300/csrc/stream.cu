@@ -4,7 +4,7 @@
 // split storages, the D2Q9 lattice (Sec. II.C, isotropy) and the spatially varying diffusion
 // (the flux form of vard.cu).
 //
-// A warp owns a strip of kStCols columns and a segment of kStSeg rows and walks down it.  The
+// A warp owns a strip of kStCols columns and a segment of rows and walks down it.  The
 // rows of the planes its update reads arrive by cp.async in a ring of Cell::kRing rows in
 // shared memory, kRing - 3 rows ahead of the rows being read, so every plane is read from
 // global memory once per step (the two rows beyond a segment's ends a second time) and no
@@ -38,7 +38,6 @@ namespace {
 
 constexpr int kStCols = 64;     // columns per strip: two per lane
 constexpr int kStStride = 72;   // floats per plane row in the ring
-constexpr int kStSeg = 128;     // rows per segment
 
 // Column index of ring column x: link_index for the halo columns -1 and nx; columns
 // further out (the unused tail of a strip past the grid) read a clamped in-range cell.
@@ -68,7 +67,7 @@ __device__ __forceinline__ float2 ld2(const float* p, int i) { return make_float
 
 template <class Cell>
 __global__ void __launch_bounds__(32 * Cell::kWarps, Cell::kMinBlocks)
-    stream_kernel(const GridView g, const Cell cell, const int nstrips, const int nitems) {
+    stream_kernel(const GridView g, const Cell cell, const int nstrips, const int nitems, const int seg) {
   constexpr int NP = Cell::kPlanes, NH = Cell::kHaloPlanes, RING = Cell::kRing;
   constexpr int ROWF = NP * kStStride;
   static_assert(NH <= 16 && NH <= NP && RING >= 4, "ring shape");
@@ -79,9 +78,10 @@ __global__ void __launch_bounds__(32 * Cell::kWarps, Cell::kMinBlocks)
   float* ring = st_smem + (size_t)warp * (RING * ROWF);
   const int strip = item % nstrips;
   const int64_t xs = (int64_t)strip * kStCols;
-  const int64_t y0 = (int64_t)(item / nstrips) * kStSeg;
-  const int64_t y1 = y0 + kStSeg < g.ny ? y0 + kStSeg : g.ny;
+  const int64_t y0 = (int64_t)(item / nstrips) * seg;
+  const int64_t y1 = y0 + seg < g.ny ? y0 + seg : g.ny;
   const bool vec = xs + kStCols <= g.nx;
+  const int w = vec ? kStCols : (int)(g.nx - xs);
   const int64_t xl = st_col(xs - 1, g), xr = st_col(xs + kStCols, g);
   const int64_t q0 = y0 - 1;  // first logical row in the ring
   auto issue = [&](int64_t q) {  // rows q0 .. y1 (one beyond the segment on each side)
@@ -103,10 +103,20 @@ __global__ void __launch_bounds__(32 * Cell::kWarps, Cell::kMinBlocks)
             cp_async4(dst + f * kStStride + (left ? 3 : 4 + kStCols), cell.src(f, g) + row + xh);
         }
       } else {
-        for (int u = lane; u < NP * (kStCols + 2); u += 32) {
-          const int f = u / (kStCols + 2), i = 3 + u % (kStCols + 2);
-          const int64_t xc = st_col(xs - 4 + i, g);
-          if (SSLBM_IN(xc, 1, g.nx, 4)) cp_async4(dst + f * kStStride + i, cell.src(f, g) + row + xc);
+        // w columns of the strip lie in the grid: whole groups of 4 as vectors, then the left halo
+        // (j = 0), the rest and the right halo (column w) one by one
+        for (int u = lane; u < NP * 16; u += 32) {
+          const int f = u >> 4, part = u & 15;
+          if (4 * part + 3 < w && SSLBM_IN(xs + 4 * part, 4, g.nx, 4))
+            cp_async16(dst + f * kStStride + 4 + 4 * part, cell.src(f, g) + row + xs + 4 * part);
+        }
+        for (int u = lane; u < NP * 8; u += 32) {
+          const int f = u >> 3, j = u & 7;
+          const int c = j == 0 ? -1 : (w & ~3) + j - 1;
+          if (c <= w && (f < NH || (c >= 0 && c < w))) {
+            const int64_t xc = st_col(xs + c, g);
+            if (SSLBM_IN(xc, 1, g.nx, 7)) cp_async4(dst + f * kStStride + 4 + c, cell.src(f, g) + row + xc);
+          }
         }
       }
     }
@@ -147,7 +157,7 @@ __global__ void __launch_bounds__(32 * Cell::kWarps, Cell::kMinBlocks)
 // warps per SM) 77.3 GLUPS; 8 and 4 warps 76.5; 7 and 3 warps 68.3; 6 and 4 warps 61.3; 10
 // and 2 warps (three CTAs per SM) 66.6.
 struct KahanCell {
-  static constexpr int kPlanes = 10, kHaloPlanes = 9, kRing = 8, kWarps = 2, kMinBlocks = 4;
+  static constexpr int kPlanes = 10, kHaloPlanes = 9, kRing = 8, kWarps = 2, kMinBlocks = 4, kSeg = 64;
   static constexpr bool kPacked = false;
   const float* in;
   float* out;
@@ -203,7 +213,7 @@ __device__ __forceinline__ void st2(float* o, int64_t plane_off, float2 v, bool 
 // 6 CTAs 37.7.  The laplacian with one normalisation (dw::lap5_diff) instead of seven
 // add_abs: 43.8, the same errors (the native FP64 kernel: 11.9).
 struct DwCell {
-  static constexpr int kPlanes = 10, kHaloPlanes = 8, kRing = 4, kWarps = 4, kMinBlocks = 4;
+  static constexpr int kPlanes = 10, kHaloPlanes = 8, kRing = 4, kWarps = 4, kMinBlocks = 4, kSeg = 40;
   static constexpr bool kPacked = true;
   const float* in;
   float* out;
@@ -259,7 +269,7 @@ struct DwCell {
 template <int MODE>
 struct D2q5Cell {
   static constexpr int kPlanes = mode_planes<MODE>(), kHaloPlanes = kPlanes - 1;
-  static constexpr int kRing = 8, kWarps = 4, kMinBlocks = 4;
+  static constexpr int kRing = 8, kWarps = 4, kMinBlocks = 4, kSeg = 40;
   static constexpr bool kPacked = true;
   static constexpr int kD = kPlanes - 1;  // ring plane of D
   const float* in;
@@ -312,7 +322,7 @@ struct D2q5Cell {
 // own value (halfway bounce-back); the cells on the domain's edge take the links one by one
 // from the ring with that substitution.
 struct D2q9Cell {
-  static constexpr int kPlanes = 5, kHaloPlanes = 4, kRing = 8, kWarps = 4, kMinBlocks = 4;
+  static constexpr int kPlanes = 5, kHaloPlanes = 4, kRing = 8, kWarps = 4, kMinBlocks = 4, kSeg = 40;
   static constexpr bool kPacked = true;
   const float* in;
   float* out;
@@ -398,7 +408,7 @@ struct D2q9Cell {
 // and summed as ((+x) + (-x)) + ((+y) + (-y)) (the order of vard.cu), then seird_cell.  Ring
 // planes: S, E, I, R, kx (x neighbours), ky, D.
 struct VardCell {
-  static constexpr int kPlanes = 7, kHaloPlanes = 5, kRing = 8, kWarps = 4, kMinBlocks = 3;
+  static constexpr int kPlanes = 7, kHaloPlanes = 5, kRing = 8, kWarps = 4, kMinBlocks = 3, kSeg = 64;
   static constexpr bool kPacked = true;
   const float* in;
   const float* kx;
@@ -446,10 +456,34 @@ struct VardCell {
   }
 };
 
-// One launch: a warp per (strip, 128-row segment).  Cutting the rows so that the items fill
-// the resident warps exactly once (segments of ~900 rows at 8192^2, no tail wave) measured
-// slower at 8192^2 for every cell -- 65.2 against 76.3 GLUPS for the Kahan storage, 114.9
-// against 141.6 for D2Q9 -- so the grid keeps short segments and several waves.
+int sm_count(int dev) {
+  static std::atomic<int> cache[64];
+  const int i = dev & 63;
+  int v = cache[i].load(std::memory_order_relaxed);
+  if (!v && cudaDeviceGetAttribute(&v, cudaDevAttrMultiProcessorCount, dev) == cudaSuccess)
+    cache[i].store(v, std::memory_order_relaxed);
+  return v > 0 ? v : 1;
+}
+
+// Rows per segment, a warp per (strip, segment): whole waves of the `warps` that are resident
+// at once, as few as keep a segment within cap rows.  A segment reads two rows more than it
+// writes (from L2 mostly) and computes none twice, so short ones cost little: below one wave
+// the rows are simply spread over the resident warps.  With 128-row segments on every grid,
+// as before, a 1024^2 step left most SMs idle: 154 us for the double word, 57 for FP32, 90
+// for Kahan; now 26.7, 10.3 and 18.4, and 200^2 takes 6.2 us instead of 440, 176 and 338.  On
+// large grids a partial last wave cost as much: 2048^2 with 40 rows exactly takes 55 us for
+// the varying diffusion, with a whole wave (36 rows) 41.  One long wave is slow again, all warps
+// then stream from rows far apart: 4096^2 FP32 at 54 rows 123 us, at 36 rows 117, at 128 rows
+// 140; Kahan and the varying diffusion (fewer resident warps) still gain at 64 rows (228 and
+// 144 us at 4096^2 against 231 and 147 at 40).  8192^2 FP32: 428 us (128 rows: 450).
+int seg_rows(int64_t ny, int64_t nstrips, int64_t warps, int cap) {
+  const int64_t waves = (ny * nstrips + cap * warps - 1) / (cap * warps);
+  int64_t nseg = waves * warps / nstrips;
+  if (nseg < 1) nseg = 1;
+  const int64_t rows = (ny + nseg - 1) / nseg;
+  return (int)(rows < cap ? rows : cap);
+}
+
 template <class Cell>
 cudaError_t launch_stream(const GridView& g, const Cell& cell, cudaStream_t s) {
   constexpr size_t smem = sizeof(float) * Cell::kRing * Cell::kPlanes * kStStride * Cell::kWarps;
@@ -462,11 +496,12 @@ cudaError_t launch_stream(const GridView& g, const Cell& cell, cudaStream_t s) {
     done.fetch_or(1ull << (dev & 63), std::memory_order_release);
   }
   const int64_t nstrips = (g.nx + kStCols - 1) / kStCols;
-  const int64_t items = nstrips * ((g.ny + kStSeg - 1) / kStSeg);
+  const int seg = seg_rows(g.ny, nstrips, (int64_t)Cell::kMinBlocks * Cell::kWarps * sm_count(dev), Cell::kSeg);
+  const int64_t items = nstrips * ((g.ny + seg - 1) / seg);
   if (items > 0x7fffffffLL - Cell::kWarps) return cudaErrorInvalidConfiguration;
   if (items == 0) return cudaSuccess;
   stream_kernel<Cell><<<(unsigned)((items + Cell::kWarps - 1) / Cell::kWarps), 32 * Cell::kWarps, smem, s>>>(
-      g, cell, (int)nstrips, (int)items);
+      g, cell, (int)nstrips, (int)items, seg);
   return cudaGetLastError();
 }
 
