@@ -27,8 +27,10 @@
 #include <cstdarg>
 #include <cstdio>
 #include <new>
+#include <utility>
 #include <vector>
 
+#include "fno_bwd.cuh"
 #include "fno_fused.cuh"
 #include "fno_gemm.cuh"
 #include "handles_access.cuh"
@@ -313,6 +315,16 @@ __global__ void conserve_kernel(float* __restrict__ y, const double* __restrict_
   }
 }
 
+// per sample: seed[b] = lambda = sum(dy y) / sum y, seed[B + b] = sigma of E and I
+__global__ void seed_lambda_kernel(const double* __restrict__ sums, const float* __restrict__ x,
+                                   float* __restrict__ seed, int B, int64_t P) {
+  const int b = blockIdx.x * blockDim.x + threadIdx.x;
+  if (b >= B) return;
+  const double sy = sums[2 * b + 1];
+  seed[b] = sy > 0.0 ? (float)(sums[2 * b] / sy) : 0.f;
+  seed[B + b] = scale_from_e(x[((int64_t)b * kCin + 7) * P]);
+}
+
 // dd = sigma r [y > 0] (dy - lambda), lambda = sum(dy y) / sum y: the derivative with respect to
 // delta = Q2 p + q2 through y = r v, r = sum u / sum v, v_c = sigma_c max(x_c + delta_c, 0)
 // (dL/dv = r (dy - sum(dy v) / sum v), and sum(dy v) / sum v = sum(dy y) / sum y)  (b = blockIdx.y)
@@ -446,59 +458,94 @@ __global__ void dhat_combine_adj_kernel(const float* __restrict__ dG, const floa
   }
 }
 
-// per sample: sums[3b] += sum (y - t), sums[3b+1] += sum t, sums[3b+2] += sum max(-y, 0)
+// hi + lo <- hi + lo + x, hi + x exactly (Knuth's TwoSum): about twice FP32's precision without
+// FP64 arithmetic, of which this GPU has little
+__device__ __forceinline__ void two_sum_add(float& hi, float& lo, float x) {
+  const float s = __fadd_rn(hi, x);
+  const float bp = __fsub_rn(s, hi);
+  lo = __fadd_rn(lo, __fadd_rn(__fsub_rn(hi, __fsub_rn(s, bp)), __fsub_rn(x, bp)));
+  hi = s;
+}
+
+// per sample b = blockIdx.y: sums[3b] += sum (y - t), sums[3b+1] += sum t, sums[3b+2] += sum max(-y, 0).
+// Bound by its 8 bytes per value: every value added in FP64 took 84 us at B = 16, 256 x 256 (42 MB);
+// 21 us
+// with TwoSum pairs.
 __global__ void loss_sums_kernel(const float* __restrict__ y, const float* __restrict__ tgt,
                                  double* __restrict__ sums, int64_t P5) {
+  __shared__ double sh[64];
   const int64_t b = blockIdx.y;
-  double se = 0.0, st = 0.0, sn = 0.0;
-  for (int64_t t = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; t < P5;
-       t += (int64_t)gridDim.x * blockDim.x) {
-    const float tv = tgt[b * P5 + t], yv = y[b * P5 + t];
-    se += (double)(yv - tv);
-    st += tv;
-    sn += yv < 0.f ? -(double)yv : 0.0;
+  float eh = 0.f, el = 0.f, th = 0.f, tl = 0.f, nh = 0.f, nl = 0.f;
+  auto take = [&](float yv, float tv) {
+    two_sum_add(eh, el, yv - tv);
+    two_sum_add(th, tl, tv);
+    if (yv < 0.f) two_sum_add(nh, nl, -yv);
+  };
+  const float* yb = y + b * P5;
+  const float* tb = tgt + b * P5;
+  const int64_t stride = (int64_t)gridDim.x * blockDim.x, i0 = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+  if ((P5 & 3) == 0 && ((reinterpret_cast<uintptr_t>(yb) | reinterpret_cast<uintptr_t>(tb)) & 15) == 0) {
+    for (int64_t i = i0; i < P5 / 4; i += stride) {
+      const float4 yv = reinterpret_cast<const float4*>(yb)[i], tv = reinterpret_cast<const float4*>(tb)[i];
+      take(yv.x, tv.x), take(yv.y, tv.y), take(yv.z, tv.z), take(yv.w, tv.w);
+    }
+  } else {
+    for (int64_t i = i0; i < P5; i += stride) take(yb[i], tb[i]);
   }
-  for (int off = 16; off > 0; off >>= 1) {
-    se += __shfl_down_sync(0xffffffffu, se, off);
-    st += __shfl_down_sync(0xffffffffu, st, off);
-    sn += __shfl_down_sync(0xffffffffu, sn, off);
-  }
-  if ((threadIdx.x & 31) == 0) {
-    atomicAdd(sums + 3 * b, se);
-    atomicAdd(sums + 3 * b + 1, st);
-    atomicAdd(sums + 3 * b + 2, sn);
-  }
+  block_add2((double)eh + (double)el, (double)th + (double)tl, sums + 3 * b, sh);
+  __syncthreads();
+  block_add1((double)nh + (double)nl, sums + 3 * b + 2, sh);
 }
 
 // The training loss (N = B * 5 * P):
 //   mse_w = (1/N) sum ((y - t) / sigma_c)^2,  r_b = sum(y_b - t_b) / sum t_b,
 //   n_b = sum max(-y_b, 0) / sum t_b,  L = mse_w + lm mean_b r_b^2 + ln mean_b n_b^2;
-// dy = dL/dy; loss receives mse_w.  sums may be NULL when lm = ln = 0.
+// dy = dL/dy; loss receives mse_w.  sums may be NULL when lm = ln = 0.  b = blockIdx.y: the
+// sample's constants are formed once per block and the squares added as TwoSum pairs, each
+// product with its FMA remainder.  Bound by its 12 bytes per value; with the constants formed and
+// the squares added in FP64 per value, as before, 765 us at B = 16, 256 x 256 (63 MB);
+// now 31.
 __global__ void loss_kernel(const float* __restrict__ y, const float* __restrict__ tgt,
                             const float* __restrict__ x, float* __restrict__ dy, double* __restrict__ loss,
                             int64_t N, int64_t P, const double* __restrict__ sums, float lm, float ln, int B) {
-  double acc = 0.0;
-  const float inv = 1.f / (float)N;
-  for (int64_t t = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; t < N;
-       t += (int64_t)gridDim.x * blockDim.x) {
-    const int64_t b = t / (5 * P);
-    const int c = (int)((t - b * 5 * P) / P);
-    const float d = y[t] - tgt[t];
-    const float rs = (c == 1 || c == 2) ? 1.f / scale_from_e(x[(b * kCin + 7) * P]) : 1.f;
-    const float dn = d * rs;
-    float g = 2.f * dn * rs * inv;
-    if (sums) {
-      const double st = sums[3 * b + 1];
-      if (st != 0.0) {
-        g += (float)(2.0 * lm / B * (sums[3 * b] / st) / st);
-        if (y[t] < 0.f) g -= (float)(2.0 * ln / B * (sums[3 * b + 2] / st) / st);
-      }
-    }
-    dy[t] = g;
-    acc += (double)dn * dn;
+  __shared__ double sh[64];
+  __shared__ float gsh[2];
+  const int64_t b = blockIdx.y;
+  const float inv = 1.f / (float)N, rsg = 1.f / scale_from_e(x[(b * kCin + 7) * P]);
+  if (threadIdx.x == 0) {  // one thread: the FP64 divisions in every thread took 45 us
+    const double st = sums ? sums[3 * b + 1] : 0.0;
+    gsh[0] = st != 0.0 ? (float)(2.0 * lm / B * (sums[3 * b] / st) / st) : 0.f;
+    gsh[1] = st != 0.0 ? (float)(2.0 * ln / B * (sums[3 * b + 2] / st) / st) : 0.f;
   }
-  for (int off = 16; off > 0; off >>= 1) acc += __shfl_down_sync(0xffffffffu, acc, off);
-  if ((threadIdx.x & 31) == 0) atomicAdd(loss, acc / (double)N);
+  __syncthreads();
+  const float gm = gsh[0], gn = gsh[1];
+  float hi = 0.f, lo = 0.f;
+  const int64_t stride = (int64_t)gridDim.x * blockDim.x, i0 = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+  for (int c = 0; c < 5; ++c) {
+    const float rs = (c == 1 || c == 2) ? rsg : 1.f;
+    const float* yb = y + (b * 5 + c) * P;
+    const float* tb = tgt + (b * 5 + c) * P;
+    float* db = dy + (b * 5 + c) * P;
+    auto one = [&](float yv, float tv) {
+      const float dn = (yv - tv) * rs;
+      const float sq = __fmul_rn(dn, dn);
+      two_sum_add(hi, lo, sq);
+      lo = __fadd_rn(lo, __fmaf_rn(dn, dn, -sq));
+      float g = 2.f * dn * rs * inv + gm;
+      if (yv < 0.f) g -= gn;
+      return g;
+    };
+    if ((P & 3) == 0 && ((reinterpret_cast<uintptr_t>(yb) | reinterpret_cast<uintptr_t>(tb) |
+                          reinterpret_cast<uintptr_t>(db)) & 15) == 0) {
+      for (int64_t i = i0; i < P / 4; i += stride) {
+        const float4 yv = reinterpret_cast<const float4*>(yb)[i], tv = reinterpret_cast<const float4*>(tb)[i];
+        reinterpret_cast<float4*>(db)[i] = make_float4(one(yv.x, tv.x), one(yv.y, tv.y), one(yv.z, tv.z), one(yv.w, tv.w));
+      }
+    } else {
+      for (int64_t i = i0; i < P; i += stride) db[i] = one(yb[i], tb[i]);
+    }
+  }
+  block_add1(((double)hi + (double)lo) / (double)N, loss, sh);
 }
 
 // Adam (decoupled weight decay), then refresh the BF16 copy used as GEMM operand
@@ -1117,6 +1164,73 @@ int forward_impl(sslbm_fno* f, int B, const float* x, float* y, int store) {
   return st;
 }
 
+// the fused backward pass (fno_bwd.cu), from the seed's sums on
+int backward_fused(sslbm_fno* f, int B, const float* x, const float* dy, const double* sums) {
+  namespace F = sslbm::fno_fused;
+  const Layout& L = f->L;
+  const int W = L.W, m = L.m, n = L.n;
+  float* g = f->grad();
+  F::BwdArgs a{};
+  a.B = B;
+  a.x = x;
+  a.F = f->Fx();
+  a.dG1 = f->at<float>(f->bu.h1);
+  a.dH1 = f->at<float>(f->bu.h1);
+  a.scale = 1.f / ((float)n * (float)n);
+  a.dy = dy;
+  a.y = f->at<float>(f->bu.ycache);
+  float* seed = f->at<float>(f->bu.mscale);
+  seed_lambda_kernel<<<(B + 31) / 32, 32, 0, f->stream>>>(sums, x, seed, B, L.P);
+  CK(cudaGetLastError(), "seed lambda");
+  a.seed = seed;
+  a.ratio = f->at<float>(f->bu.ratio);
+  a.zp = f->at<bf16>(f->bu.zp);
+  a.p = f->at<bf16>(f->bu.p);
+  a.hL = f->h(L.L, B);
+  a.Q1 = f->theta16() + L.off_Q1;
+  a.Q2 = f->theta16() + L.off_Q2;
+  a.gQ1 = g + L.off_Q1;
+  a.gq1 = g + L.off_q1;
+  a.gQ2 = g + L.off_Q2;
+  a.gq2 = g + L.off_q2;
+  float* dz = f->at<float>(f->bu.f32a);
+  float* other = f->at<float>(f->bu.f32b);
+  a.dz = dz;
+  a.hprev = f->h(L.L - 1, B);
+  a.gW = g + L.off_B[L.L - 1];
+  a.gb = g + L.off_b[L.L - 1];
+  CK(F::launch_bwd_row(F::BWD_LAST, W, m, L.H, n, a, f->stream), "fused backward, projection");
+  for (int l = L.L; l >= 1; --l) {
+    F::BwdSpectral sp{};
+    sp.dG1 = a.dG1;
+    sp.Fy = f->Fy();
+    sp.Fyi = f->Fyi();
+    sp.hat = f->hat(l, B);
+    sp.R = f->theta() + L.off_R[l - 1];
+    sp.dG = f->at<float>(f->bu.dg);
+    sp.dhat = f->at<float>(f->bu.tt);
+    sp.dR = g + L.off_R[l - 1];
+    sp.dH1 = a.dG1;
+    CK(F::launch_bwd_spectral(W, m, L.H, B, n, sp, f->stream), "fused backward, spectral");
+    a.dzin = dz;
+    a.Bl = f->theta16() + L.off_B[l - 1];
+    if (l > 1) {
+      a.z = f->z(l - 1, B);
+      a.hprev = f->h(l - 2, B);
+      a.dz = other;
+      a.gW = g + L.off_B[l - 2];
+      a.gb = g + L.off_b[l - 2];
+      CK(F::launch_bwd_row(F::BWD_MID, W, m, L.H, n, a, f->stream), "fused backward, layer");
+      std::swap(dz, other);
+    } else {
+      a.gW = g + L.off_A0;
+      a.gb = g + L.off_a0;
+      CK(F::launch_bwd_row(F::BWD_FIRST, W, m, L.H, n, a, f->stream), "fused backward, lift");
+    }
+  }
+  return SSLBM_OK;
+}
+
 int backward_impl(sslbm_fno* f, int B, const float* x, const float* dy_out) {
   const Layout& L = f->L;
   const int W = L.W;
@@ -1132,6 +1246,7 @@ int backward_impl(sslbm_fno* f, int B, const float* x, const float* dy_out) {
   dim3 sgrid((unsigned)std::min<int64_t>(64, (5 * P + kThreads - 1) / kThreads), B);
   seed_sums_kernel<<<sgrid, kThreads, 0, f->stream>>>(dy_out, ycache, sums, 5 * P);
   CK(cudaGetLastError(), "seed sums");
+  if (sslbm::fno_fused::supported(W, L.m, L.H, L.n)) return backward_fused(f, B, x, dy_out, sums);
   scale_dy_kernel<<<dim3(rows_grid(P), B), kThreads, 0, f->stream>>>(dy_out, x, ycache, sums,
                                                                     f->at<float>(f->bu.ratio), dy, P);
   CK(cudaGetLastError(), "output scale");
@@ -1347,7 +1462,8 @@ int sslbm_fno_train_step(sslbm_fno* f, int batch, const float* x, const float* t
     loss_sums_kernel<<<grid, kThreads, 0, f->stream>>>(y_scratch, target, sums, P5);
     CK(cudaGetLastError(), "loss sums");
   }
-  loss_kernel<<<blocks_for(N), kThreads, 0, f->stream>>>(y_scratch, target, x, dy_scratch, dl, N, f->L.P, sums,
+  loss_kernel<<<dim3((unsigned)std::min<int64_t>(64, (f->L.P + 4 * kThreads - 1) / (4 * kThreads)), batch), kThreads, 0,
+                f->stream>>>(y_scratch, target, x, dy_scratch, dl, N, f->L.P, sums,
                                                          f->mass_weight, f->neg_weight, batch);
   CK(cudaGetLastError(), "loss");
   if ((st = backward_impl(f, batch, x, dy_scratch))) return st;
