@@ -224,7 +224,9 @@ int sslbm_set_diffusivity_scale(sslbm_handle* h, const void* kx, const void* ky,
  * Several steps are fused per pass over memory (temporal blocking, depth set by
  * sslbm_set_blocking or sslbm_autotune; D2Q5 in every FP32 storage, D2Q9 and varying
  * diffusion in FP32); n steps
- * take ceil(n / depth) passes whose depths differ by at most one.  Results do not depend on
+ * take ceil(n / depth) passes whose depths differ by at most one.  Under the default blocking,
+ * small grids of the FP32 and FP32_DEV storages, of D2Q9 and of the varying diffusion take
+ * passes of their own depth, chosen by the grid and n.  Results do not depend on
  * the depth: every depth performs the same floating-point operations in the same order.
  * Enqueues on the handle's stream and returns. */
 int sslbm_step(sslbm_handle* h, int64_t n);

@@ -18,6 +18,7 @@
 
 #include "bounds.cuh"
 #include "sslbm_internal.cuh"
+#include "tile.cuh"
 #include "variants.cuh"
 
 using sslbm::Coeffs;
@@ -153,6 +154,7 @@ struct sslbm_handle {
   int s_cur = 0, b_cur = 0;
   int64_t s_steps = 0, b_steps = 0;
   int depth = 1, seg_rows = 0;
+  bool auto_blocking = true;  // the default blocking, or an autotuned choice of the tile passes
   int seg_cache[SSLBM_MAX_DEPTH + 1] = {0};
   bool fuse_diag = false;   // sslbm_set_fused_diagnostics
   bool diag_ready = false;  // diag_result() holds the diagnostics of the current SSLBM state
@@ -233,6 +235,13 @@ static cudaError_t launch_pass(sslbm_handle* h, int k, int seg) {
               : sslbm::launch_sslbm_step1(h->g.precision, h->gv, h->coeffs(), h->s_buf[h->s_cur], out, h->stream);
   return q9 ? sslbm::launch_sslbm9_blocked(h->gv, &h->cf, h->s_buf[h->s_cur], out, k, seg, h->stream)
             : sslbm::launch_sslbm_blocked(h->g.precision, h->gv, &h->cf, h->s_buf[h->s_cur], out, k, seg, h->stream);
+}
+
+// One register-tile pass of k steps (tile.cu), the same buffers.
+static cudaError_t launch_tile_pass(sslbm_handle* h, int nr, int k) {
+  const char* ky = h->kappa ? h->kappa + h->L.plane_bytes : nullptr;
+  return sslbm::launch_tile(h->g.lattice, h->g.precision, h->gv, &h->cf, h->s_buf[h->s_cur], h->s_buf[1 - h->s_cur],
+                            h->kappa, ky, nr, k, h->stream);
 }
 
 static int default_seg(const sslbm_handle* h, int k) {
@@ -545,10 +554,27 @@ int sslbm_step(sslbm_handle* h, int64_t n) {
   if (h->g.lattice == SSLBM_LATTICE_D2Q5_VARD && !h->kappa_ok)
     return fail(SSLBM_ERR_BAD_ARG, "the diffusivity scale fields are not set (sslbm_set_diffusivity_scale)");
   const bool blocked = can_block(h);
+  bool tiles = blocked && h->auto_blocking && !h->fuse_diag;
   if (n > 0) h->diag_ready = false;
   while (n > 0) {
     int k = 1;
     cudaError_t e;
+    if (tiles && n > 1) {
+      // a small grid under the default blocking: register-tile passes, their depths differing by at
+      // most one as below
+      sslbm::TilePlan plan{0, 0};
+      if (sslbm::tile_plan(h->g.lattice, h->g.precision, h->gv, n, &plan)) {
+        const int64_t passes = (n + plan.depth - 1) / plan.depth;
+        k = (int)((n + passes - 1) / passes);
+        e = launch_tile_pass(h, plan.nr, k);
+        if (e != cudaSuccess) return cuda_fail(e, "SSLBM step launch");
+        h->s_cur = 1 - h->s_cur;
+        h->s_steps += k;
+        n -= k;
+        continue;
+      }
+      tiles = false;
+    }
     if (blocked && h->depth > 1 && n > 1) {
       // depth >= 2: the temporal-blocked kernel; a single step uses the one-step kernel,
       // which produces the same bits.  The n steps take ceil(n / depth) passes whose depths
@@ -665,12 +691,12 @@ int sslbm_debug_bounds(long long* count, long long* value, long long* limit, int
   int (*const take[])(sslbm::OobRecord*) = {sslbm::oob_take_kernels, sslbm::oob_take_ensemble, sslbm::oob_take_bgk,
                                             sslbm::oob_take_io, sslbm::oob_take_stream,
                                             sslbm::oob_take_d2q9, sslbm::oob_take_d2q9a, sslbm::oob_take_vard,
-                                            sslbm::oob_take_kahan, sslbm::oob_take_diag};
-  const int tu_site[] = {0, 100, 200, 300, 400, 500, 600, 700, 800, 900};  // offset by translation unit
+                                            sslbm::oob_take_kahan, sslbm::oob_take_diag, sslbm::oob_take_tile};
+  const int tu_site[] = {0, 100, 200, 300, 400, 500, 600, 700, 800, 900, 1100};  // offset by translation unit
   unsigned long long total = 0;
   sslbm::OobRecord first{};
   int first_site = -1;
-  for (int i = 0; i < 10; ++i) {
+  for (int i = 0; i < 11; ++i) {
     sslbm::OobRecord r{};
     if (take[i](&r) != 0) return fail(SSLBM_ERR_CUDA, "reading the bounds record of unit %d", i);
     if (r.count && first_site < 0) {
@@ -836,6 +862,7 @@ int sslbm_set_blocking(sslbm_handle* h, int k, int seg_rows) {
                 "temporal blocking is provided for the FP32 storages on D2Q5 and for FP32 on D2Q9 "
                 "and the varying-diffusion lattice");
   h->depth = k == 0 ? (blocked ? 4 : 1) : k;
+  h->auto_blocking = k == 0 && seg_rows == 0;
   if (seg_rows > 0 && seg_rows < 4 * h->depth) seg_rows = 4 * h->depth;
   h->seg_rows = seg_rows;
   return SSLBM_OK;
@@ -853,6 +880,7 @@ struct TuneKey {
 struct TuneResult {
   int depth, seg_rows;
   double ms_per_step;
+  bool tiles;  // the tile passes of the default blocking
 };
 std::mutex g_tune_mu;
 std::map<TuneKey, TuneResult> g_tune_cache;
@@ -872,7 +900,7 @@ int sslbm_autotune(sslbm_handle* h, double budget_ms, int* depth_out, int* seg_o
     return fail(SSLBM_ERR_BAD_ARG, "the diffusivity scale fields are not set (sslbm_set_diffusivity_scale)");
   DeviceGuard dg(h->device);
   const TuneKey key{h->device, h->g.precision, h->g.lattice, h->g.bc, h->g.nx, h->g.ny};
-  TuneResult best{1, 0, 0.0};
+  TuneResult best{1, 0, 0.0, false};
   bool cached = false;
   {
     std::lock_guard<std::mutex> lock(g_tune_mu);
@@ -883,9 +911,12 @@ int sslbm_autotune(sslbm_handle* h, double budget_ms, int* depth_out, int* seg_o
     }
   }
   if (!cached) {
+    // (depth, segment rows); the tile passes of a small grid as (depth, -rows per warp)
     std::vector<std::pair<int, int>> cand;
     cand.push_back({1, 0});
     if (can_block(h)) {
+      sslbm::TilePlan plan{0, 0};
+      if (sslbm::tile_plan(h->g.lattice, h->g.precision, h->gv, 1000, &plan)) cand.push_back({plan.depth, -plan.nr});
       for (int d = 2; d <= SSLBM_MAX_DEPTH; ++d) {
         const int base = default_seg(h, d);
         int segs[3] = {base, base / 2, base * 2};
@@ -907,10 +938,14 @@ int sslbm_autotune(sslbm_handle* h, double budget_ms, int* depth_out, int* seg_o
     }
     const double per_cand = budget_ms / (double)cand.size();
     best.ms_per_step = 1e300;
+    double tile_ms = 1e300;
+    auto pass = [&](const std::pair<int, int>& c) {
+      return c.second < 0 ? launch_tile_pass(h, -c.second, c.first) : launch_pass(h, c.first, c.second);
+    };
     for (auto& c : cand) {
       // one untimed launch (also sizes the repetition count), then the timed repetitions
       e = cudaEventRecord(e0, h->stream);
-      if (e == cudaSuccess) e = launch_pass(h, c.first, c.second);
+      if (e == cudaSuccess) e = pass(c);
       if (e == cudaSuccess) e = cudaEventRecord(e1, h->stream);
       if (e == cudaSuccess) e = cudaEventSynchronize(e1);
       float ms1 = 0.f;
@@ -919,7 +954,7 @@ int sslbm_autotune(sslbm_handle* h, double budget_ms, int* depth_out, int* seg_o
       if (reps < 2) reps = 2;
       if (reps > 50) reps = 50;
       if (e == cudaSuccess) e = cudaEventRecord(e0, h->stream);
-      for (int r = 0; r < reps && e == cudaSuccess; ++r) e = launch_pass(h, c.first, c.second);
+      for (int r = 0; r < reps && e == cudaSuccess; ++r) e = pass(c);
       if (e == cudaSuccess) e = cudaEventRecord(e1, h->stream);
       if (e == cudaSuccess) e = cudaEventSynchronize(e1);
       float ms = 0.f;
@@ -930,15 +965,23 @@ int sslbm_autotune(sslbm_handle* h, double budget_ms, int* depth_out, int* seg_o
         return cuda_fail(e, "autotune timing");
       }
       const double per_step = (double)ms / (double)(reps * c.first);
-      if (per_step < best.ms_per_step) best = TuneResult{c.first, c.second, per_step};
+      if (c.second < 0)
+        tile_ms = per_step;
+      else if (per_step < best.ms_per_step)
+        best = TuneResult{c.first, c.second, per_step, false};
     }
     cudaEventDestroy(e0);
     cudaEventDestroy(e1);
+    if (tile_ms < best.ms_per_step) {  // depth and segment stay the pipeline's best, for steps that take no tiles
+      best.ms_per_step = tile_ms;
+      best.tiles = true;
+    }
     std::lock_guard<std::mutex> lock(g_tune_mu);
     g_tune_cache[key] = best;
   }
   h->depth = best.depth;
   h->seg_rows = best.depth > 1 ? best.seg_rows : 0;
+  h->auto_blocking = best.tiles;
   if (depth_out) *depth_out = best.depth;
   if (seg_out) *seg_out = h->seg_rows;
   if (ms_per_step_out) *ms_per_step_out = best.ms_per_step;
