@@ -465,7 +465,7 @@ void sslbm_fd4_destroy(sslbm_fd4* f);
 /* The whole state, [5][ny][nx] FP64 or FP32, host or device; host transfers synchronise. */
 int sslbm_fd4_write(sslbm_fd4* f, const void* src, int src_dtype, int src_on_device);
 int sslbm_fd4_read(sslbm_fd4* f, void* dst, int dst_dtype, int dst_on_device);
-/* n RK4 steps of dt (four stage launches each), stream-ordered. */
+/* n RK4 steps of dt (four stage launches each, in FP32 two launches of two stages), stream-ordered. */
 int sslbm_fd4_step(sslbm_fd4* f, int64_t n);
 int64_t sslbm_fd4_steps_done(const sslbm_fd4* f);
 /* Order of the Laplacian: 4 (default, the reference) or 2, the second-order centred

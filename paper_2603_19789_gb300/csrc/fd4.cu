@@ -6,7 +6,7 @@
 // with the reactions of Eq. (sources) evaluated at every stage.  Ghost cells: periodic wrap,
 // or (no-flux) the even reflection about the boundary face, u[-1] = u[0], u[-2] = u[1].
 //
-// One step is four stage launches.  Stage s reads the previous stage's state with the
+// One step is four stage launches in FP64, two launches of two stages each in FP32.  Stage s reads the previous stage's state with the
 // stencil and writes the next stage's state and the running sum of the slopes:
 //   s = 1: acc = k1,         t = u + (dt/2) k1
 //   s = 2: acc = acc + 2 k2, t = u + (dt/2) k2
@@ -14,11 +14,12 @@
 //   s = 4: u = u + (dt/6) (acc + k4)
 // Every operation is rounded on its own (no contraction) in the order of the formulas
 // above, so the FP64 path reproduces a plain evaluation of them operation by operation.
-// Each stage has two kernels: one cell per thread on 32 x 8 tiles (any width, any
-// precision), and for FP32 grids of width a multiple of 4 with at least 1.5 waves of tiles,
-// four cells per thread on 128 x 8 tiles; both evaluate the same expressions.
+// FP64: one cell per thread on 32 x 8 tiles.  FP32: four cells per thread on 128 x 16 tiles, two
+// stages per launch; both evaluate the same expressions.
 #include <cuda_runtime.h>
 
+#include <algorithm>
+#include <atomic>
 #include <cmath>
 #include <cstdarg>
 #include <cstdio>
@@ -158,141 +159,307 @@ __global__ void __launch_bounds__(kTX * kTY) fd4_stage_kernel(int64_t nx, int64_
   }
 }
 
-// The FP32 stage for grids whose width is a multiple of 4: a 128 x 8 tile, each thread
-// four consecutive cells of one row.  Rows are staged with 16-byte loads (row starts and
-// planes are then 16-byte aligned), the two halo columns on each side separately through
-// ghost2, and u, acc, dst move as float4.  Only the slopes of the four cells stay live
-// across planes (64 registers, four CTAs per SM).  Per cell the expressions and their
-// order are those of fd4_stage_kernel, so both give the same bits.
-constexpr int kVX = 128, kVY = 8, kVPad = 4;  // tile columns and rows; shared rows start 4 columns left
-constexpr int kVS = kVX + 2 * kVPad;            // floats per shared row
+// Two RK4 stages in one launch, FP32: stages 1 and 2 (PAIR 0) or 3 and 4 (PAIR 1) on tiles of
+// 128 x TY cells.  A CTA stages its tile of the input with a halo of four cells, evaluates the first
+// stage on the tile and two cells around it (into shared memory), then the second stage on the
+// tile; the first stage's slopes of the tile stay in registers.
+//   PAIR 0: k1 = f(u), t = u + (dt/2) k1 (on chip), k2 = f(t); writes u + (dt/2) k2 and k1 + 2 k2
+//   PAIR 1: k3 = f(src), v = u + dt k3 (on chip), k4 = f(v); writes u + (dt/6) (acc + 2 k3 + k4)
+// The second stage's ghost cells: with periodic wrap the cells beyond an edge evaluate the first
+// stage on wrapped values, which are the wrapped results; under no-flux the results are copied from
+// the cells they mirror (evaluating the reflected neighbourhood would add its terms in the
+// reverse order).  Every cell performs the operations of fd4_stage_kernel in its order.
+//
+// What bounds it: the operations, 90 per cell and stage of which none may contract, at 1.15 stage
+// evaluations per cell (TY = 16), and latency; the separate stages moved 85 planes a step through
+// HBM or L2 (340 bytes per cell), this moves 32.
+// Four separate stages and these, us per step: 200^2 25.7 and 19.0, 1000^2 79.7 and 58.5, 2048^2 314
+// and 176, 8192^2 4476 and 2462 (27.3 GLUPS; issue 59% busy, 200 instructions per cell and stage).
+// The loads of u and acc wait for HBM if issued where they are used (8192^2 3117); they are
+// requested before the right-hand sides.
+// ghost2 in 32-bit arithmetic, the wrap by one fold without a division on all but tiny grids (with
+// 64-bit modulos the tiles at an edge took 18 us)
+__device__ __forceinline__ int ghost2i(int i, int n, int bc) {
+  if (i >= 0 && i < n) return i;
+  if (bc == SSLBM_BC_PERIODIC) {
+    const int j = i < 0 ? i + n : i - n;
+    if (j >= 0 && j < n) return j;
+    const int r = i % n;
+    return r < 0 ? r + n : r;
+  }
+  if (i < 0) i = -1 - i;
+  if (i >= n) i = 2 * n - 1 - i;
+  return i < 0 ? 0 : i >= n ? n - 1 : i;  // grids narrower than the stencil
+}
 
-template <int STAGE, int ORDER>
-__global__ void __launch_bounds__(32 * kVY, 4) fd4_stage_f32v_kernel(int64_t nx, int64_t ny, int bc,
-                                                                  const Fd4Coeffs<float> k,
-                                                                  const float* __restrict__ src, const float* u,
-                                                                  float* acc, float* dst) {
-  constexpr int RY = kVY + 2 * kH;  // staged rows
-  static_assert(4 * 4 * RY <= 32 * kVY, "one thread per halo cell of the staged rows");
-  __shared__ __align__(16) float tile[4][RY][kVS];
-  const int64_t M = nx * ny;
-  const int lane = threadIdx.x & 31, wy = threadIdx.x >> 5;
-  const int64_t bx0 = (int64_t)blockIdx.x * kVX;
-  const int64_t x = bx0 + 4 * lane;
-  for (int64_t by0 = (int64_t)blockIdx.y * kVY; by0 < ny; by0 += (int64_t)gridDim.y * kVY) {
-    __syncthreads();  // the previous tile's readers are done
-    for (int j = wy; j < 4 * RY; j += kVY) {  // staged row j % RY of plane j / RY, one warp per row
-      const int r = j % RY, c = j / RY;
-      const float* row = src + c * M + ghost2(by0 + r - kH, ny, bc) * nx;
-      float4 v;
-      if (x + 3 < nx) {
-        v = *reinterpret_cast<const float4*>(row + x);
-      } else {  // past the last column: ghost images
-        v.x = row[ghost2(x, nx, bc)];
-        v.y = row[ghost2(x + 1, nx, bc)];
-        v.z = row[ghost2(x + 2, nx, bc)];
-        v.w = row[ghost2(x + 3, nx, bc)];
+constexpr int kPX = 128;          // tile columns
+constexpr int kPS = kPX + 8;      // floats per shared row: columns -4 .. 131
+
+// o[0..1] = a v[0..1], each rounded as mul
+__device__ __forceinline__ void mul2(float a, const float* v, float* o) {
+  const float2 r = __fmul2_rn(make_float2(a, a), make_float2(v[0], v[1]));
+  o[0] = r.x, o[1] = r.y;
+}
+
+// Right-hand sides of S, E, I, R (rhs[0..3]) and D (rhs[4]) for NE consecutive cells: rows are
+// pointers to the cells' first column in rows y-2 .. y+2 of field 0, fields fs floats apart.
+template <int ORDER, int NE>
+__device__ __forceinline__ void fd4_rhs(const float* m2, const float* m1, const float* c0, const float* p1,
+                                        const float* p2, const int fs, const Fd4Coeffs<float>& k, float (&rhs)[5][NE]) {
+#pragma unroll
+  for (int e = 0; e < NE; ++e) {  // reactions, Eq. (sources)
+    const float S = c0[e], E = c0[fs + e], I = c0[2 * fs + e], R = c0[3 * fs + e];
+    const float Nc = add(add(add(S, E), I), R);
+    const float F = Nc != 0.f ? dvd(mul(mul(k.beta, S), I), Nc) : 0.f;
+    const float aE = mul(k.alpha, E);
+    rhs[0][e] = -F;
+    rhs[1][e] = sub(F, aE);
+    rhs[2][e] = sub(aE, mul(k.gamma, I));
+    rhs[3][e] = mul(k.rg, I);
+    rhs[4][e] = mul(k.dg, I);
+  }
+#pragma unroll
+  for (int c = 0; c < 4; ++c) {
+    float h[NE + 4], u2[NE], u1[NE], d1[NE], d2[NE];
+    if (NE == 4) {
+      const float2 hl = *reinterpret_cast<const float2*>(c0 + c * fs - 2);
+      const float4 hc = *reinterpret_cast<const float4*>(c0 + c * fs);
+      const float2 hr = *reinterpret_cast<const float2*>(c0 + c * fs + 4);
+      const float hv[8] = {hl.x, hl.y, hc.x, hc.y, hc.z, hc.w, hr.x, hr.y};
+      const float4 a1 = *reinterpret_cast<const float4*>(m1 + c * fs), b1 = *reinterpret_cast<const float4*>(p1 + c * fs);
+      float4 a2 = make_float4(0.f, 0.f, 0.f, 0.f), b2 = a2;
+      if (ORDER == 4) {
+        a2 = *reinterpret_cast<const float4*>(m2 + c * fs);
+        b2 = *reinterpret_cast<const float4*>(p2 + c * fs);
       }
-      *reinterpret_cast<float4*>(&tile[c][r][kVPad + 4 * lane]) = v;
+      const float av[4] = {a1.x, a1.y, a1.z, a1.w}, bv[4] = {b1.x, b1.y, b1.z, b1.w};
+      const float aw[4] = {a2.x, a2.y, a2.z, a2.w}, bw[4] = {b2.x, b2.y, b2.z, b2.w};
+#pragma unroll
+      for (int e = 0; e < NE + 4; ++e) h[e] = hv[e < 8 ? e : 0];
+#pragma unroll
+      for (int e = 0; e < NE; ++e) u1[e] = av[e & 3], d1[e] = bv[e & 3], u2[e] = aw[e & 3], d2[e] = bw[e & 3];
+    } else {
+#pragma unroll
+      for (int e = 0; e < NE + 4; ++e) h[e] = c0[c * fs + e - 2];
+#pragma unroll
+      for (int e = 0; e < NE; ++e)
+        u2[e] = m2[c * fs + e], u1[e] = m1[c * fs + e], d1[e] = p1[c * fs + e], d2[e] = p2[c * fs + e];
     }
-    if (threadIdx.x < 4 * 4 * RY) {  // halo columns -2, -1, kVX, kVX+1 of every staged row
-      const int h = threadIdx.x & 3, rc = threadIdx.x >> 2;
-      const int r = rc % RY, c = rc / RY;
-      const int col = h < 2 ? h - kH : kVX + h - 2;
-      tile[c][r][kVPad + col] = src[c * M + ghost2(by0 + r - kH, ny, bc) * nx + ghost2(bx0 + col, nx, bc)];
-    }
-    __syncthreads();
-    const int64_t y = by0 + wy;
-    if (x >= nx || y >= ny) continue;
-    const int cy = wy + kH;
-    float rhs[5][4];
-    {  // reactions at this thread's four cells, Eq. (sources)
-      const float4 S4 = *reinterpret_cast<const float4*>(&tile[0][cy][kVPad + 4 * lane]);
-      const float4 E4 = *reinterpret_cast<const float4*>(&tile[1][cy][kVPad + 4 * lane]);
-      const float4 I4 = *reinterpret_cast<const float4*>(&tile[2][cy][kVPad + 4 * lane]);
-      const float4 R4 = *reinterpret_cast<const float4*>(&tile[3][cy][kVPad + 4 * lane]);
-      const float Sv[4] = {S4.x, S4.y, S4.z, S4.w}, Ev[4] = {E4.x, E4.y, E4.z, E4.w};
-      const float Iv[4] = {I4.x, I4.y, I4.z, I4.w}, Rv[4] = {R4.x, R4.y, R4.z, R4.w};
+    if constexpr (NE == 4 && ORDER == 4) {
+      // the products two at a time; the sums that take a product stay scalar (packed, the compiler
+      // may fuse the product into them)
+      float m[8], mu[4], md[4], m30[4], l[4];
+      mul2(16.f, h, m), mul2(16.f, h + 2, m + 2), mul2(16.f, h + 4, m + 4), mul2(16.f, h + 6, m + 6);
+      mul2(16.f, u1, mu), mul2(16.f, u1 + 2, mu + 2), mul2(16.f, d1, md), mul2(16.f, d1 + 2, md + 2);
+      mul2(30.f, h + 2, m30), mul2(30.f, h + 4, m30 + 2);
 #pragma unroll
-      for (int e = 0; e < 4; ++e) {
-        const float S = Sv[e], E = Ev[e], I = Iv[e], R = Rv[e];
-        const float Nc = add(add(add(S, E), I), R);
-        const float F = Nc != 0.f ? dvd(mul(mul(k.beta, S), I), Nc) : 0.f;
-        const float aE = mul(k.alpha, E);
-        rhs[0][e] = -F;
-        rhs[1][e] = sub(F, aE);
-        rhs[2][e] = sub(aE, mul(k.gamma, I));
-        rhs[3][e] = mul(k.rg, I);
-        rhs[4][e] = mul(k.dg, I);
-      }
-    }
-    // the Laplacian, one plane at a time: h[2 + e] is cell e of this thread in the centre row,
-    // h[0..1] and h[6..7] the two cells on each side; col[dy + 2][e] the rows above and below
+      for (int e = 0; e < 4; ++e)
+        l[e] = add(sub(add(sub(add(-h[e], m[1 + e]), m30[e]), m[3 + e]), h[4 + e]),
+                   sub(add(sub(add(-u2[e], mu[e]), m30[e]), md[e]), d2[e]));
+      mul2(k.d[c], l, l), mul2(k.d[c], l + 2, l + 2);
+      mul2(k.inv, l, l), mul2(k.inv, l + 2, l + 2);
 #pragma unroll
-    for (int c = 0; c < 4; ++c) {
-      const float* row = &tile[c][cy][0];
-      const float2 hl = *reinterpret_cast<const float2*>(row + 4 * lane + 2);
-      const float4 hc = *reinterpret_cast<const float4*>(row + kVPad + 4 * lane);
-      const float2 hr = *reinterpret_cast<const float2*>(row + 2 * kVPad + 4 * lane);
-      const float h[8] = {hl.x, hl.y, hc.x, hc.y, hc.z, hc.w, hr.x, hr.y};
-      float col[2 * kH + 1][4];
+      for (int e = 0; e < 4; ++e) rhs[c][e] = add(rhs[c][e], l[e]);
+    } else {
 #pragma unroll
-      for (int dy = -kH; dy <= kH; ++dy) {
-        if (dy != 0 && (ORDER == 4 || dy == -1 || dy == 1)) {
-          const float4 t = *reinterpret_cast<const float4*>(&tile[c][cy + dy][kVPad + 4 * lane]);
-          col[dy + kH][0] = t.x, col[dy + kH][1] = t.y, col[dy + kH][2] = t.z, col[dy + kH][3] = t.w;
-        }
-      }
-#pragma unroll
-      for (int e = 0; e < 4; ++e) {
-        const float u0 = h[2 + e];
-        float lx, ly;
-        if (ORDER == 4) {
-          lx = sub(add(sub(add(-h[e], mul(16.f, h[1 + e])), mul(30.f, u0)), mul(16.f, h[3 + e])), h[4 + e]);
-          ly = sub(add(sub(add(-col[0][e], mul(16.f, col[1][e])), mul(30.f, u0)), mul(16.f, col[3][e])),
-                   col[4][e]);
-        } else {
-          lx = add(sub(h[1 + e], mul(2.f, u0)), h[3 + e]);
-          ly = add(sub(col[1][e], mul(2.f, u0)), col[3][e]);
-        }
-        rhs[c][e] = add(rhs[c][e], mul(mul(k.d[c], add(lx, ly)), ORDER == 4 ? k.inv : k.inv2));
-      }
-    }
-#pragma unroll
-    for (int c = 0; c < 5; ++c) {
-      const int64_t i = c * M + y * nx + x;
-      const float4 uu = *reinterpret_cast<const float4*>(u + i);
-      const float uv[4] = {uu.x, uu.y, uu.z, uu.w};
-      float o[4], a[4];
-      if (STAGE == 1) {
-#pragma unroll
-        for (int e = 0; e < 4; ++e) {
-          a[e] = rhs[c][e];
-          o[e] = add(uv[e], mul(k.half_dt, rhs[c][e]));
-        }
+    for (int e = 0; e < NE; ++e) {
+      const float u0 = h[2 + e];
+      float lx, ly;
+      if (ORDER == 4) {
+        lx = sub(add(sub(add(-h[e], mul(16.f, h[1 + e])), mul(30.f, u0)), mul(16.f, h[3 + e])), h[4 + e]);
+        ly = sub(add(sub(add(-u2[e], mul(16.f, u1[e])), mul(30.f, u0)), mul(16.f, d1[e])), d2[e]);
       } else {
-        const float4 aa = *reinterpret_cast<const float4*>(acc + i);
-        const float av[4] = {aa.x, aa.y, aa.z, aa.w};
-#pragma unroll
-        for (int e = 0; e < 4; ++e) {
-          if (STAGE == 4) {
-            o[e] = add(uv[e], mul(k.dt6, add(av[e], rhs[c][e])));
-          } else {
-            a[e] = add(av[e], mul(2.f, rhs[c][e]));
-            o[e] = add(uv[e], mul(STAGE == 2 ? k.half_dt : k.dt, rhs[c][e]));
-          }
-        }
+        lx = add(sub(h[1 + e], mul(2.f, u0)), h[3 + e]);
+        ly = add(sub(u1[e], mul(2.f, u0)), d1[e]);
       }
-      if (STAGE != 4) *reinterpret_cast<float4*>(acc + i) = make_float4(a[0], a[1], a[2], a[3]);
-      *reinterpret_cast<float4*>(dst + i) = make_float4(o[0], o[1], o[2], o[3]);
+      rhs[c][e] = add(rhs[c][e], mul(mul(k.d[c], add(lx, ly)), ORDER == 4 ? k.inv : k.inv2));
+    }
     }
   }
 }
 
+template <int TY>
+constexpr size_t fd4_pair_smem() {
+  return sizeof(float) * 4 * (2 * TY + 12) * kPS;
+}
+
+// u: the step's state; src: the input of the pair (PAIR 0: u); acc: running sum of the slopes
+// (PAIR 0: written); dst: PAIR 0 the next stage's state (S, E, I, R), PAIR 1 the next state, not
+// u or src.  Rows are pitch floats apart, a multiple of 4.
+template <int PAIR, int ORDER, int TY>
+__global__ void __launch_bounds__(256, TY > 8 ? 2 : 3)
+    fd4_pair_kernel(const int nx, const int ny, const int pitch, const int bc, const Fd4Coeffs<float> k,
+                    const float* __restrict__ src, const float* __restrict__ u, float* __restrict__ acc,
+                    float* __restrict__ dst) {
+  constexpr int RA = TY + 8, RB = TY + 4, FA = RA * kPS, FB = RB * kPS, NR = TY / 8;
+  static_assert(TY % 8 == 0, "whole rows per warp");
+  extern __shared__ __align__(16) float fd4_smem[];
+  float* A = fd4_smem;          // [4][RA][kPS]: the input, rows by0 - 4 ..
+  float* B = fd4_smem + 4 * FA;  // [4][RB][kPS]: the first stage's result, rows by0 - 2 ..
+  const int64_t M = (int64_t)pitch * ny;
+  const int tid = threadIdx.x, lane = tid & 31, w = tid >> 5;
+  const int ntx = (nx + kPX - 1) / kPX;
+  const int bx0 = (int)(blockIdx.x % ntx) * kPX, by0 = (int)(blockIdx.x / ntx) * TY;
+  const float cA = PAIR == 0 ? k.half_dt : k.dt;
+  static_assert(4 * RB <= 128, "a thread per cell of the side columns");
+
+  // the next launch may be scheduled while this one runs; it waits here for all of this one
+  asm volatile("griddepcontrol.launch_dependents;\n" ::: "memory");
+  asm volatile("griddepcontrol.wait;\n" ::: "memory");
+
+  // the input tile: rows of 34 groups of four columns, one warp per row; rows past the domain's
+  // last needed one are skipped (no cell that is written reads them)
+  for (int j = w; j < 4 * RA; j += 8) {
+    const int c = j / RA, r = j - c * RA;
+    if (by0 + r - 4 >= ny + 4) continue;
+    const float* row = src + c * M + (int64_t)ghost2i(by0 + r - 4, ny, bc) * pitch;
+    float* d = A + c * FA + r * kPS;
+    for (int q = lane; q < kPS / 4; q += 32) {
+      const int x = bx0 - 4 + 4 * q;
+      if (x >= nx + 4) continue;
+      if (x >= 0 && x + 3 < nx) {
+        asm volatile("cp.async.cg.shared.global [%0], [%1], 16;\n" ::"r"((unsigned)__cvta_generic_to_shared(d + 4 * q)),
+                     "l"(row + x)
+                     : "memory");
+      } else {
+#pragma unroll
+        for (int e = 0; e < 4; ++e)
+          asm volatile("cp.async.ca.shared.global [%0], [%1], 4;\n" ::"r"(
+                           (unsigned)__cvta_generic_to_shared(d + 4 * q + e)),
+                       "l"(row + ghost2i(x + e, nx, bc))
+                       : "memory");
+      }
+    }
+  }
+  asm volatile("cp.async.wait_all;\n" ::: "memory");
+  __syncthreads();
+
+  const int x = bx0 + 4 * lane;
+  // four cells of a row of a global plane (the row's padding included)
+  auto load4 = [&](const float* p, float (&v)[4]) {
+    const float4 t = x < nx ? *reinterpret_cast<const float4*>(p) : make_float4(0.f, 0.f, 0.f, 0.f);
+    v[0] = t.x, v[1] = t.y, v[2] = t.z, v[3] = t.w;
+  };
+  auto store4 = [&](float* p, const float (&v)[4]) {
+    if (x < nx) *reinterpret_cast<float4*>(p) = make_float4(v[0], v[1], v[2], v[3]);
+  };
+  // first stage of tile row r (-2 .. TY + 1), the lane's four columns; u is requested before the
+  // right-hand sides are evaluated
+  auto stage1 = [&](int r, float (&rhs)[5][4]) {
+    const float* c0 = A + (r + 4) * kPS + 4 + 4 * lane;
+    float uv[4][4];
+    const float* ur = u + (int64_t)ghost2i(by0 + r, ny, bc) * pitch;
+#pragma unroll
+    for (int c = 0; c < 4; ++c) {
+      if (PAIR == 0) {
+        const float4 t = *reinterpret_cast<const float4*>(c0 + c * FA);
+        uv[c][0] = t.x, uv[c][1] = t.y, uv[c][2] = t.z, uv[c][3] = t.w;
+      } else if (x + 3 < nx) {
+        load4(ur + c * M + x, uv[c]);
+      } else {
+#pragma unroll
+        for (int e = 0; e < 4; ++e) uv[c][e] = x + e < nx + 2 ? ur[c * M + ghost2i(x + e, nx, bc)] : 0.f;
+      }
+    }
+    fd4_rhs<ORDER, 4>(c0 - 2 * kPS, c0 - kPS, c0, c0 + kPS, c0 + 2 * kPS, FA, k, rhs);
+    float* o = B + (r + 2) * kPS + 4 + 4 * lane;
+#pragma unroll
+    for (int c = 0; c < 4; ++c) {
+      float v[4];
+#pragma unroll
+      for (int e = 0; e < 4; ++e) v[e] = add(uv[c][e], mul(cA, rhs[c][e]));
+      *reinterpret_cast<float4*>(o + c * FB) = make_float4(v[0], v[1], v[2], v[3]);
+    }
+  };
+  float ka[NR][5][4];  // the first stage's slopes of the warp's tile rows
+#pragma unroll
+  for (int i = 0; i < NR; ++i) stage1(w + 8 * i, ka[i]);
+  if (w < 4) {  // the two rows above and below
+    float t[5][4];
+    stage1(w < 2 ? w - 2 : TY + w - 2, t);
+  }
+  if (tid >= 128 && tid < 128 + 4 * RB) {  // the two columns on each side
+    const int r = (tid - 128) >> 2, h = tid & 3, col = h < 2 ? h - 2 : kPX + h - 2;
+    const float* c0 = A + (r + 2) * kPS + 4 + col;
+    float t[5][1];
+    fd4_rhs<ORDER, 1>(c0 - 2 * kPS, c0 - kPS, c0, c0 + kPS, c0 + 2 * kPS, FA, k, t);
+    const int64_t row = (int64_t)ghost2i(by0 + r - 2, ny, bc) * pitch;
+    const int64_t gx = ghost2i(bx0 + col, nx, bc);
+#pragma unroll
+    for (int c = 0; c < 4; ++c)
+      B[c * FB + r * kPS + 4 + col] = add(PAIR == 0 ? c0[c * FA] : u[c * M + row + gx], mul(cA, t[c][0]));
+  }
+  __syncthreads();
+
+  if (bc != SSLBM_BC_PERIODIC && (bx0 == 0 || by0 == 0 || bx0 + kPX + 2 > nx || by0 + TY + 2 > ny)) {
+    // mirror images of the first stage's results: columns beyond the walls, then rows
+    for (int i = tid; i < 4 * RB * 4; i += 256) {
+      const int h = i & 3, r = (i >> 2) % RB, c = (i >> 2) / RB;
+      const int gx = h < 2 ? h - 2 : nx + h - 2;  // -2, -1, nx, nx + 1
+      if (gx >= bx0 - 2 && gx < bx0 + kPX + 2)
+        B[c * FB + r * kPS + 4 + gx - bx0] = B[c * FB + r * kPS + 4 + ghost2i(gx, nx, bc) - bx0];
+    }
+    __syncthreads();
+    for (int i = tid; i < 4 * 4 * (kPX + 4); i += 256) {
+      const int col = i % (kPX + 4) - 2, h = i / (kPX + 4) & 3, c = i / (kPX + 4) / 4;
+      const int gy = h < 2 ? h - 2 : ny + h - 2;
+      if (gy >= by0 - 2 && gy < by0 + TY + 2)
+        B[c * FB + (gy - by0 + 2) * kPS + 4 + col] = B[c * FB + (ghost2i(gy, ny, bc) - by0 + 2) * kPS + 4 + col];
+    }
+    __syncthreads();
+  }
+
+#pragma unroll
+  for (int i = 0; i < NR; ++i) {
+    const int r = w + 8 * i, y = by0 + r;
+    if (y >= ny) continue;
+    const float* c0 = B + (r + 2) * kPS + 4 + 4 * lane;
+    float rhs[5][4];
+    const int64_t o = (int64_t)y * pitch + x;
+    float ag[5][4], ug[5][4];
+    if (PAIR == 1) {  // requested before the right-hand sides
+#pragma unroll
+      for (int c = 0; c < 5; ++c) {
+        load4(acc + c * M + o, ag[c]);
+        load4(u + c * M + o, ug[c]);
+      }
+    }
+    fd4_rhs<ORDER, 4>(c0 - 2 * kPS, c0 - kPS, c0, c0 + kPS, c0 + 2 * kPS, FB, k, rhs);
+#pragma unroll
+    for (int c = 0; c < 5; ++c) {
+      float out[4];
+      if (PAIR == 0) {
+        float av[4];
+#pragma unroll
+        for (int e = 0; e < 4; ++e) av[e] = add(ka[i][c][e], mul(2.f, rhs[c][e]));
+        store4(acc + c * M + o, av);
+        if (c < 4) {  // D enters no right-hand side
+          const float* uc = A + c * FA + (r + 4) * kPS + 4 + 4 * lane;
+#pragma unroll
+          for (int e = 0; e < 4; ++e) out[e] = add(uc[e], mul(k.half_dt, rhs[c][e]));
+          store4(dst + c * M + o, out);
+        }
+      } else {
+#pragma unroll
+        for (int e = 0; e < 4; ++e)
+          out[e] = add(ug[c][e], mul(k.dt6, add(add(ag[c][e], mul(2.f, ka[i][c][e])), rhs[c][e])));
+        store4(dst + c * M + o, out);
+      }
+    }
+  }
+}
+
+// Rows of nx values, ldb apart, from rows lda apart.
 template <typename A, typename B>
-__global__ void convert_kernel(const A* __restrict__ a, B* __restrict__ b, int64_t n) {
-  for (int64_t t = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; t < n; t += (int64_t)gridDim.x * blockDim.x)
-    b[t] = (B)a[t];
+__global__ void convert_kernel(const A* __restrict__ a, int64_t lda, B* __restrict__ b, int64_t ldb, int64_t nx,
+                               int64_t rows) {
+  for (int64_t y = blockIdx.y; y < rows; y += gridDim.y)
+    for (int64_t x = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; x < nx; x += (int64_t)gridDim.x * blockDim.x)
+      b[y * ldb + x] = (B)a[y * lda + x];
+}
+
+dim3 convert_grid(int64_t nx, int64_t rows) {
+  return dim3((unsigned)((nx + 255) / 256), (unsigned)std::min<int64_t>(65535, rows));
 }
 
 size_t rup(size_t v) { return (v + 255) / 256 * 256; }
@@ -309,11 +476,12 @@ int check_grid(const sslbm_grid* g) {
   return SSLBM_OK;
 }
 
-size_t state_bytes(const sslbm_grid* g) {
-  return rup((size_t)5 * g->nx * g->ny * (g->precision == SSLBM_FP64 ? 8 : 4));
-}
+// Elements from row to row of the state: FP32 rows are padded to whole groups of four cells.
+int64_t row_pitch(const sslbm_grid* g) { return g->precision == SSLBM_FP64 ? g->nx : (g->nx + 3) / 4 * 4; }
 
-unsigned blocks1(int64_t n) { return (unsigned)std::min<int64_t>(65536, (n + 255) / 256); }
+size_t state_bytes(const sslbm_grid* g) {
+  return rup((size_t)5 * row_pitch(g) * g->ny * (g->precision == SSLBM_FP64 ? 8 : 4));
+}
 
 }  // namespace
 
@@ -328,7 +496,9 @@ struct sslbm_fd4 {
   int64_t steps = 0;
   int order = 4;  // order of the Laplacian: 4 (the reference) or 2
   int sms = 1;    // multiprocessors of the device
-  void* buf(int i) const { return ws + (size_t)i * sb; }  // 0 u, 1 t1, 2 t2, 3 acc
+  int cur = 0;    // the state's buffer: 0, or after an odd number of FP32 steps 3
+  void* buf(int i) const { return ws + (size_t)i * sb; }  // FP64: 0 u, 1 t1, 2 t2, 3 acc; FP32: 0 and 3 u, 1 t, 2 acc
+  void* state() const { return buf(cur); }
 };
 
 namespace {
@@ -344,20 +514,52 @@ struct DevGuard {
   }
 };
 
-template <int ORDER>
-cudaError_t run_step_f32v(const sslbm_fd4* f, const Fd4Coeffs<float>& k) {
+template <int PAIR, int ORDER, int TY>
+cudaError_t launch_pair(const sslbm_fd4* f, const float* src, const float* u, float* acc, float* dst) {
+  // the dynamic shared-memory limit, once per device (a bit per device; setting it twice is harmless)
+  static std::atomic<unsigned long long> done{0};
+  auto kern = fd4_pair_kernel<PAIR, ORDER, TY>;
+  if (!(done.load(std::memory_order_acquire) & (1ull << (f->device & 63)))) {
+    cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)fd4_pair_smem<TY>());
+    if (e != cudaSuccess) return e;
+    done.fetch_or(1ull << (f->device & 63), std::memory_order_release);
+  }
   const int64_t nx = f->g.nx, ny = f->g.ny;
-  dim3 grid((unsigned)((nx + kVX - 1) / kVX), (unsigned)std::min<int64_t>(65535, (ny + kVY - 1) / kVY));
-  float* u = static_cast<float*>(f->buf(0));
-  float* t1 = static_cast<float*>(f->buf(1));
-  float* t2 = static_cast<float*>(f->buf(2));
-  float* acc = static_cast<float*>(f->buf(3));
-  const int bc = f->g.bc;
-  fd4_stage_f32v_kernel<1, ORDER><<<grid, 32 * kVY, 0, f->stream>>>(nx, ny, bc, k, u, u, acc, t1);
-  fd4_stage_f32v_kernel<2, ORDER><<<grid, 32 * kVY, 0, f->stream>>>(nx, ny, bc, k, t1, u, acc, t2);
-  fd4_stage_f32v_kernel<3, ORDER><<<grid, 32 * kVY, 0, f->stream>>>(nx, ny, bc, k, t2, u, acc, t1);
-  fd4_stage_f32v_kernel<4, ORDER><<<grid, 32 * kVY, 0, f->stream>>>(nx, ny, bc, k, t1, u, acc, u);
-  return cudaGetLastError();
+  const int64_t ctas = (nx + kPX - 1) / kPX * ((ny + TY - 1) / TY);
+  if (ctas > 0x7fffffffLL) return cudaErrorInvalidConfiguration;
+  cudaLaunchAttribute at[1];
+  at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  at[0].val.programmaticStreamSerializationAllowed = 1;
+  cudaLaunchConfig_t cfg{};
+  cfg.gridDim = dim3((unsigned)ctas);
+  cfg.blockDim = dim3(256);
+  cfg.dynamicSmemBytes = fd4_pair_smem<TY>();
+  cfg.stream = f->stream;
+  cfg.attrs = at;
+  cfg.numAttrs = 1;
+  return cudaLaunchKernelEx(&cfg, kern, (int)nx, (int)ny, (int)row_pitch(&f->g), (int)f->g.bc, f->k32, src, u, acc, dst);
+}
+
+// One FP32 step: two launches, the state alternating between its two buffers.
+template <int ORDER, int TY>
+cudaError_t run_step_pairs(sslbm_fd4* f) {
+  float* u = static_cast<float*>(f->state());
+  float* t = static_cast<float*>(f->buf(1));
+  float* acc = static_cast<float*>(f->buf(2));
+  float* next = static_cast<float*>(f->buf(3 - f->cur));
+  cudaError_t e = launch_pair<0, ORDER, TY>(f, u, u, acc, t);
+  if (e == cudaSuccess) e = launch_pair<1, ORDER, TY>(f, t, u, acc, next);
+  if (e == cudaSuccess) f->cur = 3 - f->cur;
+  return e;
+}
+
+template <int ORDER>
+cudaError_t run_step_f32(sslbm_fd4* f) {
+  // 16-row tiles evaluate 1.15 first stages per cell, 8-row tiles 1.28 but give twice the CTAs and
+  // three per SM: below three 16-row tiles per SM (us per step, 8 and 16 rows: 400^2 26 and 30,
+  // 801 x 700 42 and 49, 1000^2 59 and 59, 2048^2 187 and 176)
+  const int64_t tiles = (f->g.nx + kPX - 1) / kPX * ((f->g.ny + 15) / 16);
+  return tiles >= 3 * (int64_t)f->sms ? run_step_pairs<ORDER, 16>(f) : run_step_pairs<ORDER, 8>(f);
 }
 
 template <typename T, int ORDER>
@@ -375,14 +577,6 @@ cudaError_t run_step(const sslbm_fd4* f, const Fd4Coeffs<T>& k) {
   fd4_stage_kernel<T, 3, ORDER><<<grid, block, 0, f->stream>>>(nx, ny, bc, k, t2, u, acc, t1);
   fd4_stage_kernel<T, 4, ORDER><<<grid, block, 0, f->stream>>>(nx, ny, bc, k, t1, u, acc, u);
   return cudaGetLastError();
-}
-
-// The four-cells-per-thread FP32 stage needs a width that is a multiple of 4, and at
-// least 1.5 waves of its tiles (four resident per SM): on smaller grids the one-cell tiles
-// keep more of the GPU busy.
-bool use_f32v(const sslbm_fd4* f) {
-  const int64_t tiles = ((f->g.nx + kVX - 1) / kVX) * ((f->g.ny + kVY - 1) / kVY);
-  return f->g.nx % 4 == 0 && tiles >= 6 * (int64_t)f->sms;
 }
 
 template <typename T>
@@ -470,25 +664,28 @@ int sslbm_fd4_write(sslbm_fd4* f, const void* src, int src_dtype, int src_on_dev
   if (!f || !src) return err(SSLBM_ERR_BAD_ARG, "NULL argument");
   if (src_dtype != SSLBM_DT_F64 && src_dtype != SSLBM_DT_F32) return err(SSLBM_ERR_BAD_ARG, "dtype %d", src_dtype);
   DevGuard dg(f->device);
-  const int64_t n = 5 * f->g.nx * f->g.ny;
+  const int64_t nx = f->g.nx, rows = 5 * f->g.ny, pitch = row_pitch(&f->g);
   const size_t esz = src_dtype == SSLBM_DT_F64 ? 8 : 4;
-  const void* s = src;
-  if (!src_on_device) {  // stage through the second stage buffer (two buffers when FP32 holds FP64)
-    CK(cudaMemcpyAsync(f->buf(1), src, (size_t)n * esz, cudaMemcpyHostToDevice, f->stream), "host -> device");
-    s = f->buf(1);
-  }
   const bool f64 = f->g.precision == SSLBM_FP64;
-  if (src_dtype == SSLBM_DT_F64 && f64)
-    CK(cudaMemcpyAsync(f->buf(0), s, (size_t)n * 8, cudaMemcpyDeviceToDevice, f->stream), "copy");
-  else if (src_dtype == SSLBM_DT_F32 && !f64)
-    CK(cudaMemcpyAsync(f->buf(0), s, (size_t)n * 4, cudaMemcpyDeviceToDevice, f->stream), "copy");
-  else if (src_dtype == SSLBM_DT_F64)
-    convert_kernel<double, float><<<blocks1(n), 256, 0, f->stream>>>(static_cast<const double*>(s),
-                                                                     static_cast<float*>(f->buf(0)), n);
-  else
-    convert_kernel<float, double><<<blocks1(n), 256, 0, f->stream>>>(static_cast<const float*>(s),
-                                                                     static_cast<double*>(f->buf(0)), n);
-  CK(cudaGetLastError(), "convert");
+  f->cur = 0;
+  if ((src_dtype == SSLBM_DT_F64) == f64) {
+    CK(cudaMemcpy2DAsync(f->buf(0), pitch * esz, src, nx * esz, nx * esz, rows,
+                         src_on_device ? cudaMemcpyDeviceToDevice : cudaMemcpyHostToDevice, f->stream),
+       "copy");
+  } else {
+    const void* s = src;
+    if (!src_on_device) {  // stage through the scratch buffers (two when FP32 holds FP64)
+      CK(cudaMemcpyAsync(f->buf(1), src, (size_t)(rows * nx) * esz, cudaMemcpyHostToDevice, f->stream), "host -> device");
+      s = f->buf(1);
+    }
+    if (f64)
+      convert_kernel<float, double><<<convert_grid(nx, rows), 256, 0, f->stream>>>(
+          static_cast<const float*>(s), nx, static_cast<double*>(f->buf(0)), pitch, nx, rows);
+    else
+      convert_kernel<double, float><<<convert_grid(nx, rows), 256, 0, f->stream>>>(
+          static_cast<const double*>(s), nx, static_cast<float*>(f->buf(0)), pitch, nx, rows);
+    CK(cudaGetLastError(), "convert");
+  }
   if (!src_on_device) CK(cudaStreamSynchronize(f->stream), "sync");
   f->steps = 0;
   return SSLBM_OK;
@@ -498,20 +695,25 @@ int sslbm_fd4_read(sslbm_fd4* f, void* dst, int dst_dtype, int dst_on_device) {
   if (!f || !dst) return err(SSLBM_ERR_BAD_ARG, "NULL argument");
   if (dst_dtype != SSLBM_DT_F64 && dst_dtype != SSLBM_DT_F32) return err(SSLBM_ERR_BAD_ARG, "dtype %d", dst_dtype);
   DevGuard dg(f->device);
-  const int64_t n = 5 * f->g.nx * f->g.ny;
+  const int64_t nx = f->g.nx, rows = 5 * f->g.ny, pitch = row_pitch(&f->g);
   const size_t esz = dst_dtype == SSLBM_DT_F64 ? 8 : 4;
-  void* d = dst_on_device ? dst : f->buf(1);
   const bool f64 = f->g.precision == SSLBM_FP64;
-  if ((dst_dtype == SSLBM_DT_F64) == f64)
-    CK(cudaMemcpyAsync(d, f->buf(0), (size_t)n * esz, cudaMemcpyDeviceToDevice, f->stream), "copy");
-  else if (f64)
-    convert_kernel<double, float><<<blocks1(n), 256, 0, f->stream>>>(static_cast<const double*>(f->buf(0)),
-                                                                     static_cast<float*>(d), n);
-  else
-    convert_kernel<float, double><<<blocks1(n), 256, 0, f->stream>>>(static_cast<const float*>(f->buf(0)),
-                                                                     static_cast<double*>(d), n);
-  CK(cudaGetLastError(), "convert");
-  if (!dst_on_device) CK(cudaMemcpyAsync(dst, d, (size_t)n * esz, cudaMemcpyDeviceToHost, f->stream), "device -> host");
+  if ((dst_dtype == SSLBM_DT_F64) == f64) {
+    CK(cudaMemcpy2DAsync(dst, nx * esz, f->state(), pitch * esz, nx * esz, rows,
+                         dst_on_device ? cudaMemcpyDeviceToDevice : cudaMemcpyDeviceToHost, f->stream),
+       "copy");
+  } else {
+    void* d = dst_on_device ? dst : f->buf(1);
+    if (f64)
+      convert_kernel<double, float><<<convert_grid(nx, rows), 256, 0, f->stream>>>(
+          static_cast<const double*>(f->state()), pitch, static_cast<float*>(d), nx, nx, rows);
+    else
+      convert_kernel<float, double><<<convert_grid(nx, rows), 256, 0, f->stream>>>(
+          static_cast<const float*>(f->state()), pitch, static_cast<double*>(d), nx, nx, rows);
+    CK(cudaGetLastError(), "convert");
+    if (!dst_on_device)
+      CK(cudaMemcpyAsync(dst, d, (size_t)(rows * nx) * esz, cudaMemcpyDeviceToHost, f->stream), "device -> host");
+  }
   CK(cudaStreamSynchronize(f->stream), "sync");
   return SSLBM_OK;
 }
@@ -524,10 +726,8 @@ int sslbm_fd4_step(sslbm_fd4* f, int64_t n) {
     cudaError_t e;
     if (f->g.precision == SSLBM_FP64)
       e = f->order == 4 ? run_step<double, 4>(f, f->k64) : run_step<double, 2>(f, f->k64);
-    else if (use_f32v(f))
-      e = f->order == 4 ? run_step_f32v<4>(f, f->k32) : run_step_f32v<2>(f, f->k32);
     else
-      e = f->order == 4 ? run_step<float, 4>(f, f->k32) : run_step<float, 2>(f, f->k32);
+      e = f->order == 4 ? run_step_f32<4>(f) : run_step_f32<2>(f);
     if (e != cudaSuccess) return cuda_err(e, "FD4 stage launch");
     ++f->steps;
   }
