@@ -25,6 +25,7 @@
 #include <cstdio>
 #include <new>
 
+#include "pdl.cuh"
 #include "sslbm.h"
 
 namespace sslbm {
@@ -303,9 +304,7 @@ __global__ void __launch_bounds__(256, TY > 8 ? 2 : 3)
   const float cA = PAIR == 0 ? k.half_dt : k.dt;
   static_assert(4 * RB <= 128, "a thread per cell of the side columns");
 
-  // the next launch may be scheduled while this one runs; it waits here for all of this one
-  asm volatile("griddepcontrol.launch_dependents;\n" ::: "memory");
-  asm volatile("griddepcontrol.wait;\n" ::: "memory");
+  sslbm::pdl_enter();
 
   // the input tile: rows of 34 groups of four columns, one warp per row; rows past the domain's
   // last needed one are skipped (no cell that is written reads them)
@@ -527,17 +526,8 @@ cudaError_t launch_pair(const sslbm_fd4* f, const float* src, const float* u, fl
   const int64_t nx = f->g.nx, ny = f->g.ny;
   const int64_t ctas = (nx + kPX - 1) / kPX * ((ny + TY - 1) / TY);
   if (ctas > 0x7fffffffLL) return cudaErrorInvalidConfiguration;
-  cudaLaunchAttribute at[1];
-  at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
-  at[0].val.programmaticStreamSerializationAllowed = 1;
-  cudaLaunchConfig_t cfg{};
-  cfg.gridDim = dim3((unsigned)ctas);
-  cfg.blockDim = dim3(256);
-  cfg.dynamicSmemBytes = fd4_pair_smem<TY>();
-  cfg.stream = f->stream;
-  cfg.attrs = at;
-  cfg.numAttrs = 1;
-  return cudaLaunchKernelEx(&cfg, kern, (int)nx, (int)ny, (int)row_pitch(&f->g), (int)f->g.bc, f->k32, src, u, acc, dst);
+  return sslbm::launch_pdl(kern, dim3((unsigned)ctas), dim3(256), fd4_pair_smem<TY>(), f->stream, (int)nx, (int)ny,
+                           (int)row_pitch(&f->g), (int)f->g.bc, f->k32, src, u, acc, dst);
 }
 
 // One FP32 step: two launches, the state alternating between its two buffers.

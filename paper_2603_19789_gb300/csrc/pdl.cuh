@@ -1,0 +1,33 @@
+// pdl.cuh -- programmatic dependent launch for kernels that follow one another on a stream: the
+// next launch's CTAs are scheduled, and compute their indices, while the last CTAs of the current
+// one still run.  A kernel launched by launch_pdl calls pdl_enter() before its first global access;
+// it returns when every earlier kernel of the stream has completed and its writes are visible, so the
+// order of memory accesses is that of ordinary launches.
+#pragma once
+#include <cuda_runtime.h>
+
+#include <utility>
+
+namespace sslbm {
+
+__device__ __forceinline__ void pdl_enter() {
+  asm volatile("griddepcontrol.launch_dependents;\n" ::: "memory");
+  asm volatile("griddepcontrol.wait;\n" ::: "memory");
+}
+
+template <typename... P, typename... A>
+cudaError_t launch_pdl(void (*kern)(P...), dim3 grid, dim3 block, size_t smem, cudaStream_t s, A&&... args) {
+  cudaLaunchAttribute at[1];
+  at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  at[0].val.programmaticStreamSerializationAllowed = 1;
+  cudaLaunchConfig_t cfg{};
+  cfg.gridDim = grid;
+  cfg.blockDim = block;
+  cfg.dynamicSmemBytes = smem;
+  cfg.stream = s;
+  cfg.attrs = at;
+  cfg.numAttrs = 1;
+  return cudaLaunchKernelEx(&cfg, kern, std::forward<A>(args)...);
+}
+
+}  // namespace sslbm

@@ -1,9 +1,7 @@
 // sslbm_kernels.cu -- SSLBM time-step kernels (Sec. II.C, Eq. sslbm_final_clean with the
 // sources of Eq. sources and the deceased update of Eq. rhoD).
 //
-//   step1_kernel    one FP64 step per launch: each thread updates two consecutive cells of a
-//                   row with 16-byte vector loads (double2) of the centre, upper and lower rows
-//                   and two scalar edge loads; neighbouring rows come from L1/L2.  The FP32
+//   step1_kernel    one FP64 step per launch, a cell per thread; neighbours come from L1/L2.  The FP32
 //                   storages advance one step per launch in the streaming kernel (stream.cu).
 //   pipe_kernel     (pipe_launch.cuh) K steps per launch (temporal blocking, K = 2..8) for
 //                   FP32, FP32 deviation-S and FP32 split-S (a sixth plane); pipe_d2q9*.cu and
@@ -30,6 +28,7 @@
 #include <atomic>
 
 #include "bounds.cuh"
+#include "pdl.cuh"
 #include "sslbm_internal.cuh"
 #include "pipe_launch.cuh"
 
@@ -39,68 +38,76 @@ namespace sslbm {
 
 namespace {
 
-// One FP64 step: each thread updates two consecutive cells of a row.
-__global__ void __launch_bounds__(256, 1) step1_kernel(const GridView g, const Coeffs<double> k,
-                                                    const double* __restrict__ in, double* __restrict__ out) {
-  constexpr int V = 2;
-  const int64_t nvec = (g.nx + V - 1) / V;
-  const int64_t vx = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-  if (vx >= nvec) return;
-  const int64_t x0 = vx * V;
-  const int nvalid = (int)((g.nx - x0) < V ? (g.nx - x0) : V);
-  const int64_t xl = link_index(x0 - 1, g.nx, g.bc);
-  const int64_t xr = link_index(x0 + nvalid, g.nx, g.bc);
-  for (int64_t y = (int64_t)blockIdx.y * blockDim.y + threadIdx.y; y < g.ny;
-       y += (int64_t)gridDim.y * blockDim.y) {
-    const int64_t yu = link_index(y - 1, g.ny, g.bc), yd = link_index(y + 1, g.ny, g.bc);
-    if (!(SSLBM_IN(yu, 1, g.ny, 10) && SSLBM_IN(yd, 1, g.ny, 11) && SSLBM_IN(x0, V, g.pitch, 12) &&
-          SSLBM_IN(xl, 1, g.nx, 13) && SSLBM_IN(xr, 1, g.nx, 14)))
-      continue;
-    const int64_t rc = y * g.pitch;
-    const int64_t ru = yu * g.pitch;
-    const int64_t rd = yd * g.pitch;
-    double c[4][V], lap[4][V];
-#pragma unroll
-    for (int f = 0; f < 4; ++f) {
-      const double* P = in + f * g.plane;
-      const double2 cv = *reinterpret_cast<const double2*>(P + rc + x0);
-      const double2 uv = *reinterpret_cast<const double2*>(P + ru + x0);
-      const double2 dv = *reinterpret_cast<const double2*>(P + rd + x0);
-      c[f][0] = cv.x, c[f][1] = cv.y;
-      const double u[V] = {uv.x, uv.y}, d[V] = {dv.x, dv.y};
-      const double L = P[rc + xl];
-      const double R = P[rc + xr];
-      // the right neighbour of the first cell is the second cell unless the row ends there
-      lap[f][0] = lap5(c[f][0], L, nvalid > 1 ? c[f][1] : R, u[0], d[0]);
-      lap[f][1] = lap5(c[f][1], c[f][0], R, u[1], d[1]);
-    }
-    const double2 Dv = *reinterpret_cast<const double2*>(in + 4 * g.plane + rc + x0);
-    const double D[V] = {Dv.x, Dv.y};
-    double n[5][V];
-#pragma unroll
-    for (int j = 0; j < V; ++j)
-      seird_cell(k, c[0][j], c[1][j], c[2][j], c[3][j], D[j], lap[0][j], lap[1][j], lap[2][j], lap[3][j], n[0][j],
-                 n[1][j], n[2][j], n[3][j], n[4][j]);
-    if (nvalid == V) {
-#pragma unroll
-      for (int f = 0; f < 5; ++f)
-        *reinterpret_cast<double2*>(out + f * g.plane + rc + x0) = make_double2(n[f][0], n[f][1]);
-    } else {
-#pragma unroll
-      for (int f = 0; f < 5; ++f) out[f * g.plane + rc + x0] = n[f][0];
-    }
+constexpr int kStep1Threads = 1024;
+
+// One FP64 step, a cell per thread: the cells are numbered along the rows (x fastest), CTA b takes
+// the `per` cells from b * per on.  Bound by the FP64 pipe (two lanes per SM): 38 operations per cell,
+// 15.2 GLUPS at 2 GHz; wider accesses would not help, the pipe takes 16 times longer over a cell
+// than its 21 loads do.  8192^2 13.95 GLUPS; two cells per thread with the earlier force_quot 11.8.
+__global__ void __launch_bounds__(kStep1Threads) step1_kernel(const GridView g, const Coeffs<double> k,
+                                                              const double* __restrict__ in,
+                                                              double* __restrict__ out, const int per) {
+  pdl_enter();
+  if ((int)threadIdx.x >= per) return;
+  int64_t x, y;
+  const int64_t i = (int64_t)blockIdx.x * per + threadIdx.x;
+  if (g.nx <= 0x7fffffff && i <= 0x7fffffff) {
+    const unsigned yy = (unsigned)i / (unsigned)g.nx;
+    y = yy;
+    x = (unsigned)i - yy * (unsigned)g.nx;
+  } else {
+    y = i / g.nx;
+    x = i - y * g.nx;
   }
+  if (y >= g.ny) return;
+  const int64_t yu = link_index(y - 1, g.ny, g.bc), yd = link_index(y + 1, g.ny, g.bc);
+  const int64_t xl = link_index(x - 1, g.nx, g.bc), xr = link_index(x + 1, g.nx, g.bc);
+  if (!(SSLBM_IN(yu, 1, g.ny, 10) && SSLBM_IN(yd, 1, g.ny, 11) && SSLBM_IN(x, 1, g.nx, 12) &&
+        SSLBM_IN(xl, 1, g.nx, 13) && SSLBM_IN(xr, 1, g.nx, 14)))
+    return;
+  const int64_t rc = y * g.pitch, o = rc + x;
+  double c[5], l[4], r[4], u[4], d[4];
+#pragma unroll
+  for (int f = 0; f < 4; ++f) {
+    const double* P = in + f * g.plane;
+    c[f] = P[o], l[f] = P[rc + xl], r[f] = P[rc + xr];
+    u[f] = P[yu * g.pitch + x], d[f] = P[yd * g.pitch + x];
+  }
+  c[4] = in[4 * g.plane + o];
+  double lap[4], n[5];
+#pragma unroll
+  for (int f = 0; f < 4; ++f) lap[f] = lap5(c[f], l[f], r[f], u[f], d[f]);
+  seird_cell(k, c[0], c[1], c[2], c[3], c[4], lap[0], lap[1], lap[2], lap[3], n[0], n[1], n[2], n[3], n[4]);
+#pragma unroll
+  for (int f = 0; f < 5; ++f) out[f * g.plane + o] = n[f];
 }
 
+// Small grids (at most kStep1Threads cells per SM): one CTA per SM with an equal share of the cells,
+// and enough shared memory reserved that an SM holds two, one of this launch and one of the next:
+// with small CTAs the dependent launch's go where there is room and some SMs get twice the work
+// (200^2, us per step: 10.3 with 64 x 8 blocks of two cells, 8.2 with 64-thread CTAs, 10.6 with
+// those and dependent launches, 5.2 with even shares).  Larger grids: 64-thread CTAs.
 cudaError_t launch_step1_fp64(const GridView& g, const void* coeffs, const void* in, void* out, cudaStream_t s) {
-  const int64_t nvec = (g.nx + 1) / 2;
-  dim3 block(32, 8);
-  int64_t gy = (g.ny + 7) / 8;
-  if (gy > 65535) gy = 65535;
-  dim3 grid((unsigned)((nvec + 31) / 32), (unsigned)gy);
-  step1_kernel<<<grid, block, 0, s>>>(g, *static_cast<const Coeffs<double>*>(coeffs),
-                                      static_cast<const double*>(in), static_cast<double*>(out));
-  return cudaGetLastError();
+  constexpr size_t kReserve = 100 * 1024;
+  static std::atomic<int> sms_of[64];  // multiprocessors; set after the kernel's shared-memory limit
+  int dev = 0;
+  cudaError_t e = cudaGetDevice(&dev);
+  if (e != cudaSuccess) return e;
+  int sms = sms_of[dev & 63].load(std::memory_order_acquire);
+  if (!sms) {
+    if ((e = cudaFuncSetAttribute(step1_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kReserve)) != cudaSuccess)
+      return e;
+    if ((e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev)) != cudaSuccess) return e;
+    sms_of[dev & 63].store(sms, std::memory_order_release);
+  }
+  const int64_t cells = g.nx * g.ny;
+  const bool even = cells <= (int64_t)kStep1Threads * sms;
+  const int per = even ? (int)((cells + sms - 1) / sms) : 64;
+  const int64_t ctas = (cells + per - 1) / per;  // up to 2^31 - 1: 1.4e11 cells, 5.5 TB per state
+  if (ctas > 0x7fffffffLL) return cudaErrorInvalidConfiguration;
+  return launch_pdl(step1_kernel, dim3((unsigned)ctas), dim3((per + 31) / 32 * 32), even ? kReserve : 0, s, g,
+                    *static_cast<const Coeffs<double>*>(coeffs), static_cast<const double*>(in),
+                    static_cast<double*>(out), per);
 }
 
 }  // namespace

@@ -25,6 +25,7 @@
 #include <cmath>
 
 #include "bounds.cuh"
+#include "pdl.cuh"
 #include "sslbm_internal.cuh"
 #include "tile.cuh"
 
@@ -135,9 +136,7 @@ __global__ void __launch_bounds__(32 * kTW, 1) tile_kernel(const GridView g, con
   const bool c0 = x >= -K && x < nx + K, c1 = x + 1 >= -K && x + 1 < nx + K;  // cells that can matter
   const int x0 = ghost32(x, nx, bc), x1 = ghost32(x + 1, nx, bc);
 
-  // the next pass may be scheduled while this one runs; it waits below for all of this one
-  asm volatile("griddepcontrol.launch_dependents;\n" ::: "memory");
-  asm volatile("griddepcontrol.wait;\n" ::: "memory");
+  pdl_enter();
 
   auto load = [&](const float* p, int64_t row) {
     float2 v = make_float2(0.f, 0.f);
@@ -263,19 +262,9 @@ cudaError_t launch_t(const GridView& g, const void* coeffs, const void* in, void
   const int64_t ntx = (g.nx + kTCols - 2 * ke - 1) / (kTCols - 2 * ke);
   const int64_t nty = (g.ny + kTW * NR - 2 * K - 1) / (kTW * NR - 2 * K);
   if (ntx * nty > 0x7fffffffLL) return cudaErrorInvalidConfiguration;
-  cudaLaunchAttribute at[1];
-  at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
-  at[0].val.programmaticStreamSerializationAllowed = 1;
-  cudaLaunchConfig_t cfg{};
-  cfg.gridDim = dim3((unsigned)(ntx * nty));
-  cfg.blockDim = dim3(32 * kTW);
-  cfg.dynamicSmemBytes = sizeof(TileSmem);
-  cfg.stream = s;
-  cfg.attrs = at;
-  cfg.numAttrs = 1;
-  return cudaLaunchKernelEx(&cfg, tile_kernel<MODE, NR>, g, *static_cast<const Coeffs<float>*>(coeffs),
-                            static_cast<const float*>(in), static_cast<float*>(out), static_cast<const float*>(kx),
-                            static_cast<const float*>(ky), K, (int)ntx);
+  return launch_pdl(tile_kernel<MODE, NR>, dim3((unsigned)(ntx * nty)), dim3(32 * kTW), sizeof(TileSmem), s, g,
+                    *static_cast<const Coeffs<float>*>(coeffs), static_cast<const float*>(in), static_cast<float*>(out),
+                    static_cast<const float*>(kx), static_cast<const float*>(ky), K, (int)ntx);
 }
 
 template <int MODE>
