@@ -9,6 +9,7 @@
 
 #include "bounds.cuh"
 #include "sslbm_internal.cuh"
+#include "pdl.cuh"
 #include "sslbm_pipe.cuh"
 
 namespace sslbm {
@@ -37,6 +38,7 @@ __global__ void __launch_bounds__(32 * K, MODE == MODE_KAHAN ? 1 : 16 / K) pipe_
   extern __shared__ __align__(16) unsigned char pipe_smem[];
   PipeSmem<K, NF>& sm = *reinterpret_cast<PipeSmem<K, NF>*>(pipe_smem);
   float* rk = reinterpret_cast<float*>(pipe_smem + sizeof(PipeSmem<K, NF>));
+  pdl_enter();
   const int strip = (int)(blockIdx.x % (unsigned)nstrips);
   const int64_t y0 = (int64_t)(blockIdx.x / (unsigned)nstrips) * seg_rows;
   const int64_t y1 = (y0 + seg_rows < g.ny) ? y0 + seg_rows : g.ny;
@@ -83,11 +85,10 @@ cudaError_t launch_blocked_t(const GridView& g, const void* coeffs, const void* 
   const int64_t blocks = nstrips * nseg;
   if (blocks > 0x7fffffffLL) return cudaErrorInvalidConfiguration;
   if (DIAG && (blocks > kDiagBlocks || diag == nullptr)) return cudaErrorInvalidConfiguration;
-  pipe_kernel<MODE, K, DIAG><<<(unsigned)blocks, 32 * K, pipe_smem_bytes<MODE, K, DIAG>(), s>>>(
-      g, *static_cast<const Coeffs<float>*>(coeffs), static_cast<const float*>(in),
-      static_cast<float*>(out), seg_rows, (int)nstrips, static_cast<const float*>(kx),
-      static_cast<const float*>(ky), diag);
-  return cudaGetLastError();
+  return launch_pdl(pipe_kernel<MODE, K, DIAG>, dim3((unsigned)blocks), dim3(32 * K), pipe_smem_bytes<MODE, K, DIAG>(), s,
+                    g, *static_cast<const Coeffs<float>*>(coeffs), static_cast<const float*>(in),
+                    static_cast<float*>(out), seg_rows, (int)nstrips, static_cast<const float*>(kx),
+                    static_cast<const float*>(ky), diag);
 }
 
 template <int MODE, int K>

@@ -27,6 +27,7 @@
 
 #include "bounds.cuh"
 #include "dword.cuh"
+#include "pdl.cuh"
 #include "sslbm_internal.cuh"
 #include "sslbm_pipe.cuh"
 #include "variants.cuh"
@@ -74,6 +75,7 @@ __global__ void __launch_bounds__(32 * Cell::kWarps, Cell::kMinBlocks)
   extern __shared__ __align__(16) float st_smem[];
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   const int item = blockIdx.x * Cell::kWarps + warp;
+  pdl_enter();
   if (item >= nitems) return;
   float* ring = st_smem + (size_t)warp * (RING * ROWF);
   const int strip = item % nstrips;
@@ -500,9 +502,8 @@ cudaError_t launch_stream(const GridView& g, const Cell& cell, cudaStream_t s) {
   const int64_t items = nstrips * ((g.ny + seg - 1) / seg);
   if (items > 0x7fffffffLL - Cell::kWarps) return cudaErrorInvalidConfiguration;
   if (items == 0) return cudaSuccess;
-  stream_kernel<Cell><<<(unsigned)((items + Cell::kWarps - 1) / Cell::kWarps), 32 * Cell::kWarps, smem, s>>>(
-      g, cell, (int)nstrips, (int)items, seg);
-  return cudaGetLastError();
+  return launch_pdl(stream_kernel<Cell>, dim3((unsigned)((items + Cell::kWarps - 1) / Cell::kWarps)),
+                    dim3(32 * Cell::kWarps), smem, s, g, cell, (int)nstrips, (int)items, seg);
 }
 
 }  // namespace
