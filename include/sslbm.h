@@ -395,7 +395,8 @@ int sslbm_ensemble_create(int n, const sslbm_scenario* sc, int precision, void* 
 void sslbm_ensemble_destroy(sslbm_ensemble* e);
 
 /* Tile shape of the persistent launch: steps fused per pass (depth in {2..6, 8}) and the
- * row-segment length of a tile (>= 4 * depth); the tile width is one 128-column strip. */
+ * row-segment length of a tile (>= 4 * depth); the tile width is one 128-column strip.  Without
+ * this call: depth 4 and a segment length by the scenarios' sizes. */
 int sslbm_ensemble_set_tiling(sslbm_ensemble* e, int depth, int seg_rows);
 int sslbm_ensemble_get_tiling(const sslbm_ensemble* e, int* depth, int* seg_rows);
 

@@ -207,6 +207,23 @@ static bool ten_planes(const sslbm_handle* h) {
   return h->g.precision == SSLBM_FP32_KAHAN || h->g.precision == SSLBM_FP64_DW;
 }
 
+// Whether a kernel on the handle's device can use the caller's device buffer as values of this size;
+// memory of another device or of odd alignment is left to the copies.
+static bool kernel_access(const sslbm_handle* h, const void* p, size_t size) {
+  if (reinterpret_cast<uintptr_t>(p) % size) return false;
+  cudaPointerAttributes attr;
+  if (cudaPointerGetAttributes(&attr, p) != cudaSuccess) {
+    cudaGetLastError();
+    return false;
+  }
+  return attr.type != cudaMemoryTypeDevice || attr.device == h->device;
+}
+
+// The compartments with a compensation plane: the first n.
+static int comp_planes(const sslbm_handle* h) {
+  return ten_planes(h) ? 5 : h->g.precision == SSLBM_FP32_SPLIT ? 1 : 0;
+}
+
 // The D2Q5 FP32 storages and the FP32 D2Q9 and varying-diffusion lattices have the
 // temporal-blocked kernel.
 static bool can_block(const sslbm_handle* h) {
@@ -389,6 +406,16 @@ int sslbm_write(sslbm_handle* h, int scheme, int comp, const void* src, int src_
   if (!bgk) h->diag_ready = false;
   char* staging = bgk ? h->b_buf[1 - h->b_cur] : h->s_buf[1 - h->s_cur];
   const int own_dtype = h->g.precision == SSLBM_FP64 ? SSLBM_DT_F64 : SSLBM_DT_F32;
+  const int n_comp = comp_planes(h);
+  const int dev_S = h->g.precision == SSLBM_FP32_DEV ? 1 : 0;
+  if (!bgk && src_on_device && kernel_access(h, src, usize)) {  // every plane in one launch
+    cudaError_t e = sslbm::launch_planes_write(h->g.precision, h->gv, src, src_dtype, h->s_plane(h->s_cur, c0),
+                                               n_comp ? h->s_plane(h->s_cur, 5 + c0) : nullptr, n_comp, c0, c1 - c0,
+                                               dev_S, h->p.s_ref, h->stream);
+    if (e != cudaSuccess) return cuda_fail(e, "write kernel");
+    if (comp == SSLBM_ALL) h->s_steps = 0;
+    return SSLBM_OK;
+  }
   for (int c = c0; c < c1; ++c) {
     const char* s = static_cast<const char*>(src) + (size_t)(c - c0) * plane_user;
     // values stored as given (same type, no deviation or compensation plane): one strided copy
@@ -412,12 +439,9 @@ int sslbm_write(sslbm_handle* h, int scheme, int comp, const void* src, int src_
       e = sslbm::launch_bgk_init(h->g.precision, h->gv, c, s, src_dtype, h->b_buf[h->b_cur],
                                  h->stream);
     } else {
-      const bool kahan = ten_planes(h);
-      const bool split = h->g.precision == SSLBM_FP32_SPLIT && c == SSLBM_S;
-      const int dev_S = (h->g.precision == SSLBM_FP32_DEV && c == SSLBM_S) ? 1 : 0;
-      e = sslbm::launch_plane_write(h->g.precision, h->gv, s, src_dtype, h->s_plane(h->s_cur, c),
-                                    (kahan || split) ? h->s_plane(h->s_cur, 5 + c) : nullptr, dev_S,
-                                    h->p.s_ref, h->stream);
+      e = sslbm::launch_planes_write(h->g.precision, h->gv, s, src_dtype, h->s_plane(h->s_cur, c),
+                                     c < n_comp ? h->s_plane(h->s_cur, 5 + c) : nullptr, n_comp, c, 1, dev_S,
+                                     h->p.s_ref, h->stream);
     }
     if (e != cudaSuccess) return cuda_fail(e, "write kernel");
   }
@@ -455,8 +479,9 @@ int sslbm_set_diffusivity_scale(sslbm_handle* h, const void* kx, const void* ky,
       if (e != cudaSuccess) return cuda_fail(e, "cudaMemcpyAsync(H2D)");
       s = staging;
     }
-    cudaError_t e = sslbm::launch_plane_write(h->g.precision, h->gv, s, src_dtype,
-                                              h->kappa + (size_t)f * h->L.plane_bytes, nullptr, 0, 0.0, h->stream);
+    cudaError_t e = sslbm::launch_planes_write(h->g.precision, h->gv, s, src_dtype,
+                                               h->kappa + (size_t)f * h->L.plane_bytes, nullptr, 0, 0, 1, 0, 0.0,
+                                               h->stream);
     if (e != cudaSuccess) return cuda_fail(e, "scale field write kernel");
   }
   cudaError_t e = sslbm::launch_vard_check(h->g.precision, h->gv, h->kappa, h->kappa + h->L.plane_bytes,
@@ -496,6 +521,14 @@ int sslbm_read(sslbm_handle* h, int scheme, int comp, void* dst, int dst_dtype, 
   const bool bgk = scheme == SSLBM_SCHEME_BGK;
   char* staging = bgk ? h->b_buf[1 - h->b_cur] : h->s_buf[1 - h->s_cur];
   const int own_dtype = h->g.precision == SSLBM_FP64 ? SSLBM_DT_F64 : SSLBM_DT_F32;
+  const int n_comp = comp_planes(h);
+  const int dev_S = h->g.precision == SSLBM_FP32_DEV ? 1 : 0;
+  if (!bgk && dst_on_device && kernel_access(h, dst, usize)) {  // every plane in one launch
+    cudaError_t e = sslbm::launch_planes_read(h->g.precision, h->gv, h->s_plane(h->s_cur, c0),
+                                              n_comp ? h->s_plane(h->s_cur, 5 + c0) : nullptr, n_comp, c0, c1 - c0,
+                                              dev_S, h->p.s_ref, dst, dst_dtype, h->stream);
+    return e == cudaSuccess ? SSLBM_OK : cuda_fail(e, "read kernel");
+  }
   for (int c = c0; c < c1; ++c) {
     char* d = static_cast<char*>(dst) + (size_t)(c - c0) * plane_user;
     // values stored as they are returned: one strided copy out of the pitched plane
@@ -514,12 +547,9 @@ int sslbm_read(sslbm_handle* h, int scheme, int comp, void* dst, int dst_dtype, 
       e = sslbm::launch_bgk_density(h->g.precision, h->gv, c, h->b_buf[h->b_cur], target,
                                     dst_dtype, h->stream);
     } else {
-      const bool kahan = ten_planes(h);
-      const bool split = h->g.precision == SSLBM_FP32_SPLIT && c == SSLBM_S;
-      const int dev_S = (h->g.precision == SSLBM_FP32_DEV && c == SSLBM_S) ? 1 : 0;
-      e = sslbm::launch_plane_read(h->g.precision, h->gv, h->s_plane(h->s_cur, c),
-                                   (kahan || split) ? h->s_plane(h->s_cur, 5 + c) : nullptr, dev_S,
-                                   h->p.s_ref, target, dst_dtype, h->stream);
+      e = sslbm::launch_planes_read(h->g.precision, h->gv, h->s_plane(h->s_cur, c),
+                                    c < n_comp ? h->s_plane(h->s_cur, 5 + c) : nullptr, n_comp, c, 1, dev_S,
+                                    h->p.s_ref, target, dst_dtype, h->stream);
     }
     if (e != cudaSuccess) return cuda_fail(e, "read kernel");
     if (!dst_on_device) {

@@ -28,6 +28,7 @@
 #include <vector>
 
 #include "bounds.cuh"
+#include "diag.cuh"
 #include "sslbm_internal.cuh"
 #include "sslbm_pipe.cuh"
 #include "handles_access.cuh"
@@ -48,6 +49,8 @@ struct EnsScenario {
   Coeffs<float> k;
   int64_t off;  // element offset of the scenario's planes in each buffer
   int nstrips, seg_rows, tiles, tile_base;
+  int64_t diag_base;  // first diagnostics partial
+  int diag_blocks;
 };
 
 struct EnsControl {
@@ -137,6 +140,29 @@ __global__ void __launch_bounds__(32 * K, 16 / K)
   }
 }
 
+// Diagnostics of the scenarios i0 + blockIdx.y, all in one launch: partials, the blocks of a scenario
+// as launch_diagnostics cuts them (so the totals are those of the grid alone, bit for bit), and their
+// totals (NCOMP = 1: plane 5 compensates S).  A reduction and a total per scenario, as before, took
+// 986 us for 32 scenarios of 256^2 to 1024^2, now 186.
+template <int NCOMP>
+__global__ void __launch_bounds__(256) ens_diag_kernel(const EnsScenario* __restrict__ tab, const int i0,
+                                                       const float* __restrict__ buf, double* __restrict__ partials) {
+  const EnsScenario& sc = tab[i0 + blockIdx.y];
+  if ((int)blockIdx.x >= sc.diag_blocks) return;
+  const GridView g = sc.g;
+  const float* st = buf + sc.off;
+  sslbm::diag_rows_f32x4<0, NCOMP>(g, st, NCOMP ? st + 5 * g.plane : nullptr, (int)blockIdx.x, sc.diag_blocks,
+                                   partials + (sc.diag_base + blockIdx.x) * sslbm::kDiagSlots);
+}
+
+__global__ void __launch_bounds__(256) ens_diag_final_kernel(const EnsScenario* __restrict__ tab, const int i0,
+                                                             const double* __restrict__ partials,
+                                                             double* __restrict__ results) {
+  const int i = i0 + (int)blockIdx.x;
+  sslbm::diag_total(partials + tab[i].diag_base * sslbm::kDiagSlots, tab[i].diag_blocks,
+                    results + (size_t)i * sslbm::kDiagSlots);
+}
+
 typedef void (*EnsKernel)(const EnsScenario*, int, int, int, float*, float*, EnsControl*, unsigned*,
                           long long, long long);
 
@@ -204,7 +230,9 @@ int make_layout(int n, const sslbm_scenario* sc, int precision, EnsLayout* L) {
   L->off_tab = off;
   off += round_up((size_t)n * sizeof(EnsScenario), kAlign);
   L->off_partials = off;
-  off += round_up((size_t)sslbm::kDiagBlocks * sslbm::kDiagSlots * sizeof(double), kAlign);
+  int64_t blocks = 0;
+  for (int i = 0; i < n; ++i) blocks += sslbm::diag_blocks(sc[i].ny);
+  off += round_up((size_t)blocks * sslbm::kDiagSlots * sizeof(double), kAlign);
   L->off_results = off;
   off += round_up((size_t)n * sslbm::kDiagSlots * sizeof(double), kAlign);
   for (int b = 0; b < 2; ++b) {
@@ -275,6 +303,7 @@ namespace {
 int upload_table(sslbm_ensemble* e) {
   e->tab.resize(e->n);
   int base = 0;
+  int64_t diag_base = 0;
   for (int i = 0; i < e->n; ++i) {
     const sslbm_scenario& s = e->sc[i];
     EnsScenario& t = e->tab[i];
@@ -298,6 +327,9 @@ int upload_table(sslbm_ensemble* e) {
     t.tiles = t.nstrips * nsegs;
     t.tile_base = base;
     base += t.tiles;
+    t.diag_base = diag_base;
+    t.diag_blocks = (int)sslbm::diag_blocks(s.ny);
+    diag_base += t.diag_blocks;
   }
   e->total_tiles = base;
   cudaError_t ce = cudaMemcpyAsync(e->dtab(), e->tab.data(), sizeof(EnsScenario) * e->n,
@@ -311,6 +343,19 @@ int upload_table(sslbm_ensemble* e) {
     e->exec_blocks = -1;
   }
   return SSLBM_OK;
+}
+
+// Default segment length: the longest (least pipeline fill) that still gives every resident CTA a
+// tile of each step-block.  32 scenarios of 256^2 to 1024^2, 200 steps: 128 rows 4.9 ms (750 tiles
+// for 608 CTAs), 64 rows 5.5, 256 rows 7.1 (400 tiles).
+int default_seg_rows(const sslbm_ensemble* e, int ctas) {
+  const int hl = (e->depth + 3) / 4, wv = 128 - 8 * hl;
+  for (int seg : {256, 128, 64, 32}) {
+    int64_t tiles = 0;
+    for (const sslbm_scenario& s : e->sc) tiles += (s.nx + wv - 1) / wv * ((s.ny + seg - 1) / seg);
+    if (tiles >= ctas) return seg;
+  }
+  return 4 * e->depth;
 }
 
 int resident_ctas(EnsKernel kern, int depth, int precision, int* out) {
@@ -442,6 +487,13 @@ int sslbm_ensemble_create(int n, const sslbm_scenario* sc, int precision, void* 
     delete e;
     return cuda_err(ce, "cudaMemsetAsync(workspace)");
   }
+  int sms = 0;
+  ce = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, e->device);
+  if (ce != cudaSuccess) {
+    delete e;
+    return cuda_err(ce, "cudaDeviceGetAttribute");
+  }
+  e->seg_rows = default_seg_rows(e, 4 * sms);
   st = upload_table(e);
   if (st) {
     delete e;
@@ -495,19 +547,21 @@ int sslbm_ensemble_write(sslbm_ensemble* e, int idx, const void* src, int src_dt
   DevGuard dg(e->device);
   const GridView g = e->gv(idx);
   const size_t bytes = (size_t)g.nx * g.ny * (src_dtype == SSLBM_DT_F64 ? 8 : 4);
+  const int dev_S = e->precision == SSLBM_FP32_DEV ? 1 : 0;
+  const int n_comp = e->precision == SSLBM_FP32_SPLIT ? 1 : 0;
+  void* comp = n_comp ? e->plane(e->cur, idx, 5) : nullptr;
+  if (on_device) {  // the five planes in one launch
+    cudaError_t ce = sslbm::launch_planes_write(SSLBM_FP32, g, src, src_dtype, e->plane(e->cur, idx, 0), comp, n_comp, 0,
+                                                5, dev_S, e->sc[idx].s_ref, e->stream);
+    return ce == cudaSuccess ? SSLBM_OK : cuda_err(ce, "plane write");
+  }
   char* staging = reinterpret_cast<char*>(e->plane(1 - e->cur, idx, 0));
   for (int c = 0; c < 5; ++c) {
-    const char* s = static_cast<const char*>(src) + c * bytes;
-    cudaError_t ce;
-    if (!on_device) {
-      ce = cudaMemcpyAsync(staging, s, bytes, cudaMemcpyHostToDevice, e->stream);
-      if (ce != cudaSuccess) return cuda_err(ce, "cudaMemcpyAsync(H2D)");
-      s = staging;
-    }
-    const int dev_S = (e->precision == SSLBM_FP32_DEV && c == 0) ? 1 : 0;
-    void* comp = (e->precision == SSLBM_FP32_SPLIT && c == 0) ? e->plane(e->cur, idx, 5) : nullptr;
-    ce = sslbm::launch_plane_write(SSLBM_FP32, g, s, src_dtype, e->plane(e->cur, idx, c), comp, dev_S,
-                                   e->sc[idx].s_ref, e->stream);
+    cudaError_t ce = cudaMemcpyAsync(staging, static_cast<const char*>(src) + c * bytes, bytes, cudaMemcpyHostToDevice,
+                                     e->stream);
+    if (ce != cudaSuccess) return cuda_err(ce, "cudaMemcpyAsync(H2D)");
+    ce = sslbm::launch_planes_write(SSLBM_FP32, g, staging, src_dtype, e->plane(e->cur, idx, c),
+                                    c < n_comp ? comp : nullptr, n_comp, c, 1, dev_S, e->sc[idx].s_ref, e->stream);
     if (ce != cudaSuccess) return cuda_err(ce, "plane write");
   }
   if (!on_device) {
@@ -525,19 +579,21 @@ int sslbm_ensemble_read(sslbm_ensemble* e, int idx, void* dst, int dst_dtype, in
   DevGuard dg(e->device);
   const GridView g = e->gv(idx);
   const size_t bytes = (size_t)g.nx * g.ny * (dst_dtype == SSLBM_DT_F64 ? 8 : 4);
+  const int dev_S = e->precision == SSLBM_FP32_DEV ? 1 : 0;
+  const int n_comp = e->precision == SSLBM_FP32_SPLIT ? 1 : 0;
+  const void* comp = n_comp ? e->plane(e->cur, idx, 5) : nullptr;
   char* staging = reinterpret_cast<char*>(e->plane(1 - e->cur, idx, 0));
-  for (int c = 0; c < 5; ++c) {
-    char* d = static_cast<char*>(dst) + c * bytes;
-    const int dev_S = (e->precision == SSLBM_FP32_DEV && c == 0) ? 1 : 0;
-    const void* comp = (e->precision == SSLBM_FP32_SPLIT && c == 0) ? e->plane(e->cur, idx, 5) : nullptr;
-    cudaError_t ce = sslbm::launch_plane_read(SSLBM_FP32, g, e->plane(e->cur, idx, c), comp, dev_S,
-                                              e->sc[idx].s_ref, on_device ? d : staging, dst_dtype,
-                                              e->stream);
+  if (on_device) {  // the five planes in one launch
+    cudaError_t ce = sslbm::launch_planes_read(SSLBM_FP32, g, e->plane(e->cur, idx, 0), comp, n_comp, 0, 5, dev_S,
+                                               e->sc[idx].s_ref, dst, dst_dtype, e->stream);
     if (ce != cudaSuccess) return cuda_err(ce, "plane read");
-    if (!on_device) {
-      ce = cudaMemcpyAsync(d, staging, bytes, cudaMemcpyDeviceToHost, e->stream);
-      if (ce != cudaSuccess) return cuda_err(ce, "cudaMemcpyAsync(D2H)");
-    }
+  }
+  for (int c = 0; c < 5 && !on_device; ++c) {
+    cudaError_t ce = sslbm::launch_planes_read(SSLBM_FP32, g, e->plane(e->cur, idx, c), c < n_comp ? comp : nullptr,
+                                               n_comp, c, 1, dev_S, e->sc[idx].s_ref, staging, dst_dtype, e->stream);
+    if (ce != cudaSuccess) return cuda_err(ce, "plane read");
+    ce = cudaMemcpyAsync(static_cast<char*>(dst) + c * bytes, staging, bytes, cudaMemcpyDeviceToHost, e->stream);
+    if (ce != cudaSuccess) return cuda_err(ce, "cudaMemcpyAsync(D2H)");
   }
   cudaError_t ce = cudaStreamSynchronize(e->stream);
   if (ce != cudaSuccess) return cuda_err(ce, "cudaStreamSynchronize");
@@ -575,11 +631,16 @@ int sslbm_ensemble_diagnostics(sslbm_ensemble* e, double* totals, double* peak_I
   DevGuard dg(e->device);
   double* partials = reinterpret_cast<double*>(e->ws + e->L.off_partials);
   double* results = reinterpret_cast<double*>(e->ws + e->L.off_results);
-  for (int i = 0; i < e->n; ++i) {
-    const bool split = e->precision == SSLBM_FP32_SPLIT;  // S = value - compensation (plane 5)
-    cudaError_t ce = sslbm::launch_diagnostics(SSLBM_FP32, 0, e->gv(i), e->plane(e->cur, i, 0),
-                                               split ? e->plane(e->cur, i, 5) : nullptr, partials,
-                                               results + (size_t)i * sslbm::kDiagSlots, e->stream, 1);
+  int most = 1;
+  for (const EnsScenario& t : e->tab) most = std::max(most, t.diag_blocks);
+  for (int i0 = 0; i0 < e->n; i0 += 65535) {  // a grid's limit in y
+    const int nb = std::min(e->n - i0, 65535);
+    if (e->precision == SSLBM_FP32_SPLIT)
+      ens_diag_kernel<1><<<dim3(most, nb), 256, 0, e->stream>>>(e->dtab(), i0, e->buf(e->cur), partials);
+    else
+      ens_diag_kernel<0><<<dim3(most, nb), 256, 0, e->stream>>>(e->dtab(), i0, e->buf(e->cur), partials);
+    ens_diag_final_kernel<<<nb, 256, 0, e->stream>>>(e->dtab(), i0, partials, results);
+    cudaError_t ce = cudaGetLastError();
     if (ce != cudaSuccess) return cuda_err(ce, "diagnostics");
   }
   std::vector<double> r((size_t)e->n * sslbm::kDiagSlots);

@@ -5,6 +5,8 @@
 #include <stdint.h>
 
 #include "bounds.cuh"
+#include "diag.cuh"
+#include "pdl.cuh"
 #include "sslbm_internal.cuh"
 
 SSLBM_OOB_ACCESSOR(io)
@@ -13,71 +15,134 @@ namespace sslbm {
 
 namespace {
 
-dim3 row_grid(const GridView& g, int threads) {
-  int64_t gy = g.ny < 65535 ? g.ny : 65535;
-  return dim3((unsigned)((g.nx + threads - 1) / threads), (unsigned)gy);
+// The caller's contiguous ny x nx planes (type U) to or from the pitched planes (type T), planes c0
+// .. c0 + gridDim.z - 1 of a state in one launch.  A stored value is v - comp[c] for the first n_comp
+// planes (comps != NULL: on write the rounding residue of the value, so that value - compensation
+// reproduces the input), and s_ref - v for plane 0 under dev_S; both are evaluated in double.  Planes
+// stored as given are copied.
+// Bound by HBM on large grids and by the launch on small ones: a launch per plane (or a strided
+// copy per plane) cost an ensemble of 32 scenarios 957 us to write and 1232 to read, now 186 and 524;
+// the strided device copies of an 8192^2 state took 1.15 ms each way, this 0.45.
+// vec: nx is a multiple of 4 and the caller's planes are 16-byte aligned, so a thread moves four
+// cells at a time; else cells 128 apart, so that a warp's accesses stay contiguous.
+template <typename T>
+struct Vec4 {
+  T v[4];
+};
+template <typename T>
+__device__ __forceinline__ Vec4<T> ld_vec(const T* p) {
+  Vec4<T> r;
+  if constexpr (sizeof(T) == 4) {
+    *reinterpret_cast<float4*>(r.v) = *reinterpret_cast<const float4*>(p);
+  } else {
+    *reinterpret_cast<double2*>(r.v) = *reinterpret_cast<const double2*>(p);
+    *reinterpret_cast<double2*>(r.v + 2) = *reinterpret_cast<const double2*>(p + 2);
+  }
+  return r;
+}
+template <typename T>
+__device__ __forceinline__ void st_vec(T* p, const Vec4<T>& r) {
+  if constexpr (sizeof(T) == 4) {
+    *reinterpret_cast<float4*>(p) = *reinterpret_cast<const float4*>(r.v);
+  } else {
+    *reinterpret_cast<double2*>(p) = *reinterpret_cast<const double2*>(r.v);
+    *reinterpret_cast<double2*>(p + 2) = *reinterpret_cast<const double2*>(r.v + 2);
+  }
 }
 
-// plane <- src (contiguous).  dev_S: store s_ref - value.  comp (Kahan): the rounding residue
-// of the stored value, so that value - compensation reproduces the input.
-template <typename T, typename U>
-__global__ void plane_write_kernel(const GridView g, const U* __restrict__ src,
-                                   T* __restrict__ plane, T* __restrict__ comp, int dev_S,
-                                   double s_ref) {
-  const int64_t x = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-  if (x >= g.nx) return;
+constexpr int kIoThreads = 128;
+
+template <typename T, typename U, bool WRITE>
+__global__ void __launch_bounds__(kIoThreads) planes_io_kernel(const GridView g, U* __restrict__ user,
+                                                               T* __restrict__ planes, T* __restrict__ comps,
+                                                               const int n_comp, const int c0, const int dev_S,
+                                                               const double s_ref, const int vec) {
+  pdl_enter();
+  const int c = c0 + (int)blockIdx.z;
+  U* up = user + (int64_t)blockIdx.z * g.nx * g.ny;
+  T* pp = planes + (int64_t)blockIdx.z * g.plane;
+  T* cp = comps != nullptr && c < n_comp ? comps + (int64_t)blockIdx.z * g.plane : nullptr;
+  const bool dev = dev_S && c == 0;
+  const bool plain = cp == nullptr && !dev;
+  auto put = [&](U a, T& hi, T& lo) {
+    if (plain) {
+      hi = (T)a;
+    } else {
+      double v = (double)a;
+      if (dev) v = s_ref - v;
+      hi = (T)v;
+      lo = (T)((double)hi - v);
+    }
+  };
+  auto get = [&](T hi, T lo) {
+    if (plain) return (U)hi;
+    double v = (double)hi;
+    if (cp) v -= (double)lo;
+    if (dev) v = s_ref - v;
+    return (U)v;
+  };
+  const int64_t xb = (int64_t)blockIdx.x * 4 * kIoThreads;
   for (int64_t y = blockIdx.y; y < g.ny; y += gridDim.y) {
-    double v = (double)src[y * g.nx + x];
-    if (dev_S) v = s_ref - v;
-    const T hi = (T)v;
-    plane[y * g.pitch + x] = hi;
-    if (comp) comp[y * g.pitch + x] = (T)((double)hi - v);
-  }
-}
-
-// dst (contiguous) <- plane, evaluated in double: value - compensation, s_ref - sigma.
-template <typename T, typename U>
-__global__ void plane_read_kernel(const GridView g, const T* __restrict__ plane,
-                                  const T* __restrict__ comp, int dev_S, double s_ref,
-                                  U* __restrict__ dst) {
-  const int64_t x = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-  if (x >= g.nx) return;
-  for (int64_t y = blockIdx.y; y < g.ny; y += gridDim.y) {
-    double v = (double)plane[y * g.pitch + x];
-    if (comp) v -= (double)comp[y * g.pitch + x];
-    if (dev_S) v = s_ref - v;
-    dst[y * g.nx + x] = (U)v;
-  }
-}
-
-// Block-wide reduction of kDiagSlots values (sums of slots 0..4, max of slot 5) in a fixed
-// order, result valid in thread 0.
-__device__ void block_reduce6(double (&v)[kDiagSlots]) {
-  __shared__ double sh[32][kDiagSlots];
-  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    U* ur = up + y * g.nx;
+    T* pr = pp + y * g.pitch;
+    T* cr = cp + (cp ? y * g.pitch : 0);
+    if (vec) {
+      const int64_t x = xb + 4 * threadIdx.x;
+      if (x >= g.nx) continue;
+      if (WRITE) {
+        const Vec4<U> a = ld_vec(ur + x);
+        Vec4<T> hi, lo;
 #pragma unroll
-  for (int off = 16; off > 0; off >>= 1) {
+        for (int e = 0; e < 4; ++e) put(a.v[e], hi.v[e], lo.v[e]);
+        st_vec(pr + x, hi);
+        if (cp) st_vec(cr + x, lo);
+      } else {
+        const Vec4<T> hi = ld_vec(pr + x);
+        Vec4<T> lo = hi;
+        if (cp) lo = ld_vec(cr + x);
+        Vec4<U> a;
 #pragma unroll
-    for (int j = 0; j < 5; ++j) v[j] += __shfl_down_sync(0xffffffffu, v[j], off);
-    v[5] = fmax(v[5], __shfl_down_sync(0xffffffffu, v[5], off));
-  }
-  if (lane == 0) {
+        for (int e = 0; e < 4; ++e) a.v[e] = get(hi.v[e], lo.v[e]);
+        st_vec(ur + x, a);
+      }
+    } else {
 #pragma unroll
-    for (int j = 0; j < kDiagSlots; ++j) sh[warp][j] = v[j];
-  }
-  __syncthreads();
-  if (warp == 0) {
-    const int nw = (blockDim.x + 31) >> 5;
-#pragma unroll
-    for (int j = 0; j < 5; ++j) v[j] = lane < nw ? sh[lane][j] : 0.0;
-    v[5] = lane < nw ? sh[lane][5] : -DBL_MAX;
-#pragma unroll
-    for (int off = 16; off > 0; off >>= 1) {
-#pragma unroll
-      for (int j = 0; j < 5; ++j) v[j] += __shfl_down_sync(0xffffffffu, v[j], off);
-      v[5] = fmax(v[5], __shfl_down_sync(0xffffffffu, v[5], off));
+      for (int e = 0; e < 4; ++e) {
+        const int64_t x = xb + threadIdx.x + e * kIoThreads;
+        if (x >= g.nx) break;
+        if (WRITE) {
+          T hi, lo;
+          put(ur[x], hi, lo);
+          pr[x] = hi;
+          if (cp) cr[x] = lo;
+        } else {
+          const T hi = pr[x];
+          ur[x] = get(hi, cp ? cr[x] : hi);
+        }
+      }
     }
   }
+}
+
+template <typename T, typename U, bool WRITE>
+cudaError_t planes_io_t(const GridView& g, void* user, void* planes, void* comps, int n_comp, int c0, int nplanes,
+                        int dev_S, double s_ref, cudaStream_t s) {
+  const dim3 grid((unsigned)((g.nx + 4 * kIoThreads - 1) / (4 * kIoThreads)), (unsigned)(g.ny < 4096 ? g.ny : 4096),
+                  (unsigned)nplanes);
+  const int vec = g.nx % 4 == 0 && reinterpret_cast<uintptr_t>(user) % 16 == 0;
+  return launch_pdl(planes_io_kernel<T, U, WRITE>, grid, dim3(kIoThreads), 0, s, g, static_cast<U*>(user),
+                    static_cast<T*>(planes), static_cast<T*>(comps), n_comp, c0, dev_S, s_ref, vec);
+}
+
+template <bool WRITE>
+cudaError_t planes_io(int precision, const GridView& g, void* user, int dtype, void* planes, void* comps, int n_comp,
+                      int c0, int nplanes, int dev_S, double s_ref, cudaStream_t s) {
+  const bool t64 = precision == SSLBM_FP64, u64 = dtype == SSLBM_DT_F64;
+  if (t64)
+    return u64 ? planes_io_t<double, double, WRITE>(g, user, planes, comps, n_comp, c0, nplanes, dev_S, s_ref, s)
+               : planes_io_t<double, float, WRITE>(g, user, planes, comps, n_comp, c0, nplanes, dev_S, s_ref, s);
+  return u64 ? planes_io_t<float, double, WRITE>(g, user, planes, comps, n_comp, c0, nplanes, dev_S, s_ref, s)
+             : planes_io_t<float, float, WRITE>(g, user, planes, comps, n_comp, c0, nplanes, dev_S, s_ref, s);
 }
 
 // Per-block partial totals of the five compartments and the maximum of I.
@@ -121,175 +186,31 @@ __global__ void __launch_bounds__(256) diag_partial_kernel(const GridView g,
   }
 }
 
-// Knuth's TwoSum: hi + lo <- hi + x with the rounding error of the addition carried into lo,
-// so that FP32 arithmetic keeps the running sum to about twice FP32's precision.
-__device__ __forceinline__ void two_sum_add(float& hi, float& lo, float x) {
-  const float s = __fadd_rn(hi, x);
-  const float bp = __fsub_rn(s, hi);
-  const float e = __fadd_rn(__fsub_rn(hi, __fsub_rn(s, bp)), __fsub_rn(x, bp));
-  hi = s;
-  lo = __fadd_rn(lo, e);
-}
-
-// The FP32 partials of diag_partial_kernel without per-cell FP64 arithmetic (few FP64 units
-// on this GPU): each thread reads 4 cells per plane at a time (16-byte loads; the pitch and
-// the plane stride are multiples of 4) and keeps its share of the rows as a TwoSum pair per
-// compartment, renormalised (Fast2Sum) after every 4 cells and added to the FP64 partial every
-// kFlushRows rows and at the end.  After a renormalisation the pair's low part is at most half
-// an ulp of its high part, so the pair's own rounding stays near FP32's unit roundoff squared
-// per group of 4 cells.  (Adding the pair to FP64 after every row, the earlier form, took
-// 265 us per 8192^2 call against 255 us now: GB300 has few FP64 units.)
-// NCOMP: the first NCOMP compartments carry a compensation plane (0; 1 for the split S; 5 for
-// Kahan), subtracted from the values.  The peak of I is taken in FP32 (the same value as in
-// FP64), or in FP64 as value minus compensation when I has one.
 template <int LAYOUT, int NCOMP>
 __global__ void __launch_bounds__(256) diag_partial_f32x4_kernel(const GridView g, const float* __restrict__ st,
                                                                  const float* __restrict__ comp,
                                                                  double* __restrict__ partials) {
-  constexpr int kFlushRows = 16;
-  double v[kDiagSlots] = {0.0, 0.0, 0.0, 0.0, 0.0, -DBL_MAX};
-  float hi[5] = {0.f, 0.f, 0.f, 0.f, 0.f}, lo[5] = {0.f, 0.f, 0.f, 0.f, 0.f};
-  float pk = -FLT_MAX;
-  int rows = 0;
-  auto flush = [&]() {
-#pragma unroll
-    for (int c = 0; c < 5; ++c) {
-      v[c] += (double)hi[c] + (double)lo[c];
-      hi[c] = lo[c] = 0.f;
-    }
-  };
-  for (int64_t y = blockIdx.x; y < g.ny; y += gridDim.x) {
-    for (int64_t x = 4 * (int64_t)threadIdx.x; x < g.nx; x += 4 * (int64_t)blockDim.x) {
-      if (!SSLBM_IN(x, 4, g.pitch, 30)) continue;
-      const int64_t idx = y * g.pitch + x;
-      const int nv = g.nx - x < 4 ? (int)(g.nx - x) : 4;
-      float r[5][4];
-      if (LAYOUT == 0) {
-#pragma unroll
-        for (int c = 0; c < 5; ++c) {
-          const float4 a = *reinterpret_cast<const float4*>(st + c * g.plane + idx);
-          r[c][0] = a.x, r[c][1] = a.y, r[c][2] = a.z, r[c][3] = a.w;
-        }
-      } else {
-#pragma unroll
-        for (int c = 0; c < 4; ++c) {
-          float4 a = *reinterpret_cast<const float4*>(st + (c * 5) * g.plane + idx);
-#pragma unroll
-          for (int i = 1; i < 5; ++i) {
-            const float4 b = *reinterpret_cast<const float4*>(st + (c * 5 + i) * g.plane + idx);
-            a.x = __fadd_rn(a.x, b.x), a.y = __fadd_rn(a.y, b.y), a.z = __fadd_rn(a.z, b.z), a.w = __fadd_rn(a.w, b.w);
-          }
-          r[c][0] = a.x, r[c][1] = a.y, r[c][2] = a.z, r[c][3] = a.w;
-        }
-        const float4 d = *reinterpret_cast<const float4*>(st + 20 * g.plane + idx);
-        r[4][0] = d.x, r[4][1] = d.y, r[4][2] = d.z, r[4][3] = d.w;
-      }
-      float q[5][4];
-      if (NCOMP > 0) {
-#pragma unroll
-        for (int c = 0; c < NCOMP; ++c) {
-          const float4 b = *reinterpret_cast<const float4*>(comp + c * g.plane + idx);
-          q[c][0] = b.x, q[c][1] = b.y, q[c][2] = b.z, q[c][3] = b.w;
-        }
-      }
-#pragma unroll
-      for (int j = 0; j < 4; ++j) {
-        if (j >= nv) break;
-#pragma unroll
-        for (int c = 0; c < 5; ++c) {
-          two_sum_add(hi[c], lo[c], r[c][j]);
-          if (c < NCOMP) two_sum_add(hi[c], lo[c], -q[c][j]);
-        }
-        if (NCOMP > 2)
-          v[5] = fmax(v[5], (double)r[2][j] - (double)q[2][j]);
-        else
-          pk = fmaxf(pk, r[2][j]);
-      }
-#pragma unroll
-      for (int c = 0; c < 5; ++c) {  // Fast2Sum: |lo| <= ulp(hi) / 2 again
-        const float t = __fadd_rn(hi[c], lo[c]);
-        lo[c] = __fsub_rn(lo[c], __fsub_rn(t, hi[c]));
-        hi[c] = t;
-      }
-    }
-    if (++rows == kFlushRows) {
-      flush();
-      rows = 0;
-    }
-  }
-  flush();
-  if (NCOMP <= 2) v[5] = fmax(v[5], (double)pk);
-  block_reduce6(v);
-  if (threadIdx.x == 0 && SSLBM_IN(blockIdx.x, 1, kDiagBlocks, 31)) {
-#pragma unroll
-    for (int j = 0; j < kDiagSlots; ++j) partials[blockIdx.x * kDiagSlots + j] = v[j];
-  }
+  diag_rows_f32x4<LAYOUT, NCOMP>(g, st, comp, (int)blockIdx.x, (int)gridDim.x, partials + blockIdx.x * kDiagSlots);
 }
 
 // Sum of the per-block partials in a fixed order (deterministic).
 __global__ void __launch_bounds__(256) diag_final_kernel(const double* __restrict__ partials,
                                                          int nblocks, double* __restrict__ result) {
-  double v[kDiagSlots] = {0.0, 0.0, 0.0, 0.0, 0.0, -DBL_MAX};
-  for (int b = threadIdx.x; b < nblocks; b += blockDim.x) {
-#pragma unroll
-    for (int j = 0; j < 5; ++j) v[j] += partials[b * kDiagSlots + j];
-    v[5] = fmax(v[5], partials[b * kDiagSlots + 5]);
-  }
-  block_reduce6(v);
-  if (threadIdx.x == 0) {
-#pragma unroll
-    for (int j = 0; j < kDiagSlots; ++j) result[j] = v[j];
-  }
+  diag_total(partials, nblocks, result);
 }
 
 }  // namespace
 
-cudaError_t launch_plane_write(int precision, const GridView& g, const void* src, int src_dtype,
-                               void* plane, void* comp_plane, int dev_S, double s_ref,
-                               cudaStream_t s) {
-  const dim3 grid = row_grid(g, 128);
-  if (precision == SSLBM_FP64) {
-    if (src_dtype == SSLBM_DT_F64)
-      plane_write_kernel<double, double><<<grid, 128, 0, s>>>(g, (const double*)src, (double*)plane,
-                                                              (double*)comp_plane, dev_S, s_ref);
-    else
-      plane_write_kernel<double, float><<<grid, 128, 0, s>>>(g, (const float*)src, (double*)plane,
-                                                             (double*)comp_plane, dev_S, s_ref);
-  } else {
-    if (src_dtype == SSLBM_DT_F64)
-      plane_write_kernel<float, double><<<grid, 128, 0, s>>>(g, (const double*)src, (float*)plane,
-                                                             (float*)comp_plane, dev_S, s_ref);
-    else
-      plane_write_kernel<float, float><<<grid, 128, 0, s>>>(g, (const float*)src, (float*)plane,
-                                                            (float*)comp_plane, dev_S, s_ref);
-  }
-  return cudaGetLastError();
+cudaError_t launch_planes_write(int precision, const GridView& g, const void* src, int src_dtype, void* planes,
+                                void* comps, int n_comp, int c0, int nplanes, int dev_S, double s_ref, cudaStream_t s) {
+  return planes_io<true>(precision, g, const_cast<void*>(src), src_dtype, planes, comps, n_comp, c0, nplanes, dev_S,
+                         s_ref, s);
 }
 
-cudaError_t launch_plane_read(int precision, const GridView& g, const void* plane,
-                              const void* comp_plane, int dev_S, double s_ref, void* dst,
-                              int dst_dtype, cudaStream_t s) {
-  const dim3 grid = row_grid(g, 128);
-  if (precision == SSLBM_FP64) {
-    if (dst_dtype == SSLBM_DT_F64)
-      plane_read_kernel<double, double><<<grid, 128, 0, s>>>(g, (const double*)plane,
-                                                             (const double*)comp_plane, dev_S,
-                                                             s_ref, (double*)dst);
-    else
-      plane_read_kernel<double, float><<<grid, 128, 0, s>>>(g, (const double*)plane,
-                                                            (const double*)comp_plane, dev_S,
-                                                            s_ref, (float*)dst);
-  } else {
-    if (dst_dtype == SSLBM_DT_F64)
-      plane_read_kernel<float, double><<<grid, 128, 0, s>>>(g, (const float*)plane,
-                                                            (const float*)comp_plane, dev_S, s_ref,
-                                                            (double*)dst);
-    else
-      plane_read_kernel<float, float><<<grid, 128, 0, s>>>(g, (const float*)plane,
-                                                           (const float*)comp_plane, dev_S, s_ref,
-                                                           (float*)dst);
-  }
-  return cudaGetLastError();
+cudaError_t launch_planes_read(int precision, const GridView& g, const void* planes, const void* comps, int n_comp,
+                               int c0, int nplanes, int dev_S, double s_ref, void* dst, int dst_dtype, cudaStream_t s) {
+  return planes_io<false>(precision, g, dst, dst_dtype, const_cast<void*>(planes), const_cast<void*>(comps), n_comp,
+                          c0, nplanes, dev_S, s_ref, s);
 }
 
 cudaError_t launch_diagnostics(int precision, int layout, const GridView& g, const void* planes,
@@ -297,8 +218,7 @@ cudaError_t launch_diagnostics(int precision, int layout, const GridView& g, con
                                cudaStream_t s, int n_comp) {
   if (!comp_planes) n_comp = 0;
   if (n_comp != 0 && n_comp != 1 && n_comp != 5) return cudaErrorInvalidValue;
-  int64_t blocks = g.ny < kDiagBlocks ? g.ny : kDiagBlocks;
-  if (blocks < 1) blocks = 1;
+  const int64_t blocks = diag_blocks(g.ny);
   if (precision == SSLBM_FP64) {
     if (layout == 0)
       diag_partial_kernel<double, 0><<<(unsigned)blocks, 256, 0, s>>>(

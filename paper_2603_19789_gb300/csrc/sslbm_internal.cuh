@@ -334,15 +334,14 @@ cudaError_t launch_bgk_init(int precision, const GridView& g, int comp, const vo
                             int rho_dtype, void* f, cudaStream_t s);
 cudaError_t launch_bgk_density(int precision, const GridView& g, int comp, const void* f, void* rho,
                                int rho_dtype, cudaStream_t s);
-// plane <-> contiguous user layout (dev_S: deviation storage of S; comp_plane: compensation
-// of the Kahan or split storage, the FP32 rounding residue of the value on write (so that
-// value - compensation reproduces the input) and subtracted on read)
-cudaError_t launch_plane_write(int precision, const GridView& g, const void* src, int src_dtype,
-                               void* plane, void* comp_plane, int dev_S, double s_ref,
-                               cudaStream_t s);
-cudaError_t launch_plane_read(int precision, const GridView& g, const void* plane,
-                              const void* comp_plane, int dev_S, double s_ref, void* dst,
-                              int dst_dtype, cudaStream_t s);
+// planes c0 .. c0 + nplanes - 1 of a state <-> the caller's contiguous ny x nx planes, one launch.
+// planes: plane c0; comps: the compensation of plane c0 (NULL: none), held by planes c < n_comp (Kahan
+// and the double word 5, the split storage 1): the FP32 rounding residue of the value on write, so
+// that value - compensation reproduces the input, subtracted on read.  dev_S: plane 0 is s_ref - S.
+cudaError_t launch_planes_write(int precision, const GridView& g, const void* src, int src_dtype, void* planes,
+                                void* comps, int n_comp, int c0, int nplanes, int dev_S, double s_ref, cudaStream_t s);
+cudaError_t launch_planes_read(int precision, const GridView& g, const void* planes, const void* comps, int n_comp,
+                               int c0, int nplanes, int dev_S, double s_ref, void* dst, int dst_dtype, cudaStream_t s);
 // diagnostics: per-block partial sums of the 5 compartments and max of I into `partials`
 // (kDiagBlocks x kDiagSlots doubles), then their fixed-order total into result[6].
 // layout 0: SSLBM planes; layout 1: BGK populations.
