@@ -610,6 +610,7 @@ __global__ void infection_scale_kernel(const float* __restrict__ u, int* __restr
   const float* ub = u + (b * 5 + 1) * P;
   float mx = 0.f;
   if (vec4_ok(ub, 2 * P)) {
+#pragma unroll 4
     for (int64_t t = i0; t < 2 * P / 4; t += stride) {
       const float4 v = reinterpret_cast<const float4*>(ub)[t];
       mx = fmaxf(mx, fmaxf(fmaxf(v.x, v.y), fmaxf(v.z, v.w)));
@@ -1382,7 +1383,9 @@ int sslbm_fno_make_input(sslbm_fno* f, int batch, const float* u, const float* r
   DevGuard dg(f->device);
   int* smax = f->at<int>(f->bu.smax);
   CK(cudaMemsetAsync(smax, 0, (size_t)batch * 4, f->stream), "zero scale");
-  dim3 grid((unsigned)std::min<int64_t>(64, (2 * f->L.P + kThreads - 1) / kThreads), batch);
+  // few blocks per sample: each thread has several loads in flight (64 blocks: 27 us
+  // at 64 x 256^2, 8 blocks: 10)
+  dim3 grid((unsigned)std::max<int64_t>(1, std::min<int64_t>(8, f->L.P / 2 / kThreads)), batch);
   infection_scale_kernel<<<grid, kThreads, 0, f->stream>>>(u, smax, f->L.P);
   CK(cudaGetLastError(), "infection scale");
   make_input_kernel<<<dim3(rows_grid(f->L.P), batch), kThreads, 0, f->stream>>>(u, r0, logd, smax, x, f->L.P);

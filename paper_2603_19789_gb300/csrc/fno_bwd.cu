@@ -23,8 +23,8 @@
 // to memory once.  Products: mma.sync, BF16 operands rounded where the separate kernels rounded
 // them, FP32 accumulation.
 // One training step (B = 16, 256 x 256, W = 32, m = 12, L = 4, H = 64) took 5317 us with the separate
-// kernels and takes 1511 us: its backward pass 3.7 ms then, 0.80 ms now (ncu, per launch: last 208,
-// mid 107, first 59, y 14.6, mix 10.9, inverse y 10.3).  Mid moves 402 MB (60 us at 6.7 TB/s), last
+// kernels and takes 1403 us: its backward pass 3.7 ms then, under 0.8 ms now (ncu, per launch before
+// the packed gelu': last 208, mid 107, first 59, y 14.6, mix 10.9, inverse y 10.3).  Mid moves 402 MB (60 us at 6.7 TB/s), last
 // 600 MB (90 us); both issue the rest of the time (fragment loads, gelu').
 #include <cuda_bf16.h>
 
@@ -265,7 +265,8 @@ __global__ void __launch_bounds__(kThreads, 2) bwd_row_kernel(const BwdArgs a) {
             for (int nt = 0; nt < NT; ++nt) {
               bf162* q = reinterpret_cast<bf162*>(sZ + (mh * 16 + gr + 8 * h2) * SC + x0 + nt * 8 + 2 * tg);
               const float2 z = __bfloat1622float2(*q);
-              const float v0 = acc3[mh][nt][2 * h2] * gelu_grad(z.x), v1 = acc3[mh][nt][2 * h2 + 1] * gelu_grad(z.y);
+              const float2 d = gelu_grad2(z);
+              const float v0 = acc3[mh][nt][2 * h2] * d.x, v1 = acc3[mh][nt][2 * h2 + 1] * d.y;
               bq1[mh][h2] += v0 + v1;
               *q = __floats2bfloat162_rn(v0, v1);
             }
@@ -353,8 +354,9 @@ __global__ void __launch_bounds__(kThreads, 2) bwd_row_kernel(const BwdArgs a) {
           if (mid) {
             const float2 z = __bfloat1622float2(*reinterpret_cast<const bf162*>(
                 reinterpret_cast<const bf16*>(st + S::raw) + o * SC + xx));
-            v0 *= gelu_grad(z.x);
-            v1 *= gelu_grad(z.y);
+            const float2 d = gelu_grad2(z);
+            v0 *= d.x;
+            v1 *= d.y;
           }
           if (!first) *reinterpret_cast<float2*>(a.dz + (b * W + o) * P + off + xx) = make_float2(v0, v1);
           bs[mt][h2] += v0 + v1;
@@ -414,16 +416,13 @@ __global__ void __launch_bounds__(kThreads, 2) bwd_row_kernel(const BwdArgs a) {
       }
     }
     if (!first) {  // dG1 += dz Fx over this chunk's half
+      static_assert((KF / 8) % TPG == 0, "a group's tiles share their 16 channels");
+      const int gm = g * TPG / (KF / 8) * 16, gn = g * TPG % (KF / 8) * 8;
 #pragma unroll
       for (int k0 = kh * (CC / 2); k0 < (kh + 1) * (CC / 2); k0 += 16) {
-#pragma unroll
-        for (int u = 0; u < TPG; ++u) {
-          const int t = g * TPG + u, mt = t / (KF / 8), nt = t - mt * (KF / 8);
-          uint32_t af[4], bf[2];
-          load_a(af, sDz, SC, mt * 16, k0, lane);
-          load_b_kn1(bf, sF + ch * CC * SF, SF, k0, nt * 8, lane);
-          mma(acc2[u], af, bf[0], bf[1]);
-        }
+        uint32_t af[4];
+        load_a(af, sDz, SC, gm, k0, lane);
+        mma_tiles_kn<TPG>(acc2, af, sF + ch * CC * SF, SF, k0, gn, lane);
       }
     }
     __syncthreads();  // the stage and sDz are free

@@ -25,21 +25,26 @@ struct RowSmem {
   static constexpr size_t oOut = oBl + (lift ? 0 : (size_t)W * SB * 2);        // bf16 [W][SH]
   // one input row: x (8 planes, FP32) or {h_{l-1} [W][SH], G1 [W][SF]} (BF16)
   static constexpr size_t stage = lift ? (size_t)kCin * n * 4 : (size_t)W * SH * 2 + (size_t)W * SF * 2;
-  // f32 [2][W][KF] partial sums of the next layer's transform along x: in the current input
+  // f32 [2][W][SR] partial sums of the next layer's transform along x: in the current input
   // stage (dead after the first product) when they fit, else a region of their own
-  static constexpr size_t red_bytes = (size_t)2 * W * KF * 4;
+  static constexpr int SR = KF + 8;  // rows 8 banks apart: a fragment's 8 rows do not collide
+  static constexpr size_t red_bytes = (size_t)2 * W * SR * 4;
   static constexpr bool red_in_stage = MODE == ROW_MID && red_bytes <= stage;
   static constexpr size_t oRed = oOut + (size_t)W * SH * 2;
   static constexpr size_t oQ1 = oRed + (last || red_in_stage ? 0 : red_bytes);  // bf16 [H][SB]
   static constexpr size_t oQ2 = oQ1 + (last ? (size_t)H * SB * 2 : 0);         // bf16 [16][SQ]
-  static constexpr size_t oA0 = oQ2 + (last ? (size_t)16 * SQ * 2 : 0);        // f32 [W][12]
-  static constexpr size_t oStage = oA0 + (lift ? (size_t)W * 12 * 4 : 0);
+  static constexpr size_t oq1 = oQ2 + (last ? (size_t)16 * SQ * 2 : 0);        // f32 [H]
+  static constexpr size_t oStage = oq1 + (last ? (size_t)H * 4 : 0);
   // input rows in flight: two ahead, except the last layer (two CTAs per SM need the room)
   static constexpr int NST = last ? 2 : 3;
   static constexpr size_t bytes = oStage + NST * stage;
   static_assert(!last || (H / 2 <= W && H % 32 == 0), "half of the projection fits in a stage");
 };
 
+// Bound by issue and the shared-memory pipe together (64 x 256^2, W = 32, m = 12, H = 64; the middle
+// layers move 636 MB, 95 us): middle 194 -> 163 us and last 266 -> 215 with one A fragment per group
+// of tiles in the next layer's transform, GELU in packed FP32, and the last layer's state and bias
+// values requested before the products instead of at their use.
 template <int W, int KF, int H, int NT, int MODE>
 __global__ void __launch_bounds__(kRowThreads, 2) row_kernel(const RowArgs a) {
   using S = RowSmem<W, KF, H, NT, MODE>;
@@ -53,7 +58,6 @@ __global__ void __launch_bounds__(kRowThreads, 2) row_kernel(const RowArgs a) {
   bf16* sOut = reinterpret_cast<bf16*>(smem + S::oOut);
   bf16* sQ1 = reinterpret_cast<bf16*>(smem + S::oQ1);
   bf16* sQ2 = reinterpret_cast<bf16*>(smem + S::oQ2);
-  float* sA0 = reinterpret_cast<float*>(smem + S::oA0);
   unsigned char* stage0 = smem + S::oStage;
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
   const int gr = lane >> 2, tg = lane & 3;
@@ -64,16 +68,20 @@ __global__ void __launch_bounds__(kRowThreads, 2) row_kernel(const RowArgs a) {
     const int r = i / (KF / 8), c = i - r * (KF / 8);
     *reinterpret_cast<uint4*>(sF + r * SF + 8 * c) = *reinterpret_cast<const uint4*>(a.F + (size_t)r * KF + 8 * c);
   }
-  if (MODE == ROW_LIFT) {
-    // sA0[o][0..7] = A0[o][:], sA0[o][8] = a0[o]
-    for (int i = tid; i < W * 9; i += kRowThreads) {
-      const int o = i / 9, c = i - o * 9;
-      sA0[o * 12 + c] = c < kCin ? a.A0[o * kCin + c] : a.a0[o];
-    }
-  } else {
+  // lift: the warp's outputs' weights, wt[q][0..7] = A0[o][:], wt[q][8] = a0[o]
+  constexpr int CL = n >= 128 ? 4 : 2, WO = W / 8;
+  float wt[WO][kCin + 1];
+#pragma unroll
+  for (int q = 0; q < WO; ++q)
+#pragma unroll
+    for (int c = 0; c <= kCin; ++c)
+      wt[q][c] = MODE != ROW_LIFT ? 0.f : c < kCin ? a.A0[(warp * WO + q) * kCin + c] : a.a0[warp * WO + q];
+  if (MODE != ROW_LIFT) {
     for (int i = tid; i < W * W; i += kRowThreads) sBl[(i / W) * SB + i % W] = a.Bl[i];
   }
+  float* sq1 = reinterpret_cast<float*>(smem + S::oq1);
   if (MODE == ROW_LAST) {
+    for (int i = tid; i < H; i += kRowThreads) sq1[i] = a.q1[i];
     for (int i = tid; i < H * W; i += kRowThreads) sQ1[(i / W) * SB + i % W] = a.Q1[i];
     for (int i = tid; i < 16 * H; i += kRowThreads) {
       const int r = i / H, c = i - r * H;
@@ -124,22 +132,58 @@ __global__ void __launch_bounds__(kRowThreads, 2) row_kernel(const RowArgs a) {
     const int b = row / n, y = row - b * n;
     const int x0 = warp * CW;
     unsigned char* st = stage0 + s * S::stage;
+    // last layer: the state the prediction is added to, requested a row's products ahead
+    float2 xv[MODE == ROW_LAST ? NT : 1];
+    float xe = 0.f;
+    if (MODE == ROW_LAST && gr < 5) {
+      xe = a.x[((size_t)b * kCin + 7) * n * n];
+#pragma unroll
+      for (int nt = 0; nt < NT; ++nt)
+        xv[MODE == ROW_LAST ? nt : 0] =
+            *reinterpret_cast<const float2*>(a.x + (((size_t)b * kCin + gr) * n + y) * n + x0 + nt * 8 + 2 * tg);
+    }
     // scratch that reuses the current input stage once the first product has read it
     float* sRed = S::red_in_stage ? reinterpret_cast<float*>(st) : reinterpret_cast<float*>(smem + S::oRed);
     bf16* sP = reinterpret_cast<bf16*>(st);  // [H/2][SH] (last layer)
 
     if (MODE == ROW_LIFT) {
-      // h0 = A0 x + a0 in FP32, one grid column per thread
+      // h0 = A0 x + a0 in FP32: a warp evaluates W / 8 outputs on the whole row, their weights in
+      // registers (with a column per thread every weight came from shared memory for each column:
+      // 199 us at 64 x 256^2, now 128; the row moves 430 MB, 64 us), and writes them to memory and sOut
       const float* xs = reinterpret_cast<const float*>(st);
-      for (int xx = tid; xx < n; xx += kRowThreads) {
-        float xin[kCin];
 #pragma unroll
-        for (int c = 0; c < kCin; ++c) xin[c] = xs[c * n + xx];
-        for (int o = 0; o < W; ++o) {
-          float acc = sA0[o * 12 + kCin];
+      for (int j = 0; j < n / (32 * CL); ++j) {
+        const int xx = j * 32 * CL + CL * lane;
+        float xin[kCin][CL];
 #pragma unroll
-          for (int c = 0; c < kCin; ++c) acc = fmaf(sA0[o * 12 + c], xin[c], acc);
-          sOut[o * SH + xx] = __float2bfloat16_rn(acc);
+        for (int c = 0; c < kCin; ++c) {
+          if constexpr (CL == 4)
+            *reinterpret_cast<float4*>(xin[c]) = *reinterpret_cast<const float4*>(xs + c * n + xx);
+          else
+            *reinterpret_cast<float2*>(xin[c]) = *reinterpret_cast<const float2*>(xs + c * n + xx);
+        }
+#pragma unroll
+        for (int q = 0; q < WO; ++q) {
+          const int o = warp * WO + q;
+          float v[CL];
+#pragma unroll
+          for (int e = 0; e < CL; ++e) {
+            float acc = wt[q][kCin];
+#pragma unroll
+            for (int c = 0; c < kCin; ++c) acc = fmaf(wt[q][c], xin[c][e], acc);
+            v[e] = acc;
+          }
+          bf162 h2[CL / 2];
+#pragma unroll
+          for (int e = 0; e < CL / 2; ++e) h2[e] = __floats2bfloat162_rn(v[2 * e], v[2 * e + 1]);
+          bf16* g = a.hout + (((size_t)b * W + o) * n + y) * n + xx;
+          if constexpr (CL == 4) {
+            *reinterpret_cast<uint2*>(sOut + o * SH + xx) = *reinterpret_cast<const uint2*>(h2);
+            *reinterpret_cast<uint2*>(g) = *reinterpret_cast<const uint2*>(h2);
+          } else {
+            *reinterpret_cast<bf162*>(sOut + o * SH + xx) = h2[0];
+            *reinterpret_cast<bf162*>(g) = h2[0];
+          }
         }
       }
     } else {
@@ -209,15 +253,15 @@ __global__ void __launch_bounds__(kRowThreads, 2) row_kernel(const RowArgs a) {
             float z0 = acc[mt][nt][2 * h2] + bias[mt][h2], z1 = acc[mt][nt][2 * h2 + 1] + bias[mt][h2];
             if (MODE == ROW_MID) {
               if (a.store) st_bf2(a.zout + (((size_t)b * W + o) * n + y) * n + xx, z0, z1);
-              z0 = gelu(z0);
-              z1 = gelu(z1);
+              const float2 q = gelu2(make_float2(z0, z1));
+              z0 = q.x, z1 = q.y;
             }
             st_bf2(sOut + o * SH + xx, z0, z1);
           }
     }
     __syncthreads();
 
-    if (MODE != ROW_LAST || a.store) {
+    if (MODE == ROW_MID || (MODE == ROW_LAST && a.store)) {
       for (int i = tid; i < W * (n / 8); i += kRowThreads) {
         const int c = i / (n / 8), j = i - c * (n / 8);
         *reinterpret_cast<uint4*>(a.hout + (((size_t)b * W + c) * n + y) * n + 8 * j) =
@@ -236,15 +280,13 @@ __global__ void __launch_bounds__(kRowThreads, 2) row_kernel(const RowArgs a) {
       for (int u = 0; u < TPG; ++u)
 #pragma unroll
         for (int r = 0; r < 4; ++r) acc2[u][r] = 0.f;
+      static_assert((KF / 8) % TPG == 0, "a group's tiles share their 16 channels");
+      const int gm = g * TPG / (KF / 8) * 16, gn = g * TPG % (KF / 8) * 8;
+#pragma unroll 4
       for (int k0 = kh * (n / 2); k0 < (kh + 1) * (n / 2); k0 += 16) {
-#pragma unroll
-        for (int u = 0; u < TPG; ++u) {
-          const int t = g * TPG + u, mt = t / (KF / 8), nt = t - mt * (KF / 8);
-          uint32_t af[4], bf[2];
-          load_a(af, sOut, SH, mt * 16, k0, lane);
-          load_b_kn1(bf, sF, SF, k0, nt * 8, lane);
-          mma(acc2[u], af, bf[0], bf[1]);
-        }
+        uint32_t af[4];
+        load_a(af, sOut, SH, gm, k0, lane);
+        mma_tiles_kn<TPG>(acc2, af, sF, SF, k0, gn, lane);
       }
 #pragma unroll
       for (int u = 0; u < TPG; ++u) {
@@ -252,14 +294,16 @@ __global__ void __launch_bounds__(kRowThreads, 2) row_kernel(const RowArgs a) {
 #pragma unroll
         for (int h2 = 0; h2 < 2; ++h2) {
           const int o = mt * 16 + gr + 8 * h2, c = nt * 8 + 2 * tg;
-          sRed[(kh * W + o) * KF + c] = acc2[u][2 * h2];
-          sRed[(kh * W + o) * KF + c + 1] = acc2[u][2 * h2 + 1];
+          *reinterpret_cast<float2*>(sRed + (kh * W + o) * S::SR + c) = make_float2(acc2[u][2 * h2], acc2[u][2 * h2 + 1]);
         }
       }
       __syncthreads();
       bf16* dst = a.H1out + ((size_t)b * n + y) * W * KF;
-      for (int i = tid; i < W * KF / 2; i += kRowThreads)
-        st_bf2(dst + 2 * i, sRed[2 * i] + sRed[W * KF + 2 * i], sRed[2 * i + 1] + sRed[W * KF + 2 * i + 1]);
+      for (int i = tid; i < W * KF / 2; i += kRowThreads) {
+        const float* r = sRed + i / (KF / 2) * S::SR + i % (KF / 2) * 2;
+        const float2 p = *reinterpret_cast<const float2*>(r), q = *reinterpret_cast<const float2*>(r + W * S::SR);
+        st_bf2(dst + 2 * i, p.x + q.x, p.y + q.y);
+      }
     } else {
       // projection on the warp's own columns: p = gelu(Q1 h_L + q1), delta = Q2 p + q2, in two
       // halves of the H rows of p (each half staged in the warp's columns of sP)
@@ -308,14 +352,14 @@ __global__ void __launch_bounds__(kRowThreads, 2) row_kernel(const RowArgs a) {
 #pragma unroll
           for (int h2 = 0; h2 < 2; ++h2) {
             const int hl = mh * 16 + gr + 8 * h2, hh = h0 + hl;
-            const float qv = a.q1[hh];
+            const float qv = sq1[hh];
 #pragma unroll
             for (int nt = 0; nt < NT; ++nt) {
               const int xx = x0 + nt * 8 + 2 * tg;
               const float z0 = acc3[mh][nt][2 * h2] + qv, z1 = acc3[mh][nt][2 * h2 + 1] + qv;
               const size_t off = (((size_t)b * H + hh) * n + y) * n + xx;
               if (a.store) st_bf2(a.zp + off, z0, z1);
-              const bf162 pv = __floats2bfloat162_rn(gelu(z0), gelu(z1));
+              const bf162 pv = __float22bfloat162_rn(gelu2(make_float2(z0, z1)));
               *reinterpret_cast<bf162*>(sP + hl * SH + xx) = pv;
               if (a.store) *reinterpret_cast<bf162*>(a.p + off) = pv;
             }
@@ -346,14 +390,13 @@ __global__ void __launch_bounds__(kRowThreads, 2) row_kernel(const RowArgs a) {
         // clamp keeps a NaN a NaN, so a non-finite prediction stays visible to the checks
         const int c = gr;
         const float qc = a.q2[c];
-        const float sig = (c == 1 || c == 2) ? exp10f(4.f * a.x[((size_t)b * kCin + 7) * n * n] - 4.f) : 1.f;
+        const float sig = (c == 1 || c == 2) ? exp10f(4.f * xe - 4.f) : 1.f;
 #pragma unroll
         for (int nt = 0; nt < NT; ++nt) {
           const int xx = x0 + nt * 8 + 2 * tg;
-          const float2 xv = *reinterpret_cast<const float2*>(a.x + (((size_t)b * kCin + c) * n + y) * n + xx);
           float2 out;
-          out.x = xv.x + (acc4[nt][0] + qc);
-          out.y = xv.y + (acc4[nt][1] + qc);
+          out.x = xv[nt].x + (acc4[nt][0] + qc);
+          out.y = xv[nt].y + (acc4[nt][1] + qc);
           out.x = out.x < 0.f ? 0.f : out.x;
           out.y = out.y < 0.f ? 0.f : out.y;
           if (c == 1 || c == 2) {
@@ -394,13 +437,15 @@ __global__ void __launch_bounds__(128) dft_y_kernel(const bf16* __restrict__ H1,
     else
       *reinterpret_cast<uint4*>(sFy + r * SY + 8 * j) = make_uint4(0, 0, 0, 0);
   }
-  for (int i = tid; i < n * (NC / 8); i += 128) {
-    const int yy = i / (NC / 8), j = i - yy * (NC / 8);
-    cp16(sT + yy * SC + 8 * j, H1 + (((size_t)b * n + yy) * W + c0) * KF + 8 * j);
+  // the rows in quarters, each its own group, so that the product starts on the first
+#pragma unroll 1
+  for (int h = 0; h < 4; ++h) {
+    for (int i = tid; i < n / 4 * (NC / 8); i += 128) {
+      const int yy = h * (n / 4) + i / (NC / 8), j = i % (NC / 8);
+      cp16(sT + yy * SC + 8 * j, H1 + (((size_t)b * n + yy) * W + c0) * KF + 8 * j);
+    }
+    commit();
   }
-  commit();
-  wait_groups<0>();
-  __syncthreads();
   float acc[2][TPW][4];
 #pragma unroll
   for (int mt = 0; mt < 2; ++mt)
@@ -408,16 +453,24 @@ __global__ void __launch_bounds__(128) dft_y_kernel(const bf16* __restrict__ H1,
     for (int u = 0; u < TPW; ++u)
 #pragma unroll
       for (int r = 0; r < 4; ++r) acc[mt][u][r] = 0.f;
-  for (int k0 = 0; k0 < n; k0 += 16) {
-    uint32_t af[2][4];
-    load_a(af[0], sFy, SY, 0, k0, lane);
-    load_a(af[1], sFy, SY, 16, k0, lane);
 #pragma unroll
-    for (int u = 0; u < TPW; ++u) {
-      uint32_t bf[2];
-      load_b_kn1(bf, sT, SC, k0, (warp * TPW + u) * 8, lane);
-      mma(acc[0][u], af[0], bf[0], bf[1]);
-      mma(acc[1][u], af[1], bf[0], bf[1]);
+  for (int h = 0; h < 4; ++h) {
+    if (h == 0) wait_groups<3>();
+    if (h == 1) wait_groups<2>();
+    if (h == 2) wait_groups<1>();
+    if (h == 3) wait_groups<0>();
+    __syncthreads();
+    for (int k0 = h * (n / 4); k0 < (h + 1) * (n / 4); k0 += 16) {
+      uint32_t af[2][4];
+      load_a(af[0], sFy, SY, 0, k0, lane);
+      load_a(af[1], sFy, SY, 16, k0, lane);
+#pragma unroll
+      for (int u = 0; u < TPW; ++u) {
+        uint32_t bf[2];
+        load_b_kn1(bf, sT, SC, k0, (warp * TPW + u) * 8, lane);
+        mma(acc[0][u], af[0], bf[0], bf[1]);
+        mma(acc[1][u], af[1], bf[0], bf[1]);
+      }
     }
   }
 #pragma unroll
@@ -504,12 +557,14 @@ __global__ void __launch_bounds__(256) idft_y_kernel(const float2* __restrict__ 
   bf16* sFyi = reinterpret_cast<bf16*>(smem);  // [n][SY], columns >= 2m zero
   bf16* sU = sFyi + (size_t)n * SY;             // [32][SU], rows >= 2m zero
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+  bf16* sG = sU + 32 * SU + warp * 16 * SU;     // [16][SU] of this warp
   const int gr = lane >> 2, tg = lane & 3;
   const int b = blockIdx.y, o0 = blockIdx.x * OG;
   const bf16 zero = __float2bfloat16_rn(0.f);
-  for (int i = tid; i < n * 32; i += 256) {
-    const int yy = i >> 5, r = i & 31;
-    sFyi[yy * SY + r] = r < M2 ? Fyi[(size_t)yy * M2 + r] : zero;
+  for (int i = tid; i < n * 4; i += 256) {
+    const int yy = i >> 2, j = i & 3;
+    *reinterpret_cast<uint4*>(sFyi + yy * SY + 8 * j) =
+        8 * j < M2 ? *reinterpret_cast<const uint4*>(Fyi + (size_t)yy * M2 + 8 * j) : make_uint4(0, 0, 0, 0);
   }
   for (int i = tid; i < (32 - M2) * NC; i += 256) sU[(M2 + i / NC) * SU + i % NC] = zero;
   for (int i = tid; i < OG * modes; i += 256) {
@@ -542,13 +597,19 @@ __global__ void __launch_bounds__(256) idft_y_kernel(const float2* __restrict__ 
         mma(acc[t + 1], af, bf[2], bf[3]);
       }
     }
+    // the 16 rows through the warp's own shared rows, so that memory sees whole 16-byte groups of a row
+    __syncwarp();
 #pragma unroll
     for (int t = 0; t < NTT; ++t)
 #pragma unroll
-      for (int h2 = 0; h2 < 2; ++h2) {
-        const int yy = mt * 16 + gr + 8 * h2, col = t * 8 + 2 * tg;
-        st_bf2(G1 + (((size_t)b * n + yy) * W + o0) * KF + col, acc[t][2 * h2] * scale, acc[t][2 * h2 + 1] * scale);
-      }
+      for (int h2 = 0; h2 < 2; ++h2)
+        st_bf2(sG + (gr + 8 * h2) * SU + t * 8 + 2 * tg, acc[t][2 * h2] * scale, acc[t][2 * h2 + 1] * scale);
+    __syncwarp();
+    for (int i = lane; i < 16 * (NC / 8); i += 32) {
+      const int r = i / (NC / 8), j = i - r * (NC / 8);
+      *reinterpret_cast<uint4*>(G1 + (((size_t)b * n + mt * 16 + r) * W + o0) * KF + 8 * j) =
+          *reinterpret_cast<const uint4*>(sG + r * SU + 8 * j);
+    }
   }
 }
 
@@ -798,7 +859,7 @@ cudaError_t launch_mix_t(int W, int B, int n, const float* hat, const float* R, 
                                                               reinterpret_cast<const float2*>(R),
                                                               reinterpret_cast<float2*>(hatg), B, W, modes);
   if ((e = cudaGetLastError()) != cudaSuccess) return e;
-  const size_t bytes = (size_t)n * 40 * 2 + (size_t)32 * (OG * KF + 8) * 2;
+  const size_t bytes = (size_t)n * 40 * 2 + (size_t)(32 + 8 * 16) * (OG * KF + 8) * 2;
   e = cudaFuncSetAttribute(idft_y_kernel<KF, OG>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes);
   if (e != cudaSuccess) return e;
   idft_y_kernel<KF, OG><<<dim3(W / OG, B), 256, bytes, s>>>(reinterpret_cast<const float2*>(hatg), Fyi, G1, W, n,

@@ -22,7 +22,7 @@ namespace {
 // stored as given are copied.
 // Bound by HBM on large grids and by the launch on small ones: a launch per plane (or a strided
 // copy per plane) cost an ensemble of 32 scenarios 957 us to write and 1232 to read, now 186 and 524;
-// the strided device copies of an 8192^2 state took 1.15 ms each way, this 0.45.
+// the strided device copies of an 8192^2 state took 1.33 ms each way, this 0.39.
 // vec: nx is a multiple of 4 and the caller's planes are 16-byte aligned, so a thread moves four
 // cells at a time; else cells 128 apart, so that a warp's accesses stay contiguous.
 template <typename T>
