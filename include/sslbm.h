@@ -232,7 +232,8 @@ int sslbm_set_diffusivity_scale(sslbm_handle* h, const void* kx, const void* ky,
 int sslbm_step(sslbm_handle* h, int64_t n);
 
 /* Advance the BGK state by n >= 0 steps of Eq. (pdf) (collide, then stream along
- * the D2Q5 links; no-flux walls by halfway bounce-back) with D by Eq. (rhoD). */
+ * the D2Q5 links; no-flux walls by halfway bounce-back) with D by Eq. (rhoD).  FP32 fuses up
+ * to four steps per pass, with the results of one step per pass. */
 int bgk_step(sslbm_handle* h, int64_t n);
 
 /* Steps taken by a scheme since its last full write. */

@@ -645,12 +645,22 @@ int bgk_step(sslbm_handle* h, int64_t n) {
   if (st) return st;
   if (n < 0) return fail(SSLBM_ERR_BAD_ARG, "n=%lld < 0", (long long)n);
   DeviceGuard dg(h->device);
-  for (int64_t i = 0; i < n; ++i) {
-    cudaError_t e = sslbm::launch_bgk_step(h->g.precision, h->gv, h->coeffs(), h->b_buf[h->b_cur],
-                                           h->b_buf[1 - h->b_cur], h->stream);
+  while (n > 0) {
+    // FP32: passes of up to kBgkDepth steps, their depths differing by at most one; FP64, whose
+    // arithmetic rate bounds it, and a single step: one step per launch
+    int64_t k = 1;
+    if (h->g.precision == SSLBM_FP32 && n > 1) {
+      const int64_t passes = (n + sslbm::kBgkDepth - 1) / sslbm::kBgkDepth;
+      k = (n + passes - 1) / passes;
+    }
+    cudaError_t e = k > 1 ? sslbm::launch_bgk_tile(h->gv, &h->cf, h->b_buf[h->b_cur], h->b_buf[1 - h->b_cur], (int)k,
+                                                   h->stream)
+                          : sslbm::launch_bgk_step(h->g.precision, h->gv, h->coeffs(), h->b_buf[h->b_cur],
+                                                   h->b_buf[1 - h->b_cur], h->stream);
     if (e != cudaSuccess) return cuda_fail(e, "BGK step launch");
     h->b_cur = 1 - h->b_cur;
-    h->b_steps += 1;
+    h->b_steps += k;
+    n -= k;
   }
   return SSLBM_OK;
 }
@@ -721,12 +731,13 @@ int sslbm_debug_bounds(long long* count, long long* value, long long* limit, int
   int (*const take[])(sslbm::OobRecord*) = {sslbm::oob_take_kernels, sslbm::oob_take_ensemble, sslbm::oob_take_bgk,
                                             sslbm::oob_take_io, sslbm::oob_take_stream,
                                             sslbm::oob_take_d2q9, sslbm::oob_take_d2q9a, sslbm::oob_take_vard,
-                                            sslbm::oob_take_kahan, sslbm::oob_take_diag, sslbm::oob_take_tile};
-  const int tu_site[] = {0, 100, 200, 300, 400, 500, 600, 700, 800, 900, 1100};  // offset by translation unit
+                                            sslbm::oob_take_kahan, sslbm::oob_take_diag, sslbm::oob_take_tile,
+                                            sslbm::oob_take_bgk_tile};
+  const int tu_site[] = {0, 100, 200, 300, 400, 500, 600, 700, 800, 900, 1100, 1200};  // offset by translation unit
   unsigned long long total = 0;
   sslbm::OobRecord first{};
   int first_site = -1;
-  for (int i = 0; i < 11; ++i) {
+  for (int i = 0; i < 12; ++i) {
     sslbm::OobRecord r{};
     if (take[i](&r) != 0) return fail(SSLBM_ERR_CUDA, "reading the bounds record of unit %d", i);
     if (r.count && first_site < 0) {

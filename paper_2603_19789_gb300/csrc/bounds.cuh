@@ -29,6 +29,7 @@ int oob_take_vard(OobRecord* out);
 int oob_take_kahan(OobRecord* out);
 int oob_take_diag(OobRecord* out);
 int oob_take_tile(OobRecord* out);
+int oob_take_bgk_tile(OobRecord* out);
 // Evaluate one check of index v against limit on the device, with no access behind it.
 cudaError_t launch_oob_probe(long long v, long long limit, cudaStream_t s);
 

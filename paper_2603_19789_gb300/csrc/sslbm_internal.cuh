@@ -330,6 +330,10 @@ cudaError_t launch_sslbm_blocked_diag(int precision, const GridView& g, const vo
 // compartment from / to a contiguous ny x nx plane of type rho_dtype.
 cudaError_t launch_bgk_step(int precision, const GridView& g, const void* coeffs, const void* f_in,
                             void* f_out, cudaStream_t s);
+// K such steps in one pass, FP32 (bgk_tile.cu), 1 <= K < 8; the depth that bgk_step takes.
+constexpr int kBgkDepth = 4;
+cudaError_t launch_bgk_tile(const GridView& g, const void* coeffs, const void* f_in, void* f_out, int K,
+                            cudaStream_t s);
 cudaError_t launch_bgk_init(int precision, const GridView& g, int comp, const void* rho,
                             int rho_dtype, void* f, cudaStream_t s);
 cudaError_t launch_bgk_density(int precision, const GridView& g, int comp, const void* f, void* rho,
