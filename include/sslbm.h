@@ -226,7 +226,8 @@ int sslbm_set_diffusivity_scale(sslbm_handle* h, const void* kx, const void* ky,
  * diffusion in FP32); n steps
  * take ceil(n / depth) passes whose depths differ by at most one.  Under the default blocking,
  * small grids of the FP32 and FP32_DEV storages, of D2Q9 and of the varying diffusion take
- * passes of their own depth, chosen by the grid and n.  Results do not depend on
+ * passes of their own depth, chosen by the grid and n, and the varying diffusion and the SPLIT
+ * and KAHAN storages passes of six and eight steps where n allows.  Results do not depend on
  * the depth: every depth performs the same floating-point operations in the same order.
  * Enqueues on the handle's stream and returns. */
 int sslbm_step(sslbm_handle* h, int64_t n);

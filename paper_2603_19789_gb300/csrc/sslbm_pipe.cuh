@@ -20,11 +20,21 @@
 // image, so they are substituted into the row update instead.
 #pragma once
 #include <cfloat>
+#include <type_traits>
 
 #include "bounds.cuh"
 #include "sslbm_internal.cuh"
 
 namespace sslbm {
+
+// Rows and columns inside a tile (a side is at most 2^30).  In 32 bits, the index arithmetic of
+// warp 0, which also copies the level-0 rows and which the other warps wait for, is shorter:
+// us per step at 8192^2, varying diffusion 315 -> 279 at depth 6, Kahan 437 -> 414 at depth 8,
+// D2Q9 no-flux 245 -> 222 at depth 4.  The plain, deviation and split storages keep 64 bits: the
+// compiler's schedule of their lighter rows came out slower with 32 (plain 153 -> 162 at depth 4,
+// split 191 -> 202 at depth 8).
+template <int MODE>
+using pipe_index_t = std::conditional_t<MODE == MODE_PLAIN || MODE == MODE_DEV || MODE == MODE_SPLIT, int64_t, int>;
 
 constexpr int kRing0 = 8;  // level-0 rows per tile in the ring: four pairs, three in flight
 
@@ -153,11 +163,11 @@ __device__ __forceinline__ void cell_row(const Coeffs<float>& k, const float2 (&
 template <bool ROWWALL, bool WALLS, bool ALIGNED = false>
 __device__ __forceinline__ void cell_row9(const Coeffs<float>& k, const GridView& g, const float2 (&P)[5][2],
                                           const float2 (&C)[5][2], const float2 (&N)[5][2], float2 (&M)[5][2],
-                                          const int64_t xs, const int64_t row) {
+                                          const int xs, const int row) {
   constexpr unsigned kFull = 0xffffffffu;
   const bool wl = WALLS && xs == 0;                            // column 0 is x = 0
-  const int jr = WALLS ? (int)(g.nx - 1 - xs) : -1;           // column of x = nx - 1, if in [0, 3]
-  const bool wd = ROWWALL && row == 0, wu = ROWWALL && row == g.ny - 1;
+  const int jr = WALLS ? (int)g.nx - 1 - xs : -1;             // column of x = nx - 1, if in [0, 3]
+  const bool wd = ROWWALL && row == 0, wu = ROWWALL && row == (int)g.ny - 1;
 #pragma unroll
   for (int h = 0; h < 2; ++h) {
     float2 lp[4];
@@ -314,11 +324,11 @@ __device__ __forceinline__ void cell_row_kahan(const Coeffs<float>& k, const flo
 // DIAG: the last warp also stores the row into slot row `which` of dsl (the parity's
 // diagnostics rows; zeros for cells outside the tile's output) and takes the largest I of
 // the cells it writes into *pk.
-template <int K, int NF, bool DIAG = false>
+template <int K, int NF, bool DIAG = false, class Idx = int>
 __device__ __forceinline__ void emit_row(PipeSmem<K, NF>& sm, const GridView& g, const float2 (&M)[NF][2],
                                          float* __restrict__ out, const int s, const int lane, const int par,
-                                         const int which, const bool writer, const int64_t xs, const int64_t r,
-                                         const int64_t y0, const int64_t y1, float* dsl = nullptr,
+                                         const int which, const bool writer, const Idx xs, const Idx r,
+                                         const Idx y0, const Idx y1, float* dsl = nullptr,
                                          float* pk = nullptr) {
   if (s < K - 1) {
     float* dst = &sm.rl[s < K - 1 ? s : 0][par][which][0][4 * lane];
@@ -330,7 +340,8 @@ __device__ __forceinline__ void emit_row(PipeSmem<K, NF>& sm, const GridView& g,
   if constexpr (DIAG) {
     const bool rv = writer && r >= y0 && r < y1;
     // columns xs + j that lie in the grid (a writer's first column always does)
-    const bool c1 = xs + 1 < g.nx, c2 = xs + 2 < g.nx, c3 = xs + 3 < g.nx;
+    const Idx nx = (Idx)g.nx;
+    const bool c1 = xs + 1 < nx, c2 = xs + 2 < nx, c3 = xs + 3 < nx;
     float* d = dsl + which * (NF * 128) + 4 * lane;
 #pragma unroll
     for (int f = 0; f < NF; ++f) {
@@ -347,8 +358,8 @@ __device__ __forceinline__ void emit_row(PipeSmem<K, NF>& sm, const GridView& g,
     }
   }
   if (writer && r >= y0 && r < y1 && SSLBM_IN(r, 1, g.ny, 5)) {
-    float* o = out + r * g.pitch + xs;
-    if (xs + 3 < g.nx) {
+    float* o = out + (int64_t)r * g.pitch + xs;
+    if (xs + 3 < (Idx)g.nx) {
       if (SSLBM_IN(xs, 4, g.nx, 6)) {
 #pragma unroll
         for (int f = 0; f < NF; ++f)
@@ -360,7 +371,7 @@ __device__ __forceinline__ void emit_row(PipeSmem<K, NF>& sm, const GridView& g,
         const float v[4] = {M[f][0].x, M[f][0].y, M[f][1].x, M[f][1].y};
 #pragma unroll
         for (int jj = 0; jj < 4; ++jj)
-          if (xs + jj < g.nx && SSLBM_IN(xs + jj, 1, g.nx, 7)) o[f * g.plane + jj] = v[jj];
+          if (xs + jj < (Idx)g.nx && SSLBM_IN(xs + jj, 1, g.nx, 7)) o[f * g.plane + jj] = v[jj];
       }
     }
   }
@@ -370,12 +381,12 @@ __device__ __forceinline__ void emit_row(PipeSmem<K, NF>& sm, const GridView& g,
 // 128 NF floats further), compute level-(s+1) rows b-1 (from A = b-2, B = b-1, N0) and b (from
 // B, N0, N1), hand them on or write them as rows r, r+1.  Ends with the CTA barrier.
 // DIAG: dsl, pk as in emit_row (dsl: the diagnostics rows of parity par).
-template <int MODE, int K, bool COLW = true, bool DIAG = false, int NF = mode_planes<MODE>()>
+template <int MODE, int K, bool COLW = true, bool DIAG = false, int NF = mode_planes<MODE>(), class Idx = int>
 __device__ __forceinline__ void pipe_pair(PipeSmem<K, NF>& sm, const GridView& g, const Coeffs<float>& k,
                                           const float* src, const float2 (&A)[NF][2], const float2 (&B)[NF][2],
                                           float2 (&N0)[NF][2], float2 (&N1)[NF][2], float* __restrict__ out,
                                           const int s, const int lane, const int par, const bool writer,
-                                          const int64_t xs, const int64_t r, const int64_t y0, const int64_t y1,
+                                          const Idx xs, const Idx r, const Idx y0, const Idx y1,
                                           const float* rk = nullptr, const int sk = 0, float* dsl = nullptr,
                                           float* pk = nullptr) {
   auto load_row = [&](const float* p, float2 (&R)[NF][2]) {
@@ -392,18 +403,18 @@ __device__ __forceinline__ void pipe_pair(PipeSmem<K, NF>& sm, const GridView& g
     // the nine-point stencil's wider neighbourhood
     constexpr bool W = MODE == MODE_D2Q9_NOFLUX || MODE == MODE_D2Q9_NOFLUX4;
     constexpr bool AL = MODE == MODE_D2Q9_NOFLUX4;
-    const int64_t row = r + 3 * (K - 1 - s);  // the first row this warp computes (r: the last warp's)
+    const int row = (int)r + 3 * (K - 1 - s);  // the first row this warp computes (r: the last warp's)
     load_row(src, N0);
-    if (W && (row == 0 || row == g.ny - 1))
-      cell_row9<true, W>(k, g, A, B, N0, M, xs, row);
+    if (W && (row == 0 || row == (int)g.ny - 1))
+      cell_row9<true, W>(k, g, A, B, N0, M, (int)xs, row);
     else
-      cell_row9<false, W && COLW, AL>(k, g, A, B, N0, M, xs, row);
+      cell_row9<false, W && COLW, AL>(k, g, A, B, N0, M, (int)xs, row);
     emit_row<K, NF, DIAG>(sm, g, M, out, s, lane, par, 0, writer, xs, r, y0, y1, dsl, pk);
     load_row(src + 128 * NF, N1);
-    if (W && (row + 1 == 0 || row + 1 == g.ny - 1))
-      cell_row9<true, W>(k, g, B, N0, N1, M, xs, row + 1);
+    if (W && (row + 1 == 0 || row + 1 == (int)g.ny - 1))
+      cell_row9<true, W>(k, g, B, N0, N1, M, (int)xs, row + 1);
     else
-      cell_row9<false, W && COLW, AL>(k, g, B, N0, N1, M, xs, row + 1);
+      cell_row9<false, W && COLW, AL>(k, g, B, N0, N1, M, (int)xs, row + 1);
   } else if constexpr (MODE == MODE_KAHAN) {
     // ten planes: the second row of the pair is read after the first is done
     load_row(src, N0);
@@ -444,7 +455,7 @@ __device__ __forceinline__ void pipe_pair(PipeSmem<K, NF>& sm, const GridView& g
 template <int MODE, int K, bool WRAP16 = false, bool COLW = true, bool DIAG = false, int NF = mode_planes<MODE>()>
 __device__ __forceinline__ void pipe_tile(PipeSmem<K, NF>& sm, const GridView& g, const Coeffs<float>& k,
                                           const float* __restrict__ in, float* __restrict__ out,
-                                          const int strip, const int64_t y0, const int64_t y1,
+                                          const int strip, const int64_t seg0, const int64_t seg1,
                                           const float* __restrict__ kx = nullptr,
                                           const float* __restrict__ ky = nullptr, float* rk = nullptr,
                                           DiagSmem<NF>* dsm = nullptr, double* __restrict__ diag = nullptr,
@@ -454,13 +465,15 @@ __device__ __forceinline__ void pipe_tile(PipeSmem<K, NF>& sm, const GridView& g
   constexpr int WV = 128 - 8 * HL;  // columns written per strip
   const int lane = threadIdx.x & 31;
   const int s = threadIdx.x >> 5;  // this warp computes level s + 1
-  const int64_t xs = (int64_t)strip * WV - 4 * HL + 4 * lane;
-  const bool vec_ok = xs >= 0 && xs + 3 < g.nx;
-  const bool writer = lane >= HL && lane < 32 - HL && xs < g.nx;
+  using Idx = pipe_index_t<MODE>;
+  const Idx nx = (Idx)g.nx, ny = (Idx)g.ny, y0 = (Idx)seg0, y1 = (Idx)seg1;
+  const Idx xs = (Idx)strip * WV - 4 * HL + 4 * lane;
+  const bool vec_ok = xs >= 0 && xs + 3 < nx;
+  const bool writer = lane >= HL && lane < 32 - HL && xs < nx;
   // A column more than K cells outside the domain cannot influence a written cell within
   // K steps, so lanes made only of such columns (the tail of the last strip) load nothing.
-  const bool loads = xs < g.nx + K && xs + 3 >= -K;
-  const int64_t xw = WRAP16 ? ((xs % g.nx) + g.nx) % g.nx : xs;
+  const bool loads = xs < nx + K && xs + 3 >= -K;
+  const Idx xw = WRAP16 ? ((xs % nx) + nx) % nx : xs;
   int xm[4];  // ghost images of this lane's columns, for lanes on a domain edge
 #pragma unroll
   for (int j = 0; j < 4; ++j) xm[j] = (int)ghost_index(xs + j, g.nx, g.bc);
@@ -468,9 +481,9 @@ __device__ __forceinline__ void pipe_tile(PipeSmem<K, NF>& sm, const GridView& g
   // b, b+1 with b = qa + 2t - 3s (warp 0 from the ring, the others from the previous warp's
   // output of iteration t-1) and computes level-(s+1) rows b-1 and b.  Level-0 rows span
   // [y0-K, y1+K); the last warp finishes row y1-1 once b >= y1-1 for s = K-1.
-  const int64_t qa = y0 - K, load_end = y1 + K;
+  const Idx qa = y0 - K, load_end = y1 + K;
   const int nt = (int)(((y1 - y0) + 4 * K - 4 + 1) / 2) + 1;
-  const int64_t rbase = qa - 3 * (K - 1) - 1;  // the first row the last warp emits (iteration 0)
+  const Idx rbase = qa - 3 * (K - 1) - 1;  // the first row the last warp emits (iteration 0)
 
   for (int i = threadIdx.x; i < kRing0 * NF * 128; i += 32 * K) (&sm.r0[0][0][0])[i] = 0.f;
   for (int i = threadIdx.x; i < (K - 1) * 2 * 2 * NF * 128; i += 32 * K) (&sm.rl[0][0][0][0][0])[i] = 0.f;
@@ -480,12 +493,12 @@ __device__ __forceinline__ void pipe_tile(PipeSmem<K, NF>& sm, const GridView& g
     for (int i = threadIdx.x; i < 2 * 2 * NF * 128; i += 32 * K) (&dsm->rows[0][0][0][0])[i] = 0.f;
   __syncthreads();
 
-  auto issue = [&](int64_t q) {  // warp 0: copy level-0 row q into its ring slot
+  auto issue = [&](Idx q) {  // warp 0: copy level-0 row q into its ring slot
     if (!loads || q >= load_end) return;
     const int slot = (int)((q - qa) % kRing0);
-    const int64_t yq = ghost_index(q, g.ny, g.bc);
+    const Idx yq = q >= 0 && q < ny ? q : (Idx)ghost_index(q, g.ny, g.bc);
     if (!SSLBM_IN(yq, 1, g.ny, 1)) return;
-    const int64_t row = yq * g.pitch;
+    const int64_t row = (int64_t)yq * g.pitch;
     // the state planes, and on the varying-diffusion lattice the two scale planes (static ring)
 #pragma unroll
     for (int f = 0; f < (MODE == MODE_VARD ? NF + 2 : NF); ++f) {
