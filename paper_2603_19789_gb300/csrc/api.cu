@@ -267,18 +267,6 @@ static int default_seg(const sslbm_handle* h, int k) {
                                             : sslbm::blocked_default_seg_rows(h->g.precision, h->gv, k);
 }
 
-// Steps per pipeline pass that the default blocking takes where n allows.  Measured at automatic
-// segments, no-flux, us per step of 48 steps at depth 4 against the depth below, at 8192^2, 2048^2
-// and 1700 x 1500: varying diffusion 350 -> 247, 25.3 -> 18.8, 16 -> 13; Kahan 478 -> 410, 34.6 ->
-// 29.6, 23 -> 20.3; split 213 -> 192, 16.5 -> 15.1, 11.8 -> 10.6.  The plain storage gains 5% at
-// depth 8 on 8192^2 and loses 13% on 3786 x 6055, D2Q9 is as uneven: those stay at 4.
-static int default_pass_depth(const sslbm_handle* h) {
-  if (h->g.lattice == SSLBM_LATTICE_D2Q5_VARD) return 6;
-  if (h->g.lattice == SSLBM_LATTICE_D2Q5 && (h->g.precision == SSLBM_FP32_SPLIT || h->g.precision == SSLBM_FP32_KAHAN))
-    return 8;
-  return 4;
-}
-
 int sslbm_create(const sslbm_grid* g, const sslbm_params* p, void* dev_ws, size_t ws_bytes,
                  void* stream, sslbm_handle** out) {
   if (!out) return fail(SSLBM_ERR_BAD_ARG, "out is NULL");
@@ -598,7 +586,7 @@ int sslbm_step(sslbm_handle* h, int64_t n) {
   const bool blocked = can_block(h);
   bool tiles = blocked && h->auto_blocking && !h->fuse_diag;
   // under the default blocking, the depth of most passes (a tuned or set blocking has depth or segment of its own)
-  const int deep = tiles && h->depth > 1 && h->seg_rows == 0 ? default_pass_depth(h) : h->depth;
+  const int deep = tiles && h->depth > 1 && h->seg_rows == 0 ? sslbm::default_pass_depth(h->g.lattice, h->g.precision) : h->depth;
   if (n > 0) h->diag_ready = false;
   while (n > 0) {
     int k = 1;
@@ -621,12 +609,8 @@ int sslbm_step(sslbm_handle* h, int64_t n) {
     }
     if (blocked && h->depth > 1 && n > 1) {
       // depth >= 2: the temporal-blocked kernel; a single step uses the one-step kernel,
-      // which produces the same bits.  The n steps take ceil(n / depth) passes whose depths
-      // differ by at most one (100 steps at depth 7: 10 of 7 and 5 of 6), rather than full
-      // passes and a shallow remainder, which runs at a lower rate per step.
-      // Passes deeper than h->depth are taken whole, where they leave at least three steps or none.
-      const int64_t passes = (n + h->depth - 1) / h->depth;
-      k = deep > h->depth && (n == deep || n >= deep + 3) ? deep : (int)((n + passes - 1) / passes);
+      // which produces the same bits.
+      k = sslbm::next_pass_depth(n, h->depth, deep);
       int seg = h->seg_rows;
       if (seg <= 0) {
         if (!h->seg_cache[k]) h->seg_cache[k] = default_seg(h, k);

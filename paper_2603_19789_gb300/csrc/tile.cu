@@ -278,16 +278,16 @@ cudaError_t launch_nr(const GridView& g, const void* coeffs, const void* in, voi
   }
 }
 
-// Measured on a GB300 (us): one wave of tile passes takes fix + depth * step, by rows per warp; the
-// row pipeline at its default depth (4) takes 4.5 + iterations * (it + it_cta * CTAs per SM).
+// Measured on a GB300 (us): one wave of tile passes takes fix + depth * step, by rows per warp; a
+// pass of the row pipeline takes pass + waves * iterations * (it + it_warp * warps per SM).
 struct TileCost {
   double fix[3], step[3];  // 1, 2, 4 rows per warp
-  double it, it_cta;
+  double pass, it, it_warp;
 };
-constexpr TileCost kCostD2q5{{2.1, 3.5, 4.5}, {0.38, 0.44, 0.77}, 0.70, 0.15};
-constexpr TileCost kCostD2q9{{2.1, 3.5, 4.5}, {0.40, 0.50, 1.05}, 0.90, 0.19};
-constexpr TileCost kCostD2q9Walls{{2.1, 2.8, 4.0}, {0.47, 0.85, 1.90}, 1.55, 0.37};
-constexpr TileCost kCostVard{{2.1, 2.8, 4.3}, {0.42, 0.80, 1.90}, 1.15, 0.33};
+constexpr TileCost kCostD2q5{{2.1, 3.5, 4.5}, {0.38, 0.44, 0.77}, 6.4, 0.43, 0.053};
+constexpr TileCost kCostD2q9{{2.1, 3.5, 4.5}, {0.40, 0.50, 1.05}, 5.9, 0.54, 0.068};
+constexpr TileCost kCostD2q9Walls{{2.1, 2.8, 4.0}, {0.47, 0.85, 1.90}, 18.9, 0.21, 0.134};
+constexpr TileCost kCostVard{{2.1, 2.8, 4.3}, {0.42, 0.80, 1.90}, 7.25, 0.65, 0.083};
 
 int sm_count() {
   static std::atomic<int> cache[64];
@@ -303,9 +303,12 @@ int sm_count() {
 
 // The cheaper of the two by the measured costs: tile passes recompute their halo but need no
 // pipeline fill, so they win where a pipeline would have only short segments to stream.  At the
-// shapes measured (128^2 .. 2048^2) the estimate picks the faster side except within 10% of the
-// crossing, near 1500^2 for D2Q5 (8.6 and 8.7 us per step at 1536^2) and D2Q9 (10.2 and 10.9),
-// 1500 x 1100 for the varying diffusion (11.4 and 11.6), beyond 2048^2 for the D2Q9 walls (27 and 35).
+// shapes measured (14 grids from 128^2 to 4096^2, 12000 x 300 and 430 x 5304 among them, 2 to 24
+// steps) the side it picks is 0.3% slower on average than the faster one: at most 9% for D2Q5 (1300
+// x 1000, 2 steps: 8.2 and 8.9 us per step), 14% D2Q9, 7% with walls, 3% the varying diffusion.
+// The lines, in us per step of 24 (tile, pipeline): D2Q5 430 x 5304 9.2 and 8.7, 1300 x 1000 5.0
+// and 5.8; varying diffusion 1300 x 1000 8.4 and 8.2; D2Q9 walls 2048^2 27.6 and 31.4, 3000 x 2200
+// 43.7 and 37.1.
 bool tile_plan(int lattice, int precision, const GridView& g, int64_t n, TilePlan* plan) {
   const bool d2q5 = lattice == SSLBM_LATTICE_D2Q5 && (precision == SSLBM_FP32 || precision == SSLBM_FP32_DEV);
   const bool other = (lattice == SSLBM_LATTICE_D2Q9 || lattice == SSLBM_LATTICE_D2Q5_VARD) && precision == SSLBM_FP32;
@@ -327,13 +330,22 @@ bool tile_plan(int lattice, int precision, const GridView& g, int64_t n, TilePla
       }
     }
   }
-  // the pipeline: 120-column strips, as many segments as make one wave of 4 CTAs per SM
-  const double strips = std::ceil(g.nx / 120.0);
-  const double rows = std::max(16.0, std::ceil(g.ny / std::max(1.0, std::floor(4 * sms / strips))));
-  const double ctas = strips * std::ceil(g.ny / rows);
-  const double waves = std::ceil(ctas / (4 * sms));
-  const double depth = n < 4 ? n : 4;
-  const double pipe = (4.5 + waves * ((rows + 12) / 2 + 1) * (c.it + c.it_cta * std::min(4.0, ctas / sms))) / depth;
+  // the pipeline's passes as sslbm_step cuts n steps (beyond 48 the pattern repeats): as many row
+  // segments as its automatic length makes
+  const int m = (int)std::min<int64_t>(n, 48), deep = default_pass_depth(lattice, precision);
+  double us[SSLBM_MAX_DEPTH + 1] = {0.0}, pipe = 0.0;
+  for (int left = m; left > 0;) {
+    const int k = next_pass_depth(left, 4, deep);
+    if (us[k] == 0.0) {
+      const double res = sms * (16 / k), strips = std::ceil((double)g.nx / (128 - 8 * ((k + 3) / 4)));
+      const double segs = std::max(1.0, std::floor((&c == &kCostD2q9Walls ? 2 : 1) * res / strips));
+      const double rows = std::max(4.0 * k, std::ceil(g.ny / segs)), ctas = strips * std::ceil(g.ny / rows);
+      us[k] = c.pass + std::ceil(ctas / res) * (std::floor((rows + 4 * k - 3) / 2) + 1) *
+                           (c.it + c.it_warp * k * std::min((double)(16 / k), ctas / sms));
+    }
+    pipe += us[k] / m;
+    left -= k;
+  }
   return best <= pipe;
 }
 
