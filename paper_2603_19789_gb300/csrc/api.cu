@@ -156,6 +156,7 @@ struct sslbm_handle {
   int depth = 1, seg_rows = 0;
   bool auto_blocking = true;  // the default blocking, or an autotuned choice of the tile passes
   int seg_cache[SSLBM_MAX_DEPTH + 1] = {0};
+  int last_pass = 0;  // depth of the call's last pass, 0 before the first and after a tile pass
   bool fuse_diag = false;   // sslbm_set_fused_diagnostics
   bool diag_ready = false;  // diag_result() holds the diagnostics of the current SSLBM state
 
@@ -235,6 +236,11 @@ static bool can_block(const sslbm_handle* h) {
 // One pass of k steps (k = 1: the one-step kernel) from the current buffer into the spare one,
 // on the D2Q5 or D2Q9 lattice.
 static cudaError_t launch_pass(sslbm_handle* h, int k, int seg) {
+  // A pass after one of the same depth in this call is a dependent launch; after another depth, whose
+  // CTAs are of another size, the early CTAs gather on the SMs that empty first: 7 steps (4 + 3)
+  // at 430 x 5304 11.9 us per step dependent and 10.0 ordinary, 10 steps at 4096^2 46.7 and 43.8.
+  const bool chained = h->last_pass == k;
+  h->last_pass = k;
   const bool q9 = h->g.lattice == SSLBM_LATTICE_D2Q9;
   void* out = h->s_buf[1 - h->s_cur];
   if (h->g.lattice == SSLBM_LATTICE_D2Q5_VARD) {  // scale planes kx, ky in the kappa area
@@ -243,19 +249,22 @@ static cudaError_t launch_pass(sslbm_handle* h, int k, int seg) {
     if (k == 1)
       return sslbm::launch_sslbm_vard_step(h->g.precision, h->gv, h->coeffs(), kx, ky, h->s_buf[h->s_cur], out,
                                            h->stream);
-    return sslbm::launch_sslbm_vard_blocked(h->gv, &h->cf, kx, ky, h->s_buf[h->s_cur], out, k, seg, h->stream);
+    return sslbm::launch_sslbm_vard_blocked(h->gv, &h->cf, kx, ky, h->s_buf[h->s_cur], out, k, seg, chained, h->stream);
   }
   if (k == 1 && h->g.precision == SSLBM_FP64_DW)  // the double word: its own streaming cell
     return sslbm::launch_stream_dw(h->gv, h->coeffs(), h->s_buf[h->s_cur], out, h->stream);
   if (k == 1)
     return q9 ? sslbm::launch_sslbm9_step1(h->g.precision, h->gv, h->coeffs(), h->s_buf[h->s_cur], out, h->stream)
-              : sslbm::launch_sslbm_step1(h->g.precision, h->gv, h->coeffs(), h->s_buf[h->s_cur], out, h->stream);
-  return q9 ? sslbm::launch_sslbm9_blocked(h->gv, &h->cf, h->s_buf[h->s_cur], out, k, seg, h->stream)
-            : sslbm::launch_sslbm_blocked(h->g.precision, h->gv, &h->cf, h->s_buf[h->s_cur], out, k, seg, h->stream);
+              : sslbm::launch_sslbm_step1(h->g.precision, h->gv, h->coeffs(), h->s_buf[h->s_cur], out, chained,
+                                          h->stream);
+  return q9 ? sslbm::launch_sslbm9_blocked(h->gv, &h->cf, h->s_buf[h->s_cur], out, k, seg, chained, h->stream)
+            : sslbm::launch_sslbm_blocked(h->g.precision, h->gv, &h->cf, h->s_buf[h->s_cur], out, k, seg, chained,
+                                          h->stream);
 }
 
 // One register-tile pass of k steps (tile.cu), the same buffers.
 static cudaError_t launch_tile_pass(sslbm_handle* h, int nr, int k) {
+  h->last_pass = 0;
   const char* ky = h->kappa ? h->kappa + h->L.plane_bytes : nullptr;
   return sslbm::launch_tile(h->g.lattice, h->g.precision, h->gv, &h->cf, h->s_buf[h->s_cur], h->s_buf[1 - h->s_cur],
                             h->kappa, ky, nr, k, h->stream);
@@ -586,8 +595,10 @@ int sslbm_step(sslbm_handle* h, int64_t n) {
   const bool blocked = can_block(h);
   bool tiles = blocked && h->auto_blocking && !h->fuse_diag;
   // under the default blocking, the depth of most passes (a tuned or set blocking has depth or segment of its own)
-  const int deep = tiles && h->depth > 1 && h->seg_rows == 0 ? sslbm::default_pass_depth(h->g.lattice, h->g.precision) : h->depth;
+  const int deep =
+      tiles && h->depth > 1 && h->seg_rows == 0 ? sslbm::default_pass_depth(h->g.lattice, h->g.precision) : h->depth;
   if (n > 0) h->diag_ready = false;
+  h->last_pass = 0;
   while (n > 0) {
     int k = 1;
     cudaError_t e;

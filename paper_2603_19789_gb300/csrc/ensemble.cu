@@ -616,7 +616,7 @@ int sslbm_ensemble_run(sslbm_ensemble* e, int64_t nsteps) {
       for (int i = 0; i < e->n; ++i) {
         cudaError_t ce = sslbm::launch_sslbm_step1(e->precision, e->gv(i), &e->tab[i].k,
                                                    e->buf(e->cur) + e->L.elem_off[i],
-                                                   e->buf(1 - e->cur) + e->L.elem_off[i], e->stream);
+                                                   e->buf(1 - e->cur) + e->L.elem_off[i], true, e->stream);
         if (ce != cudaSuccess) return cuda_err(ce, "remainder step");
       }
       e->cur = 1 - e->cur;

@@ -2,7 +2,8 @@
 // next launch's CTAs are scheduled, and compute their indices, while the last CTAs of the current
 // one still run.  A kernel launched by launch_pdl calls pdl_enter() before its first global access;
 // it returns when every earlier kernel of the stream has completed and its writes are visible, so the
-// order of memory accesses is that of ordinary launches.
+// order of memory accesses is that of ordinary launches.  launch_pdl_if(false, ...) is an ordinary
+// launch, for which pdl_enter() does nothing.
 #pragma once
 #include <cuda_runtime.h>
 
@@ -16,7 +17,8 @@ __device__ __forceinline__ void pdl_enter() {
 }
 
 template <typename... P, typename... A>
-cudaError_t launch_pdl(void (*kern)(P...), dim3 grid, dim3 block, size_t smem, cudaStream_t s, A&&... args) {
+cudaError_t launch_pdl_if(bool dependent, void (*kern)(P...), dim3 grid, dim3 block, size_t smem, cudaStream_t s,
+                          A&&... args) {
   cudaLaunchAttribute at[1];
   at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
   at[0].val.programmaticStreamSerializationAllowed = 1;
@@ -26,8 +28,13 @@ cudaError_t launch_pdl(void (*kern)(P...), dim3 grid, dim3 block, size_t smem, c
   cfg.dynamicSmemBytes = smem;
   cfg.stream = s;
   cfg.attrs = at;
-  cfg.numAttrs = 1;
+  cfg.numAttrs = dependent ? 1 : 0;
   return cudaLaunchKernelEx(&cfg, kern, std::forward<A>(args)...);
+}
+
+template <typename... P, typename... A>
+cudaError_t launch_pdl(void (*kern)(P...), dim3 grid, dim3 block, size_t smem, cudaStream_t s, A&&... args) {
+  return launch_pdl_if(true, kern, grid, block, smem, s, std::forward<A>(args)...);
 }
 
 }  // namespace sslbm

@@ -15,10 +15,10 @@ int blocked9_default_seg_rows(const GridView& g, int depth) {
 }
 
 cudaError_t launch_sslbm9_blocked(const GridView& g, const void* coeffs, const void* in, void* out, int depth,
-                                  int seg_rows, cudaStream_t s) {
-  if (g.bc == 0) return launch_blocked_mode<MODE_D2Q9>(g, coeffs, in, out, depth, seg_rows, s);
-  if ((g.nx & 3) == 0) return launch_sslbm9_aligned_blocked(g, coeffs, in, out, depth, seg_rows, s);
-  return launch_blocked_mode<MODE_D2Q9_NOFLUX>(g, coeffs, in, out, depth, seg_rows, s);
+                                  int seg_rows, bool chained, cudaStream_t s) {
+  if (g.bc == 0) return launch_blocked_mode<MODE_D2Q9>(g, coeffs, in, out, depth, seg_rows, chained, s);
+  if ((g.nx & 3) == 0) return launch_sslbm9_aligned_blocked(g, coeffs, in, out, depth, seg_rows, chained, s);
+  return launch_blocked_mode<MODE_D2Q9_NOFLUX>(g, coeffs, in, out, depth, seg_rows, chained, s);
 }
 
 }  // namespace sslbm

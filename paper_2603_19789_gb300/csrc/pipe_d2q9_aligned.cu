@@ -12,8 +12,8 @@ int blocked9_aligned_default_seg_rows(const GridView& g, int depth) {
 }
 
 cudaError_t launch_sslbm9_aligned_blocked(const GridView& g, const void* coeffs, const void* in, void* out,
-                                          int depth, int seg_rows, cudaStream_t s) {
-  return launch_blocked_mode<MODE_D2Q9_NOFLUX4>(g, coeffs, in, out, depth, seg_rows, s);
+                                          int depth, int seg_rows, bool chained, cudaStream_t s) {
+  return launch_blocked_mode<MODE_D2Q9_NOFLUX4>(g, coeffs, in, out, depth, seg_rows, chained, s);
 }
 
 }  // namespace sslbm

@@ -23,8 +23,9 @@ cudaError_t launch_sslbm_blocked_diag(int precision, const GridView& g, const vo
                                       void* out, int depth, int seg_rows, double* partials, cudaStream_t s) {
   if (!blocked_diag_supported(precision, g, depth, seg_rows) || !partials) return cudaErrorInvalidValue;
   if (precision == SSLBM_FP32)
-    return launch_blocked_mode<MODE_PLAIN, true>(g, coeffs, in, out, depth, seg_rows, s, nullptr, nullptr, partials);
-  return launch_blocked_mode<MODE_DEV, true>(g, coeffs, in, out, depth, seg_rows, s, nullptr, nullptr, partials);
+    return launch_blocked_mode<MODE_PLAIN, true>(g, coeffs, in, out, depth, seg_rows, false, s, nullptr, nullptr,
+                                                 partials);
+  return launch_blocked_mode<MODE_DEV, true>(g, coeffs, in, out, depth, seg_rows, false, s, nullptr, nullptr, partials);
 }
 
 }  // namespace sslbm

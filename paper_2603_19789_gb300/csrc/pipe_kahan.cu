@@ -12,8 +12,8 @@ int blocked_kahan_default_seg_rows(const GridView& g, int depth) {
 }
 
 cudaError_t launch_kahan_blocked(const GridView& g, const void* coeffs, const void* in, void* out, int depth,
-                                 int seg_rows, cudaStream_t s) {
-  return launch_blocked_mode<MODE_KAHAN>(g, coeffs, in, out, depth, seg_rows, s);
+                                 int seg_rows, bool chained, cudaStream_t s) {
+  return launch_blocked_mode<MODE_KAHAN>(g, coeffs, in, out, depth, seg_rows, chained, s);
 }
 
 }  // namespace sslbm

@@ -75,7 +75,8 @@ constexpr int64_t pipe_strip_cols(int K) { return 128 - 8 * ((K + 3) / 4); }
 // DIAG: diag receives one 6-double partial per CTA (at most kDiagBlocks CTAs).
 template <int MODE, int K, bool DIAG = false>
 cudaError_t launch_blocked_t(const GridView& g, const void* coeffs, const void* in, void* out,
-                             int seg_rows, cudaStream_t s, const void* kx = nullptr, const void* ky = nullptr,
+                             int seg_rows, bool chained, cudaStream_t s, const void* kx = nullptr,
+                             const void* ky = nullptr,
                              double* diag = nullptr) {
   constexpr int64_t WV = pipe_strip_cols(K);
   prefer_shared<MODE, K, DIAG>();
@@ -85,10 +86,10 @@ cudaError_t launch_blocked_t(const GridView& g, const void* coeffs, const void* 
   const int64_t blocks = nstrips * nseg;
   if (blocks > 0x7fffffffLL) return cudaErrorInvalidConfiguration;
   if (DIAG && (blocks > kDiagBlocks || diag == nullptr)) return cudaErrorInvalidConfiguration;
-  return launch_pdl(pipe_kernel<MODE, K, DIAG>, dim3((unsigned)blocks), dim3(32 * K), pipe_smem_bytes<MODE, K, DIAG>(), s,
-                    g, *static_cast<const Coeffs<float>*>(coeffs), static_cast<const float*>(in),
-                    static_cast<float*>(out), seg_rows, (int)nstrips, static_cast<const float*>(kx),
-                    static_cast<const float*>(ky), diag);
+  return launch_pdl_if(chained, pipe_kernel<MODE, K, DIAG>, dim3((unsigned)blocks), dim3(32 * K),
+                       pipe_smem_bytes<MODE, K, DIAG>(), s, g, *static_cast<const Coeffs<float>*>(coeffs),
+                       static_cast<const float*>(in), static_cast<float*>(out), seg_rows, (int)nstrips,
+                       static_cast<const float*>(kx), static_cast<const float*>(ky), diag);
 }
 
 template <int MODE, int K>
@@ -113,16 +114,16 @@ int default_seg_rows_t(const GridView& g) {
 
 template <int MODE, bool DIAG = false>
 cudaError_t launch_blocked_mode(const GridView& g, const void* coeffs, const void* in, void* out,
-                                int depth, int seg_rows, cudaStream_t s, const void* kx = nullptr,
+                                int depth, int seg_rows, bool chained, cudaStream_t s, const void* kx = nullptr,
                                 const void* ky = nullptr, double* diag = nullptr) {
   switch (depth) {
-    case 2: return launch_blocked_t<MODE, 2, DIAG>(g, coeffs, in, out, seg_rows, s, kx, ky, diag);
-    case 3: return launch_blocked_t<MODE, 3, DIAG>(g, coeffs, in, out, seg_rows, s, kx, ky, diag);
-    case 4: return launch_blocked_t<MODE, 4, DIAG>(g, coeffs, in, out, seg_rows, s, kx, ky, diag);
-    case 5: return launch_blocked_t<MODE, 5, DIAG>(g, coeffs, in, out, seg_rows, s, kx, ky, diag);
-    case 6: return launch_blocked_t<MODE, 6, DIAG>(g, coeffs, in, out, seg_rows, s, kx, ky, diag);
-    case 7: return launch_blocked_t<MODE, 7, DIAG>(g, coeffs, in, out, seg_rows, s, kx, ky, diag);
-    case 8: return launch_blocked_t<MODE, 8, DIAG>(g, coeffs, in, out, seg_rows, s, kx, ky, diag);
+    case 2: return launch_blocked_t<MODE, 2, DIAG>(g, coeffs, in, out, seg_rows, chained, s, kx, ky, diag);
+    case 3: return launch_blocked_t<MODE, 3, DIAG>(g, coeffs, in, out, seg_rows, chained, s, kx, ky, diag);
+    case 4: return launch_blocked_t<MODE, 4, DIAG>(g, coeffs, in, out, seg_rows, chained, s, kx, ky, diag);
+    case 5: return launch_blocked_t<MODE, 5, DIAG>(g, coeffs, in, out, seg_rows, chained, s, kx, ky, diag);
+    case 6: return launch_blocked_t<MODE, 6, DIAG>(g, coeffs, in, out, seg_rows, chained, s, kx, ky, diag);
+    case 7: return launch_blocked_t<MODE, 7, DIAG>(g, coeffs, in, out, seg_rows, chained, s, kx, ky, diag);
+    case 8: return launch_blocked_t<MODE, 8, DIAG>(g, coeffs, in, out, seg_rows, chained, s, kx, ky, diag);
     default: return cudaErrorInvalidValue;
   }
 }

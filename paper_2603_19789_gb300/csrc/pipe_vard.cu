@@ -10,8 +10,9 @@ namespace sslbm {
 int blocked_vard_default_seg_rows(const GridView& g, int depth) { return default_seg_rows_mode<MODE_VARD>(g, depth); }
 
 cudaError_t launch_sslbm_vard_blocked(const GridView& g, const void* coeffs, const void* kx, const void* ky,
-                                      const void* in, void* out, int depth, int seg_rows, cudaStream_t s) {
-  return launch_blocked_mode<MODE_VARD>(g, coeffs, in, out, depth, seg_rows, s, kx, ky);
+                                      const void* in, void* out, int depth, int seg_rows, bool chained,
+                                      cudaStream_t s) {
+  return launch_blocked_mode<MODE_VARD>(g, coeffs, in, out, depth, seg_rows, chained, s, kx, ky);
 }
 
 }  // namespace sslbm

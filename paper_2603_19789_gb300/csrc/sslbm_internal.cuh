@@ -290,31 +290,30 @@ __device__ __forceinline__ void seird_cell2(const Coeffs<float>& k, float2 x0, f
 // deviation-S, FP32 split-S and FP32 Kahan).  seg_rows > 0 is the blocked kernel's row-segment
 // length.
 cudaError_t launch_sslbm_step1(int precision, const GridView& g, const void* coeffs, const void* in,
-                               void* out, cudaStream_t s);
+                               void* out, bool chained, cudaStream_t s);
 // The streaming one-step kernel (stream.cu) of the FP32 storages: FP32, FP32 deviation-S,
 // FP32 split-S and the Kahan storage.
 cudaError_t launch_stream_d2q5(int precision, const GridView& g, const void* coeffs, const void* in, void* out,
                                cudaStream_t s);
 cudaError_t launch_sslbm_blocked(int precision, const GridView& g, const void* coeffs,
-                                 const void* in, void* out, int depth, int seg_rows,
-                                 cudaStream_t s);
+                                 const void* in, void* out, int depth, int seg_rows, bool chained, cudaStream_t s);
 bool blocked_supported(int precision, const GridView& g);
 // The Kahan storage's blocked kernel (pipe_kahan.cu) and its default segment.
 cudaError_t launch_kahan_blocked(const GridView& g, const void* coeffs, const void* in, void* out, int depth,
-                                 int seg_rows, cudaStream_t s);
+                                 int seg_rows, bool chained, cudaStream_t s);
 int blocked_kahan_default_seg_rows(const GridView& g, int depth);
 // The D2Q9 lattice (plain FP32 storage): K fused steps per launch, and its default segment.
 cudaError_t launch_sslbm9_blocked(const GridView& g, const void* coeffs, const void* in, void* out, int depth,
-                                  int seg_rows, cudaStream_t s);
+                                  int seg_rows, bool chained, cudaStream_t s);
 int blocked9_default_seg_rows(const GridView& g, int depth);
 // ... under no-flux with nx a multiple of 4 (pipe_d2q9_aligned.cu)
 cudaError_t launch_sslbm9_aligned_blocked(const GridView& g, const void* coeffs, const void* in, void* out,
-                                          int depth, int seg_rows, cudaStream_t s);
+                                          int depth, int seg_rows, bool chained, cudaStream_t s);
 int blocked9_aligned_default_seg_rows(const GridView& g, int depth);
 // The varying-diffusion lattice (plain FP32 storage, scale planes kx, ky): K fused steps per
 // launch, and its default segment.
 cudaError_t launch_sslbm_vard_blocked(const GridView& g, const void* coeffs, const void* kx, const void* ky,
-                                      const void* in, void* out, int depth, int seg_rows, cudaStream_t s);
+                                      const void* in, void* out, int depth, int seg_rows, bool chained, cudaStream_t s);
 int blocked_vard_default_seg_rows(const GridView& g, int depth);
 // Segment length that makes one blocked launch a single wave of resident warps.
 int blocked_default_seg_rows(int precision, const GridView& g, int depth);

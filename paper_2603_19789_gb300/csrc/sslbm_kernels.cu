@@ -86,8 +86,11 @@ __global__ void __launch_bounds__(kStep1Threads) step1_kernel(const GridView g, 
 // and enough shared memory reserved that an SM holds two, one of this launch and one of the next:
 // with small CTAs the dependent launch's go where there is room and some SMs get twice the work
 // (200^2, us per step: 10.3 with 64 x 8 blocks of two cells, 8.2 with 64-thread CTAs, 10.6 with
-// those and dependent launches, 5.2 with even shares).  Larger grids: 64-thread CTAs.
-cudaError_t launch_step1_fp64(const GridView& g, const void* coeffs, const void* in, void* out, cudaStream_t s) {
+// those and dependent launches, 5.2 with even shares).  Only a step after a step is a dependent
+// launch: after another kernel, two CTAs may go to one SM, and stay together from step to step (8.0).
+// Larger grids: 64-thread CTAs.
+cudaError_t launch_step1_fp64(const GridView& g, const void* coeffs, const void* in, void* out, bool chained,
+                              cudaStream_t s) {
   constexpr size_t kReserve = 100 * 1024;
   static std::atomic<int> sms_of[64];  // multiprocessors; set after the kernel's shared-memory limit
   int dev = 0;
@@ -105,9 +108,9 @@ cudaError_t launch_step1_fp64(const GridView& g, const void* coeffs, const void*
   const int per = even ? (int)((cells + sms - 1) / sms) : 64;
   const int64_t ctas = (cells + per - 1) / per;  // up to 2^31 - 1: 1.4e11 cells, 5.5 TB per state
   if (ctas > 0x7fffffffLL) return cudaErrorInvalidConfiguration;
-  return launch_pdl(step1_kernel, dim3((unsigned)ctas), dim3((per + 31) / 32 * 32), even ? kReserve : 0, s, g,
-                    *static_cast<const Coeffs<double>*>(coeffs), static_cast<const double*>(in),
-                    static_cast<double*>(out), per);
+  return launch_pdl_if(chained, step1_kernel, dim3((unsigned)ctas), dim3((per + 31) / 32 * 32), even ? kReserve : 0, s,
+                       g, *static_cast<const Coeffs<double>*>(coeffs), static_cast<const double*>(in),
+                       static_cast<double*>(out), per);
 }
 
 }  // namespace
@@ -126,9 +129,9 @@ bool blocked_supported(int precision, const GridView&) {
 }
 
 cudaError_t launch_sslbm_step1(int precision, const GridView& g, const void* coeffs, const void* in,
-                               void* out, cudaStream_t s) {
+                               void* out, bool chained, cudaStream_t s) {
   switch (precision) {
-    case SSLBM_FP64: return launch_step1_fp64(g, coeffs, in, out, s);
+    case SSLBM_FP64: return launch_step1_fp64(g, coeffs, in, out, chained, s);
     case SSLBM_FP32:
     case SSLBM_FP32_DEV:
     case SSLBM_FP32_SPLIT:
@@ -138,15 +141,15 @@ cudaError_t launch_sslbm_step1(int precision, const GridView& g, const void* coe
 }
 
 cudaError_t launch_sslbm_blocked(int precision, const GridView& g, const void* coeffs,
-                                 const void* in, void* out, int depth, int seg_rows,
+                                 const void* in, void* out, int depth, int seg_rows, bool chained,
                                  cudaStream_t s) {
   if (precision == SSLBM_FP32)
-    return launch_blocked_mode<MODE_PLAIN>(g, coeffs, in, out, depth, seg_rows, s);
+    return launch_blocked_mode<MODE_PLAIN>(g, coeffs, in, out, depth, seg_rows, chained, s);
   if (precision == SSLBM_FP32_DEV)
-    return launch_blocked_mode<MODE_DEV>(g, coeffs, in, out, depth, seg_rows, s);
+    return launch_blocked_mode<MODE_DEV>(g, coeffs, in, out, depth, seg_rows, chained, s);
   if (precision == SSLBM_FP32_SPLIT)
-    return launch_blocked_mode<MODE_SPLIT>(g, coeffs, in, out, depth, seg_rows, s);
-  if (precision == SSLBM_FP32_KAHAN) return launch_kahan_blocked(g, coeffs, in, out, depth, seg_rows, s);
+    return launch_blocked_mode<MODE_SPLIT>(g, coeffs, in, out, depth, seg_rows, chained, s);
+  if (precision == SSLBM_FP32_KAHAN) return launch_kahan_blocked(g, coeffs, in, out, depth, seg_rows, chained, s);
   return cudaErrorInvalidValue;
 }
 
