@@ -43,8 +43,9 @@ LATTICE_STEPS_PER_STEP = 100
 BYTES_PER_CELL_FP32 = 40  # read + write of five FP32 planes per launch
 BYTES_PER_CELL_FP64 = 80
 FP64_FLOPS_PER_CELL = 46  # the SSLBM update per cell-step: four laplacians, sources, update
-BGK_BYTES_PER_CELL_FP32 = 168  # 20 populations + D, read and write
-FD4_PLANES_PER_CELL = 85  # RK4 stage kernels: 15 + 25 + 25 + 20 plane reads and writes per step
+BGK_BYTES_PER_CELL_FP32 = 168 / 4  # 20 populations + D, read and written once per pass of four steps
+# RK4 plane reads and writes per step: FP64 stage kernels 15 + 25 + 25 + 20, FP32 stage pairs 32
+FD4_PLANES_PER_CELL = {"fp64": 85, "fp32": 32}
 
 
 PIPE_SOURCES = ("paper_2603_19789_gb300/csrc/sslbm_pipe.cuh", "paper_2603_19789_gb300/csrc/sslbm_internal.cuh",
@@ -674,8 +675,8 @@ def secondary_timings(L, wl, state64, state32, stream, hbm):
         sv.close()
         del sv
         torch.cuda.empty_cache()
-    # the fourth-order finite-difference reference (RK4): four stage kernels per step that
-    # move 85 planes per cell (stage states, slope sum and u, read and written)
+    # the fourth-order finite-difference reference (RK4): four stage kernels (FP64) or two kernels
+    # of two stages (FP32) per step, which move the stage states, the slope sum and u
     for prec, name, esz, reps in ((L.FP64, "fp64", 8, 3), (L.FP32, "fp32", 4, 6)):
         f = L.Fd4(NX, NY, rates, wl["d"][:4], bc=wl["bc"], precision=prec)
         f.write(state64 if prec == L.FP64 else state32)
@@ -688,7 +689,7 @@ def secondary_timings(L, wl, state64, state32, stream, hbm):
         b.synchronize()
         ms = a.elapsed_time(b) / reps
         out[f"fd4_{name}_glups"] = cells / (ms * 1e-3) / 1e9
-        out[f"fd4_{name}_hbm_frac"] = FD4_PLANES_PER_CELL * esz * cells / (ms * 1e-3) / 1e9 / hbm
+        out[f"fd4_{name}_hbm_frac"] = FD4_PLANES_PER_CELL[name] * esz * cells / (ms * 1e-3) / 1e9 / hbm
         f.close()
         del f
         torch.cuda.empty_cache()
