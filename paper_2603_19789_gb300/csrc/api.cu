@@ -19,6 +19,7 @@
 #include "bounds.cuh"
 #include "sslbm_internal.cuh"
 #include "tile.cuh"
+#include "user_memory.cuh"
 #include "variants.cuh"
 
 using sslbm::Coeffs;
@@ -208,16 +209,14 @@ static bool ten_planes(const sslbm_handle* h) {
   return h->g.precision == SSLBM_FP32_KAHAN || h->g.precision == SSLBM_FP64_DW;
 }
 
-// Whether a kernel on the handle's device can use the caller's device buffer as values of this size;
-// memory of another device or of odd alignment is left to the copies.
+// Whether a kernel on the handle's device uses the caller's device buffer directly (user_memory.cuh).
 static bool kernel_access(const sslbm_handle* h, const void* p, size_t size) {
-  if (reinterpret_cast<uintptr_t>(p) % size) return false;
   cudaPointerAttributes attr;
   if (cudaPointerGetAttributes(&attr, p) != cudaSuccess) {
     cudaGetLastError();
     return false;
   }
-  return attr.type != cudaMemoryTypeDevice || attr.device == h->device;
+  return sslbm::kernel_may_use(attr.type, attr.device, h->device, reinterpret_cast<uintptr_t>(p), size);
 }
 
 // The compartments with a compensation plane: the first n.
