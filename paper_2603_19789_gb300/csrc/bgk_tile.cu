@@ -54,8 +54,7 @@ __device__ __forceinline__ void collide2(const Coeffs<float>& k, float2 (&f)[4][
 
 template <int NW>
 __global__ void __launch_bounds__(32 * NW, NW > 8 ? 1 : 2) bgk_tile_kernel(const GridView g, const Coeffs<float> k,
-                                                                          const float* __restrict__ fin,
-                                                                          float* __restrict__ fout, const int K,
+                                                                          const float* fin, float* fout, const int K,
                                                                           const int ntx) {
   constexpr int R = 2 * NW;
   // [step parity][warp][f_2 of the last row, f_4 of the first][compartment][lane]

@@ -290,8 +290,7 @@ constexpr size_t fd4_pair_smem() {
 template <int PAIR, int ORDER, int TY>
 __global__ void __launch_bounds__(256, TY > 8 ? 2 : 3)
     fd4_pair_kernel(const int nx, const int ny, const int pitch, const int bc, const Fd4Coeffs<float> k,
-                    const float* __restrict__ src, const float* __restrict__ u, float* __restrict__ acc,
-                    float* __restrict__ dst) {
+                    const float* src, const float* u, float* acc, float* dst) {
   constexpr int RA = TY + 8, RB = TY + 4, FA = RA * kPS, FB = RB * kPS, NR = TY / 8;
   static_assert(TY % 8 == 0, "whole rows per warp");
   extern __shared__ __align__(16) float fd4_smem[];

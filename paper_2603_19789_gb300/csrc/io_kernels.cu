@@ -53,8 +53,7 @@ __device__ __forceinline__ void st_vec(T* p, const Vec4<T>& r) {
 constexpr int kIoThreads = 128;
 
 template <typename T, typename U, bool WRITE>
-__global__ void __launch_bounds__(kIoThreads) planes_io_kernel(const GridView g, U* __restrict__ user,
-                                                               T* __restrict__ planes, T* __restrict__ comps,
+__global__ void __launch_bounds__(kIoThreads) planes_io_kernel(const GridView g, U* user, T* planes, T* comps,
                                                                const int n_comp, const int c0, const int dev_S,
                                                                const double s_ref, const int vec) {
   pdl_enter();

@@ -4,6 +4,10 @@
 // it returns when every earlier kernel of the stream has completed and its writes are visible, so the
 // order of memory accesses is that of ordinary launches.  launch_pdl_if(false, ...) is an ordinary
 // launch, for which pdl_enter() does nothing.
+// The pointers such a kernel reads through are not __restrict__: that would allow the compiler to read
+// them before pdl_enter(), or through the read-only path, whose data may not change while the kernel
+// runs -- and it runs while its predecessor writes them.  (The row pipeline, which reads memory by
+// cp.async in volatile assembly alone, may keep it.)
 #pragma once
 #include <cuda_runtime.h>
 

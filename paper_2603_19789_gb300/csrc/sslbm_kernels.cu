@@ -45,8 +45,7 @@ constexpr int kStep1Threads = 1024;
 // 15.2 GLUPS at 2 GHz; wider accesses would not help, the pipe takes 16 times longer over a cell
 // than its 21 loads do.  8192^2 13.95 GLUPS; two cells per thread with the earlier force_quot 11.8.
 __global__ void __launch_bounds__(kStep1Threads) step1_kernel(const GridView g, const Coeffs<double> k,
-                                                              const double* __restrict__ in,
-                                                              double* __restrict__ out, const int per) {
+                                                              const double* in, double* out, const int per) {
   pdl_enter();
   if ((int)threadIdx.x >= per) return;
   int64_t x, y;

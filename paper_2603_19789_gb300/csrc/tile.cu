@@ -120,9 +120,8 @@ __device__ __forceinline__ void tile_row(const Coeffs<float>& k, const float2* P
 
 template <int MODE, int NR>
 __global__ void __launch_bounds__(32 * kTW, 1) tile_kernel(const GridView g, const Coeffs<float> k,
-                                                           const float* __restrict__ in, float* __restrict__ out,
-                                                           const float* __restrict__ kx,
-                                                           const float* __restrict__ ky, const int K, const int ntx) {
+                                                           const float* in, float* out, const float* kx,
+                                                           const float* ky, const int K, const int ntx) {
   constexpr int R = kTW * NR;
   constexpr bool Q9 = MODE == MODE_D2Q9 || MODE == MODE_D2Q9_NOFLUX;
   extern __shared__ __align__(16) unsigned char tile_smem[];
