@@ -1247,10 +1247,7 @@ int backward_impl(sslbm_fno* f, int B, const float* x, const float* dy_out) {
   dim3 sgrid((unsigned)std::min<int64_t>(64, (5 * P + kThreads - 1) / kThreads), B);
   seed_sums_kernel<<<sgrid, kThreads, 0, f->stream>>>(dy_out, ycache, sums, 5 * P);
   CK(cudaGetLastError(), "seed sums");
-  // the fused kernels copy rows of x in 16-byte groups; forward refuses an x of another alignment, but
-  // backward may be given a copy of its own, which the separate kernels take as it is
-  if (sslbm::fno_fused::supported(W, L.m, L.H, L.n) && reinterpret_cast<uintptr_t>(x) % 16 == 0)
-    return backward_fused(f, B, x, dy_out, sums);
+  if (sslbm::fno_fused::supported(W, L.m, L.H, L.n)) return backward_fused(f, B, x, dy_out, sums);
   scale_dy_kernel<<<dim3(rows_grid(P), B), kThreads, 0, f->stream>>>(dy_out, x, ycache, sums,
                                                                     f->at<float>(f->bu.ratio), dy, P);
   CK(cudaGetLastError(), "output scale");
