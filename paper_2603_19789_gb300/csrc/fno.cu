@@ -1153,8 +1153,16 @@ int conserve(sslbm_fno* f, int B, const float* x, float* y, int store) {
   return SSLBM_OK;
 }
 
+// With n even every kernel that reads x takes 16 bytes at a time (the fused row kernels and the cell
+// tiles of the separate products), so that x has to start on such a boundary.
+int check_x(const sslbm_fno* f, const float* x) {
+  if (f->L.P % 4 == 0 && reinterpret_cast<uintptr_t>(x) % 16) return err(SSLBM_ERR_BAD_ARG, "x must be 16-byte aligned");
+  return SSLBM_OK;
+}
+
 int forward_impl(sslbm_fno* f, int B, const float* x, float* y, int store) {
-  int st;
+  int st = check_x(f, x);
+  if (st) return st;
   if (sslbm::fno_fused::supported(f->L.W, f->L.m, f->L.H, f->L.n))
     st = forward_fused(f, B, x, y, store);
   else
@@ -1420,6 +1428,7 @@ int sslbm_fno_backward(sslbm_fno* f, int batch, const float* x, const float* dy)
   if (!x || !dy) return err(SSLBM_ERR_BAD_ARG, "NULL argument");
   if (f->cached_batch != batch)
     return err(SSLBM_ERR_STATE, "backward needs a preceding sslbm_fno_forward on the same batch");
+  if ((st = check_x(f, x))) return st;
   DevGuard dg(f->device);
   return backward_impl(f, batch, x, dy);
 }
