@@ -24,6 +24,7 @@
 #include <cstdarg>
 #include <cstdio>
 #include <new>
+#include <utility>
 
 #include "pdl.cuh"
 #include "sslbm.h"
@@ -286,17 +287,18 @@ constexpr size_t fd4_pair_smem() {
 
 // u: the step's state; src: the input of the pair (PAIR 0: u); acc: running sum of the slopes
 // (PAIR 0: written); dst: PAIR 0 the next stage's state (S, E, I, R), PAIR 1 the next state, not
-// u or src.  Rows are pitch floats apart, a multiple of 4.
-template <int PAIR, int ORDER, int TY>
+// u or src.  VEC: nx is a multiple of 4, so that every row starts on a 16-byte boundary and four
+// cells move at a time; else one by one.
+template <int PAIR, int ORDER, int TY, bool VEC>
 __global__ void __launch_bounds__(256, TY > 8 ? 2 : 3)
-    fd4_pair_kernel(const int nx, const int ny, const int pitch, const int bc, const Fd4Coeffs<float> k,
+    fd4_pair_kernel(const int nx, const int ny, const int bc, const Fd4Coeffs<float> k,
                     const float* src, const float* u, float* acc, float* dst) {
   constexpr int RA = TY + 8, RB = TY + 4, FA = RA * kPS, FB = RB * kPS, NR = TY / 8;
   static_assert(TY % 8 == 0, "whole rows per warp");
   extern __shared__ __align__(16) float fd4_smem[];
   float* A = fd4_smem;          // [4][RA][kPS]: the input, rows by0 - 4 ..
   float* B = fd4_smem + 4 * FA;  // [4][RB][kPS]: the first stage's result, rows by0 - 2 ..
-  const int64_t M = (int64_t)pitch * ny;
+  const int64_t M = (int64_t)nx * ny;
   const int tid = threadIdx.x, lane = tid & 31, w = tid >> 5;
   const int ntx = (nx + kPX - 1) / kPX;
   const int bx0 = (int)(blockIdx.x % ntx) * kPX, by0 = (int)(blockIdx.x / ntx) * TY;
@@ -310,21 +312,32 @@ __global__ void __launch_bounds__(256, TY > 8 ? 2 : 3)
   for (int j = w; j < 4 * RA; j += 8) {
     const int c = j / RA, r = j - c * RA;
     if (by0 + r - 4 >= ny + 4) continue;
-    const float* row = src + c * M + (int64_t)ghost2i(by0 + r - 4, ny, bc) * pitch;
+    const float* row = src + c * M + (int64_t)ghost2i(by0 + r - 4, ny, bc) * nx;
     float* d = A + c * FA + r * kPS;
-    for (int q = lane; q < kPS / 4; q += 32) {
-      const int x = bx0 - 4 + 4 * q;
-      if (x >= nx + 4) continue;
-      if (x >= 0 && x + 3 < nx) {
-        asm volatile("cp.async.cg.shared.global [%0], [%1], 16;\n" ::"r"((unsigned)__cvta_generic_to_shared(d + 4 * q)),
-                     "l"(row + x)
-                     : "memory");
-      } else {
+    if constexpr (VEC) {
+      for (int q = lane; q < kPS / 4; q += 32) {
+        const int x = bx0 - 4 + 4 * q;
+        if (x >= nx + 4) continue;
+        if (x >= 0 && x + 3 < nx) {
+          asm volatile("cp.async.cg.shared.global [%0], [%1], 16;\n" ::"r"(
+                           (unsigned)__cvta_generic_to_shared(d + 4 * q)),
+                       "l"(row + x)
+                       : "memory");
+        } else {
 #pragma unroll
-        for (int e = 0; e < 4; ++e)
-          asm volatile("cp.async.ca.shared.global [%0], [%1], 4;\n" ::"r"(
-                           (unsigned)__cvta_generic_to_shared(d + 4 * q + e)),
-                       "l"(row + ghost2i(x + e, nx, bc))
+          for (int e = 0; e < 4; ++e)
+            asm volatile("cp.async.ca.shared.global [%0], [%1], 4;\n" ::"r"(
+                             (unsigned)__cvta_generic_to_shared(d + 4 * q + e)),
+                         "l"(row + ghost2i(x + e, nx, bc))
+                         : "memory");
+        }
+      }
+    } else {  // a lane per column
+      for (int q = lane; q < kPS; q += 32) {
+        const int x = bx0 - 4 + q;
+        if (x < nx + 4)
+          asm volatile("cp.async.ca.shared.global [%0], [%1], 4;\n" ::"r"((unsigned)__cvta_generic_to_shared(d + q)),
+                       "l"(row + ghost2i(x, nx, bc))
                        : "memory");
       }
     }
@@ -333,20 +346,31 @@ __global__ void __launch_bounds__(256, TY > 8 ? 2 : 3)
   __syncthreads();
 
   const int x = bx0 + 4 * lane;
-  // four cells of a row of a global plane (the row's padding included)
+  // four cells of a row of a global plane, those that lie in the grid
   auto load4 = [&](const float* p, float (&v)[4]) {
-    const float4 t = x < nx ? *reinterpret_cast<const float4*>(p) : make_float4(0.f, 0.f, 0.f, 0.f);
-    v[0] = t.x, v[1] = t.y, v[2] = t.z, v[3] = t.w;
+    if (VEC) {
+      const float4 t = x < nx ? *reinterpret_cast<const float4*>(p) : make_float4(0.f, 0.f, 0.f, 0.f);
+      v[0] = t.x, v[1] = t.y, v[2] = t.z, v[3] = t.w;
+    } else {
+#pragma unroll
+      for (int e = 0; e < 4; ++e) v[e] = x + e < nx ? p[e] : 0.f;
+    }
   };
   auto store4 = [&](float* p, const float (&v)[4]) {
-    if (x < nx) *reinterpret_cast<float4*>(p) = make_float4(v[0], v[1], v[2], v[3]);
+    if (VEC) {
+      if (x < nx) *reinterpret_cast<float4*>(p) = make_float4(v[0], v[1], v[2], v[3]);
+    } else {
+#pragma unroll
+      for (int e = 0; e < 4; ++e)
+        if (x + e < nx) p[e] = v[e];
+    }
   };
   // first stage of tile row r (-2 .. TY + 1), the lane's four columns; u is requested before the
   // right-hand sides are evaluated
   auto stage1 = [&](int r, float (&rhs)[5][4]) {
     const float* c0 = A + (r + 4) * kPS + 4 + 4 * lane;
     float uv[4][4];
-    const float* ur = u + (int64_t)ghost2i(by0 + r, ny, bc) * pitch;
+    const float* ur = u + (int64_t)ghost2i(by0 + r, ny, bc) * nx;
 #pragma unroll
     for (int c = 0; c < 4; ++c) {
       if (PAIR == 0) {
@@ -381,7 +405,7 @@ __global__ void __launch_bounds__(256, TY > 8 ? 2 : 3)
     const float* c0 = A + (r + 2) * kPS + 4 + col;
     float t[5][1];
     fd4_rhs<ORDER, 1>(c0 - 2 * kPS, c0 - kPS, c0, c0 + kPS, c0 + 2 * kPS, FA, k, t);
-    const int64_t row = (int64_t)ghost2i(by0 + r - 2, ny, bc) * pitch;
+    const int64_t row = (int64_t)ghost2i(by0 + r - 2, ny, bc) * nx;
     const int64_t gx = ghost2i(bx0 + col, nx, bc);
 #pragma unroll
     for (int c = 0; c < 4; ++c)
@@ -413,7 +437,7 @@ __global__ void __launch_bounds__(256, TY > 8 ? 2 : 3)
     if (y >= ny) continue;
     const float* c0 = B + (r + 2) * kPS + 4 + 4 * lane;
     float rhs[5][4];
-    const int64_t o = (int64_t)y * pitch + x;
+    const int64_t o = (int64_t)y * nx + x;
     float ag[5][4], ug[5][4];
     if (PAIR == 1) {  // requested before the right-hand sides
 #pragma unroll
@@ -447,18 +471,13 @@ __global__ void __launch_bounds__(256, TY > 8 ? 2 : 3)
   }
 }
 
-// Rows of nx values, ldb apart, from rows lda apart.
 template <typename A, typename B>
-__global__ void convert_kernel(const A* __restrict__ a, int64_t lda, B* __restrict__ b, int64_t ldb, int64_t nx,
-                               int64_t rows) {
-  for (int64_t y = blockIdx.y; y < rows; y += gridDim.y)
-    for (int64_t x = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; x < nx; x += (int64_t)gridDim.x * blockDim.x)
-      b[y * ldb + x] = (B)a[y * lda + x];
+__global__ void convert_kernel(const A* __restrict__ a, B* __restrict__ b, int64_t n) {
+  for (int64_t t = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; t < n; t += (int64_t)gridDim.x * blockDim.x)
+    b[t] = (B)a[t];
 }
 
-dim3 convert_grid(int64_t nx, int64_t rows) {
-  return dim3((unsigned)((nx + 255) / 256), (unsigned)std::min<int64_t>(65535, rows));
-}
+unsigned blocks1(int64_t n) { return (unsigned)std::min<int64_t>(65536, (n + 255) / 256); }
 
 size_t rup(size_t v) { return (v + 255) / 256 * 256; }
 
@@ -474,11 +493,8 @@ int check_grid(const sslbm_grid* g) {
   return SSLBM_OK;
 }
 
-// Elements from row to row of the state: FP32 rows are padded to whole groups of four cells.
-int64_t row_pitch(const sslbm_grid* g) { return g->precision == SSLBM_FP64 ? g->nx : (g->nx + 3) / 4 * 4; }
-
 size_t state_bytes(const sslbm_grid* g) {
-  return rup((size_t)5 * row_pitch(g) * g->ny * (g->precision == SSLBM_FP64 ? 8 : 4));
+  return rup((size_t)5 * g->nx * g->ny * (g->precision == SSLBM_FP64 ? 8 : 4));
 }
 
 }  // namespace
@@ -494,9 +510,8 @@ struct sslbm_fd4 {
   int64_t steps = 0;
   int order = 4;  // order of the Laplacian: 4 (the reference) or 2
   int sms = 1;    // multiprocessors of the device
-  int cur = 0;    // the state's buffer: 0, or after an odd number of FP32 steps 3
-  void* buf(int i) const { return ws + (size_t)i * sb; }  // FP64: 0 u, 1 t1, 2 t2, 3 acc; FP32: 0 and 3 u, 1 t, 2 acc
-  void* state() const { return buf(cur); }
+  // 0 u, the state; scratch of a step: FP64 1 t1, 2 t2, 3 acc, FP32 1 t, 2 acc, 3 the next state
+  void* buf(int i) const { return ws + (size_t)i * sb; }
 };
 
 namespace {
@@ -512,11 +527,11 @@ struct DevGuard {
   }
 };
 
-template <int PAIR, int ORDER, int TY>
+template <int PAIR, int ORDER, int TY, bool VEC>
 cudaError_t launch_pair(const sslbm_fd4* f, const float* src, const float* u, float* acc, float* dst) {
   // the dynamic shared-memory limit, once per device (a bit per device; setting it twice is harmless)
   static std::atomic<unsigned long long> done{0};
-  auto kern = fd4_pair_kernel<PAIR, ORDER, TY>;
+  auto kern = fd4_pair_kernel<PAIR, ORDER, TY, VEC>;
   if (!(done.load(std::memory_order_acquire) & (1ull << (f->device & 63)))) {
     cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)fd4_pair_smem<TY>());
     if (e != cudaSuccess) return e;
@@ -526,29 +541,46 @@ cudaError_t launch_pair(const sslbm_fd4* f, const float* src, const float* u, fl
   const int64_t ctas = (nx + kPX - 1) / kPX * ((ny + TY - 1) / TY);
   if (ctas > 0x7fffffffLL) return cudaErrorInvalidConfiguration;
   return sslbm::launch_pdl(kern, dim3((unsigned)ctas), dim3(256), fd4_pair_smem<TY>(), f->stream, (int)nx, (int)ny,
-                           (int)row_pitch(&f->g), (int)f->g.bc, f->k32, src, u, acc, dst);
+                           (int)f->g.bc, f->k32, src, u, acc, dst);
 }
 
-// One FP32 step: two launches, the state alternating between its two buffers.
-template <int ORDER, int TY>
-cudaError_t run_step_pairs(sslbm_fd4* f) {
-  float* u = static_cast<float*>(f->state());
+// One FP32 step from u to next: two launches.
+template <int ORDER, int TY, bool VEC>
+cudaError_t run_step_pairs(const sslbm_fd4* f, const float* u, float* next) {
   float* t = static_cast<float*>(f->buf(1));
   float* acc = static_cast<float*>(f->buf(2));
-  float* next = static_cast<float*>(f->buf(3 - f->cur));
-  cudaError_t e = launch_pair<0, ORDER, TY>(f, u, u, acc, t);
-  if (e == cudaSuccess) e = launch_pair<1, ORDER, TY>(f, t, u, acc, next);
-  if (e == cudaSuccess) f->cur = 3 - f->cur;
-  return e;
+  cudaError_t e = launch_pair<0, ORDER, TY, VEC>(f, u, u, acc, t);
+  return e == cudaSuccess ? launch_pair<1, ORDER, TY, VEC>(f, t, u, acc, next) : e;
 }
 
-template <int ORDER>
-cudaError_t run_step_f32(sslbm_fd4* f) {
+template <int ORDER, bool VEC>
+cudaError_t run_step_f32(const sslbm_fd4* f, const float* u, float* next) {
   // 16-row tiles evaluate 1.15 first stages per cell, 8-row tiles 1.28 but give twice the CTAs and
   // three per SM: below three 16-row tiles per SM (us per step, 8 and 16 rows: 400^2 26 and 30,
   // 801 x 700 42 and 49, 1000^2 59 and 59, 2048^2 187 and 176)
   const int64_t tiles = (f->g.nx + kPX - 1) / kPX * ((f->g.ny + 15) / 16);
-  return tiles >= 3 * (int64_t)f->sms ? run_step_pairs<ORDER, 16>(f) : run_step_pairs<ORDER, 8>(f);
+  return tiles >= 3 * (int64_t)f->sms ? run_step_pairs<ORDER, 16, VEC>(f, u, next)
+                                      : run_step_pairs<ORDER, 8, VEC>(f, u, next);
+}
+
+// n FP32 steps: the state alternates between buffers 0 and 3 and ends in buffer 0, by a copy
+// after an odd n, so that every call finds it there and a captured call can be replayed for any n.
+// The copy moves 40 bytes per cell, a step 128.
+template <int ORDER, bool VEC>
+cudaError_t run_steps_f32(sslbm_fd4* f, int64_t n) {
+  float* a = static_cast<float*>(f->buf(0));
+  float* b = static_cast<float*>(f->buf(3));
+  cudaError_t e = cudaSuccess;
+  for (int64_t i = 0; i < n && (e = run_step_f32<ORDER, VEC>(f, a, b)) == cudaSuccess; ++i) {
+    std::swap(a, b);
+    ++f->steps;
+  }
+  if (a != f->buf(0)) {
+    const size_t bytes = (size_t)5 * f->g.nx * f->g.ny * sizeof(float);
+    const cudaError_t ce = cudaMemcpyAsync(b, a, bytes, cudaMemcpyDeviceToDevice, f->stream);
+    if (e == cudaSuccess) e = ce;
+  }
+  return e;
 }
 
 template <typename T, int ORDER>
@@ -653,26 +685,25 @@ int sslbm_fd4_write(sslbm_fd4* f, const void* src, int src_dtype, int src_on_dev
   if (!f || !src) return err(SSLBM_ERR_BAD_ARG, "NULL argument");
   if (src_dtype != SSLBM_DT_F64 && src_dtype != SSLBM_DT_F32) return err(SSLBM_ERR_BAD_ARG, "dtype %d", src_dtype);
   DevGuard dg(f->device);
-  const int64_t nx = f->g.nx, rows = 5 * f->g.ny, pitch = row_pitch(&f->g);
+  const int64_t n = 5 * f->g.nx * f->g.ny;
   const size_t esz = src_dtype == SSLBM_DT_F64 ? 8 : 4;
   const bool f64 = f->g.precision == SSLBM_FP64;
-  f->cur = 0;
   if ((src_dtype == SSLBM_DT_F64) == f64) {
-    CK(cudaMemcpy2DAsync(f->buf(0), pitch * esz, src, nx * esz, nx * esz, rows,
-                         src_on_device ? cudaMemcpyDeviceToDevice : cudaMemcpyHostToDevice, f->stream),
+    CK(cudaMemcpyAsync(f->buf(0), src, (size_t)n * esz,
+                       src_on_device ? cudaMemcpyDeviceToDevice : cudaMemcpyHostToDevice, f->stream),
        "copy");
   } else {
     const void* s = src;
     if (!src_on_device) {  // stage through the scratch buffers (two when FP32 holds FP64)
-      CK(cudaMemcpyAsync(f->buf(1), src, (size_t)(rows * nx) * esz, cudaMemcpyHostToDevice, f->stream), "host -> device");
+      CK(cudaMemcpyAsync(f->buf(1), src, (size_t)n * esz, cudaMemcpyHostToDevice, f->stream), "host -> device");
       s = f->buf(1);
     }
     if (f64)
-      convert_kernel<float, double><<<convert_grid(nx, rows), 256, 0, f->stream>>>(
-          static_cast<const float*>(s), nx, static_cast<double*>(f->buf(0)), pitch, nx, rows);
+      convert_kernel<float, double><<<blocks1(n), 256, 0, f->stream>>>(static_cast<const float*>(s),
+                                                                       static_cast<double*>(f->buf(0)), n);
     else
-      convert_kernel<double, float><<<convert_grid(nx, rows), 256, 0, f->stream>>>(
-          static_cast<const double*>(s), nx, static_cast<float*>(f->buf(0)), pitch, nx, rows);
+      convert_kernel<double, float><<<blocks1(n), 256, 0, f->stream>>>(static_cast<const double*>(s),
+                                                                       static_cast<float*>(f->buf(0)), n);
     CK(cudaGetLastError(), "convert");
   }
   if (!src_on_device) CK(cudaStreamSynchronize(f->stream), "sync");
@@ -684,24 +715,23 @@ int sslbm_fd4_read(sslbm_fd4* f, void* dst, int dst_dtype, int dst_on_device) {
   if (!f || !dst) return err(SSLBM_ERR_BAD_ARG, "NULL argument");
   if (dst_dtype != SSLBM_DT_F64 && dst_dtype != SSLBM_DT_F32) return err(SSLBM_ERR_BAD_ARG, "dtype %d", dst_dtype);
   DevGuard dg(f->device);
-  const int64_t nx = f->g.nx, rows = 5 * f->g.ny, pitch = row_pitch(&f->g);
+  const int64_t n = 5 * f->g.nx * f->g.ny;
   const size_t esz = dst_dtype == SSLBM_DT_F64 ? 8 : 4;
   const bool f64 = f->g.precision == SSLBM_FP64;
   if ((dst_dtype == SSLBM_DT_F64) == f64) {
-    CK(cudaMemcpy2DAsync(dst, nx * esz, f->state(), pitch * esz, nx * esz, rows,
-                         dst_on_device ? cudaMemcpyDeviceToDevice : cudaMemcpyDeviceToHost, f->stream),
+    CK(cudaMemcpyAsync(dst, f->buf(0), (size_t)n * esz, dst_on_device ? cudaMemcpyDeviceToDevice : cudaMemcpyDeviceToHost,
+                       f->stream),
        "copy");
   } else {
     void* d = dst_on_device ? dst : f->buf(1);
     if (f64)
-      convert_kernel<double, float><<<convert_grid(nx, rows), 256, 0, f->stream>>>(
-          static_cast<const double*>(f->state()), pitch, static_cast<float*>(d), nx, nx, rows);
+      convert_kernel<double, float><<<blocks1(n), 256, 0, f->stream>>>(static_cast<const double*>(f->buf(0)),
+                                                                       static_cast<float*>(d), n);
     else
-      convert_kernel<float, double><<<convert_grid(nx, rows), 256, 0, f->stream>>>(
-          static_cast<const float*>(f->state()), pitch, static_cast<double*>(d), nx, nx, rows);
+      convert_kernel<float, double><<<blocks1(n), 256, 0, f->stream>>>(static_cast<const float*>(f->buf(0)),
+                                                                       static_cast<double*>(d), n);
     CK(cudaGetLastError(), "convert");
-    if (!dst_on_device)
-      CK(cudaMemcpyAsync(dst, d, (size_t)(rows * nx) * esz, cudaMemcpyDeviceToHost, f->stream), "device -> host");
+    if (!dst_on_device) CK(cudaMemcpyAsync(dst, d, (size_t)n * esz, cudaMemcpyDeviceToHost, f->stream), "device -> host");
   }
   CK(cudaStreamSynchronize(f->stream), "sync");
   return SSLBM_OK;
@@ -711,12 +741,14 @@ int sslbm_fd4_step(sslbm_fd4* f, int64_t n) {
   if (!f) return err(SSLBM_ERR_BAD_ARG, "NULL handle");
   if (n < 0) return err(SSLBM_ERR_BAD_ARG, "n < 0");
   DevGuard dg(f->device);
+  if (f->g.precision == SSLBM_FP32) {
+    const bool vec = f->g.nx % 4 == 0;
+    const cudaError_t e = f->order == 4 ? (vec ? run_steps_f32<4, true>(f, n) : run_steps_f32<4, false>(f, n))
+                                        : (vec ? run_steps_f32<2, true>(f, n) : run_steps_f32<2, false>(f, n));
+    return e == cudaSuccess ? SSLBM_OK : cuda_err(e, "FD4 stage launch");
+  }
   for (int64_t i = 0; i < n; ++i) {
-    cudaError_t e;
-    if (f->g.precision == SSLBM_FP64)
-      e = f->order == 4 ? run_step<double, 4>(f, f->k64) : run_step<double, 2>(f, f->k64);
-    else
-      e = f->order == 4 ? run_step_f32<4>(f) : run_step_f32<2>(f);
+    cudaError_t e = f->order == 4 ? run_step<double, 4>(f, f->k64) : run_step<double, 2>(f, f->k64);
     if (e != cudaSuccess) return cuda_err(e, "FD4 stage launch");
     ++f->steps;
   }
