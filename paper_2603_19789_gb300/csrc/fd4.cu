@@ -6,16 +6,17 @@
 // with the reactions of Eq. (sources) evaluated at every stage.  Ghost cells: periodic wrap,
 // or (no-flux) the even reflection about the boundary face, u[-1] = u[0], u[-2] = u[1].
 //
-// One step is four stage launches in FP64, two launches of two stages each in FP32.  Stage s reads the previous stage's state with the
-// stencil and writes the next stage's state and the running sum of the slopes:
+// One step is four stage launches in FP64; in FP32 two launches of two stages each, or the four on grids
+// where those are faster (plan_step).  Stage s reads the previous stage's state with the stencil and
+// writes the next stage's state and the running sum of the slopes:
 //   s = 1: acc = k1,         t = u + (dt/2) k1
 //   s = 2: acc = acc + 2 k2, t = u + (dt/2) k2
 //   s = 3: acc = acc + 2 k3, t = u + dt k3
 //   s = 4: u = u + (dt/6) (acc + k4)
 // Every operation is rounded on its own (no contraction) in the order of the formulas
 // above, so the FP64 path reproduces a plain evaluation of them operation by operation.
-// FP64: one cell per thread on 32 x 8 tiles.  FP32: four cells per thread on 128 x 16 tiles, two
-// stages per launch; both evaluate the same expressions.
+// Stage launches: one cell per thread on 32 x 8 tiles.  Pairs: four cells per thread on tiles of 128 x 8
+// or 16; both evaluate the same expressions.
 #include <cuda_runtime.h>
 
 #include <algorithm>
@@ -553,36 +554,7 @@ cudaError_t run_step_pairs(const sslbm_fd4* f, const float* u, float* next) {
   return e == cudaSuccess ? launch_pair<1, ORDER, TY, VEC>(f, t, u, acc, next) : e;
 }
 
-template <int ORDER, bool VEC>
-cudaError_t run_step_f32(const sslbm_fd4* f, const float* u, float* next) {
-  // 16-row tiles evaluate 1.15 first stages per cell, 8-row tiles 1.28 but give twice the CTAs and
-  // three per SM: below three 16-row tiles per SM (us per step, 8 and 16 rows: 400^2 26 and 30,
-  // 801 x 700 42 and 49, 1000^2 59 and 59, 2048^2 187 and 176)
-  const int64_t tiles = (f->g.nx + kPX - 1) / kPX * ((f->g.ny + 15) / 16);
-  return tiles >= 3 * (int64_t)f->sms ? run_step_pairs<ORDER, 16, VEC>(f, u, next)
-                                      : run_step_pairs<ORDER, 8, VEC>(f, u, next);
-}
-
-// n FP32 steps: the state alternates between buffers 0 and 3 and ends in buffer 0, by a copy
-// after an odd n, so that every call finds it there and a captured call can be replayed for any n.
-// The copy moves 40 bytes per cell, a step 128.
-template <int ORDER, bool VEC>
-cudaError_t run_steps_f32(sslbm_fd4* f, int64_t n) {
-  float* a = static_cast<float*>(f->buf(0));
-  float* b = static_cast<float*>(f->buf(3));
-  cudaError_t e = cudaSuccess;
-  for (int64_t i = 0; i < n && (e = run_step_f32<ORDER, VEC>(f, a, b)) == cudaSuccess; ++i) {
-    std::swap(a, b);
-    ++f->steps;
-  }
-  if (a != f->buf(0)) {
-    const size_t bytes = (size_t)5 * f->g.nx * f->g.ny * sizeof(float);
-    const cudaError_t ce = cudaMemcpyAsync(b, a, bytes, cudaMemcpyDeviceToDevice, f->stream);
-    if (e == cudaSuccess) e = ce;
-  }
-  return e;
-}
-
+// One step of four stage launches, in place.
 template <typename T, int ORDER>
 cudaError_t run_step(const sslbm_fd4* f, const Fd4Coeffs<T>& k) {
   const int64_t nx = f->g.nx, ny = f->g.ny;
@@ -598,6 +570,74 @@ cudaError_t run_step(const sslbm_fd4* f, const Fd4Coeffs<T>& k) {
   fd4_stage_kernel<T, 3, ORDER><<<grid, block, 0, f->stream>>>(nx, ny, bc, k, t2, u, acc, t1);
   fd4_stage_kernel<T, 4, ORDER><<<grid, block, 0, f->stream>>>(nx, ny, bc, k, t1, u, acc, u);
   return cudaGetLastError();
+}
+
+// How FP32 steps are launched: the two-stage kernel with 8 or 16 rows per tile, or the four one-cell
+// stage launches; and whether the last of an odd number of steps takes the stage launches, which work
+// in place, rather than a pair and the copy into buffer 0.
+struct StepPlan {
+  int rows;  // 0: stage launches
+  bool odd_in_place;
+};
+
+// By the costs measured (us per step, 40 grids from 32^2 to 2048^2 and 3 x 100000 to 20000 x 3, both
+// boundaries).  A pair step takes whole waves of its tiles, 3 CTAs per SM with 8 rows and 2 with 16:
+// 1000^2 59 and 58, 800 x 600 40 and 34 (two waves and one), 20000 x 64 65 and 76, 2048^2 187 and 177.
+// Grids narrower than a tile waste most of it, where the 32 x 8 stage tiles do not: 64 x 20000 no-flux
+// 152 as pairs and 103 as stages, 3 x 100000 570 and 180, but 96 x 20000 155 and 181.  On small no-flux
+// grids the pairs' mirror passes cost what the launches save, most where a tile spans the domain
+// (64 x 1000 26.8 and 22.9, 20000 x 8 26.2 and 25.0).  The copy after an odd step is worth it only on
+// larger grids: one step at 128^2 31 with it and 22 in place, at 2048^2 206 and 363.
+StepPlan plan_step(const sslbm_grid& g, int sms) {
+  const double cells = (double)g.nx * g.ny, m = 1e-6;
+  const int64_t cols = (g.nx + kPX - 1) / kPX;
+  const bool walls = g.bc != SSLBM_BC_PERIODIC, vec = g.nx % 4 == 0;
+  const int64_t t8 = cols * ((g.ny + 7) / 8), t16 = cols * ((g.ny + 15) / 16);
+  const int64_t w8 = (t8 + 3 * sms - 1) / (3 * sms), w16 = (t16 + 2 * sms - 1) / (2 * sms);
+  const double edge = walls ? 2.5 + (cols == 1 || g.ny <= 8 ? 6.0 : 0.0) : 0.0;
+  double p8, p16;
+  if (w8 == 1) {  // one wave of 8-row tiles is never behind
+    p8 = t8 <= sms ? 18.5 + (vec ? 0.0 : 2.0) : 26.5;
+    p16 = 1e30;
+  } else {
+    p8 = (6.0 + 20.2 * w8) * (vec ? 1.0 : 1.3);
+    p16 = (6.0 + 25.5 * w16) * (vec ? 1.0 : 1.3);
+  }
+  const double pair = (p8 <= p16 ? p8 : p16) + edge;
+  // the stage launches: cells of whole 32 x 8 tiles, slower beyond what L2 holds
+  const double tiles = m * (double)((g.nx + kTX - 1) / kTX * kTX) * (double)((g.ny + kTY - 1) / kTY * kTY);
+  const double stage = 20.0 + (tiles > 0.02 ? 2.5 : 1.0) + 55.0 * std::min(tiles, 1.0) +
+                       85.0 * std::max(tiles - 1.0, 0.0) + (walls ? 0.0 : 3.5);
+  StepPlan plan;
+  plan.rows = pair > stage ? 0 : p8 <= p16 ? 8 : 16;
+  plan.odd_in_place = pair + 7.0 + 6.9 * m * cells > stage;
+  return plan;
+}
+
+// n FP32 steps: pairs alternate between buffers 0 and 3 and the state ends in buffer 0, so that every
+// call finds it there and a captured call can be replayed for any n.
+template <int ORDER, bool VEC>
+cudaError_t run_steps_f32(sslbm_fd4* f, int64_t n) {
+  const StepPlan plan = plan_step(f->g, f->sms);
+  float* a = static_cast<float*>(f->buf(0));
+  float* b = static_cast<float*>(f->buf(3));
+  cudaError_t e = cudaSuccess;
+  for (int64_t i = 0; i < n && e == cudaSuccess; ++i) {
+    const bool last_odd = a == f->buf(0) && i + 1 == n;
+    if (plan.rows == 0 || (last_odd && plan.odd_in_place)) {
+      e = run_step<float, ORDER>(f, f->k32);
+    } else {
+      e = plan.rows == 8 ? run_step_pairs<ORDER, 8, VEC>(f, a, b) : run_step_pairs<ORDER, 16, VEC>(f, a, b);
+      if (e == cudaSuccess) std::swap(a, b);
+    }
+    if (e == cudaSuccess) ++f->steps;
+  }
+  if (a != f->buf(0)) {
+    const size_t bytes = (size_t)5 * f->g.nx * f->g.ny * sizeof(float);
+    const cudaError_t ce = cudaMemcpyAsync(b, a, bytes, cudaMemcpyDeviceToDevice, f->stream);
+    if (e == cudaSuccess) e = ce;
+  }
+  return e;
 }
 
 template <typename T>
