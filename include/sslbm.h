@@ -229,12 +229,20 @@ int sslbm_set_diffusivity_scale(sslbm_handle* h, const void* kx, const void* ky,
  * passes of their own depth, chosen by the grid and n, and the varying diffusion and the SPLIT
  * and KAHAN storages passes of six and eight steps where n allows.  Results do not depend on
  * the depth: every depth performs the same floating-point operations in the same order.
+ * Stream capture: a pass reads one of two state buffers and writes the other, so a captured call that is
+ * replayed advances the state again only if the state is back in the buffer it was captured on.  Calls
+ * of an even number of passes leave it there: n passes where the kernel takes one step each, else
+ * ceil(n / depth) with the depth of sslbm_get_blocking.  Where the default blocking takes passes of its
+ * own depths, a captured call of n >= 2 steps makes an even number of them, and calls between replays as
+ * many as ceil(n / depth), or one more or less but of the same parity.
  * Enqueues on the handle's stream and returns. */
 int sslbm_step(sslbm_handle* h, int64_t n);
 
 /* Advance the BGK state by n >= 0 steps of Eq. (pdf) (collide, then stream along
  * the D2Q5 links; no-flux walls by halfway bounce-back) with D by Eq. (rhoD).  FP32 fuses up
- * to four steps per pass, with the results of one step per pass. */
+ * to four steps per pass, with the results of one step per pass.  Stream capture as for sslbm_step: in
+ * FP32 a captured call of n >= 2 steps can be replayed, and calls between replays leave the state in
+ * the buffer where n passes would; in FP64 a call makes n passes. */
 int bgk_step(sslbm_handle* h, int64_t n);
 
 /* Steps taken by a scheme since its last full write. */

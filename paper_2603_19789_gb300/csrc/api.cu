@@ -158,6 +158,7 @@ struct sslbm_handle {
   bool auto_blocking = true;  // the default blocking, or an autotuned choice of the tile passes
   int seg_cache[SSLBM_MAX_DEPTH + 1] = {0};
   int last_pass = 0;  // depth of the call's last pass, 0 before the first and after a tile pass
+  bool s_captured = false, b_captured = false;  // a step call of the scheme has been captured (pass_plan.cuh)
   bool fuse_diag = false;   // sslbm_set_fused_diagnostics
   bool diag_ready = false;  // diag_result() holds the diagnostics of the current SSLBM state
 
@@ -222,6 +223,16 @@ static bool kernel_access(const sslbm_handle* h, const void* p, size_t size) {
 // The compartments with a compensation plane: the first n.
 static int comp_planes(const sslbm_handle* h) {
   return ten_planes(h) ? 5 : h->g.precision == SSLBM_FP32_SPLIT ? 1 : 0;
+}
+
+// Whether what is enqueued on the handle's stream now is being captured into a graph.
+static bool capturing(const sslbm_handle* h) {
+  cudaStreamCaptureStatus s = cudaStreamCaptureStatusNone;
+  if (cudaStreamIsCapturing(h->stream, &s) != cudaSuccess) {
+    cudaGetLastError();
+    return false;
+  }
+  return s == cudaStreamCaptureStatusActive;
 }
 
 // The D2Q5 FP32 storages and the FP32 D2Q9 and varying-diffusion lattices have the
@@ -592,35 +603,32 @@ int sslbm_step(sslbm_handle* h, int64_t n) {
   if (h->g.lattice == SSLBM_LATTICE_D2Q5_VARD && !h->kappa_ok)
     return fail(SSLBM_ERR_BAD_ARG, "the diffusivity scale fields are not set (sslbm_set_diffusivity_scale)");
   const bool blocked = can_block(h);
-  bool tiles = blocked && h->auto_blocking && !h->fuse_diag;
-  // under the default blocking, the depth of most passes (a tuned or set blocking has depth or segment of its own)
-  const int deep =
-      tiles && h->depth > 1 && h->seg_rows == 0 ? sslbm::default_pass_depth(h->g.lattice, h->g.precision) : h->depth;
+  // under the default blocking, passes of this call's own choosing: the depth of most pipeline passes (a
+  // tuned or set blocking has depth or segment of its own), and the register tiles of small grids
+  const bool own_cut = blocked && h->auto_blocking && !h->fuse_diag;
+  const int deep = own_cut && h->depth > 1 && h->seg_rows == 0
+                       ? sslbm::default_pass_depth(h->g.lattice, h->g.precision)
+                       : h->depth;
+  const bool captured = n > 0 && capturing(h);
+  int parity = own_cut ? sslbm::pass_parity(n, h->depth, captured, h->s_captured) : sslbm::kAnyParity;
+  h->s_captured |= captured;
+  sslbm::TilePlan plan{0, 0};
+  const bool tiles = own_cut && n > 1 && sslbm::tile_plan(h->g.lattice, h->g.precision, h->gv, n, parity, &plan);
+  if (!tiles && deep == h->depth) parity = sslbm::kAnyParity;  // the plain cut
+  int64_t tile_passes = tiles ? sslbm::pass_count(n, plan.depth, parity) : 0;
   if (n > 0) h->diag_ready = false;
   h->last_pass = 0;
   while (n > 0) {
-    int k = 1;
     cudaError_t e;
-    if (tiles && n > 1) {
-      // a small grid under the default blocking: register-tile passes, their depths differing by at
-      // most one as below
-      sslbm::TilePlan plan{0, 0};
-      if (sslbm::tile_plan(h->g.lattice, h->g.precision, h->gv, n, &plan)) {
-        const int64_t passes = (n + plan.depth - 1) / plan.depth;
-        k = (int)((n + passes - 1) / passes);
-        e = launch_tile_pass(h, plan.nr, k);
-        if (e != cudaSuccess) return cuda_fail(e, "SSLBM step launch");
-        h->s_cur = 1 - h->s_cur;
-        h->s_steps += k;
-        n -= k;
-        continue;
-      }
-      tiles = false;
-    }
-    if (blocked && h->depth > 1 && n > 1) {
-      // depth >= 2: the temporal-blocked kernel; a single step uses the one-step kernel,
-      // which produces the same bits.
-      k = sslbm::next_pass_depth(n, h->depth, deep);
+    // a single step uses the one-step kernel, which produces the same bits
+    const int k = tiles                             ? (int)((n + tile_passes - 1) / tile_passes)
+                  : blocked && h->depth > 1 && n > 1 ? sslbm::next_pass_depth(n, h->depth, deep, parity)
+                                                     : 1;
+    --tile_passes;
+    parity = sslbm::flip_parity(parity);
+    if (k > 1 && tiles) {
+      e = launch_tile_pass(h, plan.nr, k);
+    } else if (k > 1) {
       int seg = h->seg_rows;
       if (seg <= 0) {
         if (!h->seg_cache[k]) h->seg_cache[k] = default_seg(h, k);
@@ -654,14 +662,14 @@ int bgk_step(sslbm_handle* h, int64_t n) {
   if (st) return st;
   if (n < 0) return fail(SSLBM_ERR_BAD_ARG, "n=%lld < 0", (long long)n);
   DeviceGuard dg(h->device);
+  // FP32: passes of up to kBgkDepth steps, their depths differing by at most one; FP64, whose
+  // arithmetic rate bounds it, and a single step: one step per launch
+  const bool fuse = h->g.precision == SSLBM_FP32 && n > 0, captured = fuse && capturing(h);
+  int64_t passes = fuse ? sslbm::pass_count(n, sslbm::kBgkDepth, sslbm::pass_parity(n, 1, captured, h->b_captured)) : n;
+  h->b_captured |= captured;
   while (n > 0) {
-    // FP32: passes of up to kBgkDepth steps, their depths differing by at most one; FP64, whose
-    // arithmetic rate bounds it, and a single step: one step per launch
-    int64_t k = 1;
-    if (h->g.precision == SSLBM_FP32 && n > 1) {
-      const int64_t passes = (n + sslbm::kBgkDepth - 1) / sslbm::kBgkDepth;
-      k = (n + passes - 1) / passes;
-    }
+    const int64_t k = (n + passes - 1) / passes;
+    --passes;
     cudaError_t e = k > 1 ? sslbm::launch_bgk_tile(h->gv, &h->cf, h->b_buf[h->b_cur], h->b_buf[1 - h->b_cur], (int)k,
                                                    h->stream)
                           : sslbm::launch_bgk_step(h->g.precision, h->gv, h->coeffs(), h->b_buf[h->b_cur],
@@ -966,7 +974,7 @@ int sslbm_autotune(sslbm_handle* h, double budget_ms, int* depth_out, int* seg_o
     cand.push_back({1, 0});
     if (can_block(h)) {
       sslbm::TilePlan plan{0, 0};
-      if (sslbm::tile_plan(h->g.lattice, h->g.precision, h->gv, 1000, &plan)) cand.push_back({plan.depth, -plan.nr});
+      if (sslbm::tile_plan(h->g.lattice, h->g.precision, h->gv, 1000, sslbm::kAnyParity, &plan)) cand.push_back({plan.depth, -plan.nr});
       for (int d = 2; d <= SSLBM_MAX_DEPTH; ++d) {
         const int base = default_seg(h, d);
         int segs[3] = {base, base / 2, base * 2};

@@ -308,7 +308,7 @@ int sm_count() {
 // The lines, in us per step of 24 (tile, pipeline): D2Q5 430 x 5304 9.2 and 8.7, 1300 x 1000 5.0
 // and 5.8; varying diffusion 1300 x 1000 8.4 and 8.2; D2Q9 walls 2048^2 27.6 and 31.4, 3000 x 2200
 // 43.7 and 37.1.
-bool tile_plan(int lattice, int precision, const GridView& g, int64_t n, TilePlan* plan) {
+bool tile_plan(int lattice, int precision, const GridView& g, int64_t n, int parity, TilePlan* plan) {
   const bool d2q5 = lattice == SSLBM_LATTICE_D2Q5 && (precision == SSLBM_FP32 || precision == SSLBM_FP32_DEV);
   const bool other = (lattice == SSLBM_LATTICE_D2Q9 || lattice == SSLBM_LATTICE_D2Q5_VARD) && precision == SSLBM_FP32;
   // beyond 32 cells per column and SM the pipeline is ahead whatever the estimate's error
@@ -321,7 +321,7 @@ bool tile_plan(int lattice, int precision, const GridView& g, int64_t n, TilePla
     for (int k = 2; k <= n && 2 * k < rows && k < 29; ++k) {
       const int ke = (k + 1) & ~1;
       const double ctas = std::ceil((double)g.nx / (kTCols - 2 * ke)) * std::ceil((double)g.ny / (rows - 2 * k));
-      const int64_t passes = (n + k - 1) / k;  // of equal depth, as sslbm_step cuts them
+      const int64_t passes = pass_count(n, k, parity);  // of equal depth, as sslbm_step cuts them
       const double t = std::ceil(ctas / sms) * (c.fix[i] * passes + c.step[i] * n) / n;
       if (t < best) {
         best = t;
@@ -334,7 +334,7 @@ bool tile_plan(int lattice, int precision, const GridView& g, int64_t n, TilePla
   const int m = (int)std::min<int64_t>(n, 48), deep = default_pass_depth(lattice, precision);
   double us[SSLBM_MAX_DEPTH + 1] = {0.0}, pipe = 0.0;
   for (int left = m; left > 0;) {
-    const int k = next_pass_depth(left, 4, deep);
+    const int k = next_pass_depth(left, 4, deep, kAnyParity);
     if (us[k] == 0.0) {
       const double res = sms * (16 / k), strips = std::ceil((double)g.nx / (128 - 8 * ((k + 3) / 4)));
       const double segs = std::max(1.0, std::floor((&c == &kCostD2q9Walls ? 2 : 1) * res / strips));

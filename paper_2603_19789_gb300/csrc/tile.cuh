@@ -1,5 +1,6 @@
 // tile.cuh -- the register-tile pass of small grids (tile.cu).
 #pragma once
+#include "pass_plan.cuh"
 #include "sslbm_internal.cuh"
 
 namespace sslbm {
@@ -19,21 +20,11 @@ inline int default_pass_depth(int lattice, int precision) {
   return lattice == SSLBM_LATTICE_D2Q5 && (precision == SSLBM_FP32_SPLIT || precision == SSLBM_FP32_KAHAN) ? 8 : 4;
 }
 
-// Depth of the next of the pipeline passes that cover n steps: passes deeper than depth are taken
-// whole, where they leave at least three steps or none; else ceil(n / depth) passes whose depths
-// differ by at most one (100 steps at depth 7: 10 of 7 and 5 of 6), rather than full passes and a
-// shallow remainder, which runs at a lower rate per step.
-inline int next_pass_depth(int64_t n, int depth, int deep) {
-  if (deep > depth && (n == deep || n >= deep + 3)) return deep;
-  const int64_t passes = (n + depth - 1) / depth;
-  return (int)((n + passes - 1) / passes);
-}
-
-// The tile passes' rows per warp and depth for n further steps of this grid, or false where the
-// row pipeline is expected to be faster (or the update has no tile pass).
+// The tile passes' rows per warp and depth for n steps of this grid, or false where the row pipeline is
+// expected to be faster (or the update has no tile pass).  parity: of the number of passes.
 struct TilePlan {
   int nr, depth;
 };
-bool tile_plan(int lattice, int precision, const GridView& g, int64_t n, TilePlan* plan);
+bool tile_plan(int lattice, int precision, const GridView& g, int64_t n, int parity, TilePlan* plan);
 
 }  // namespace sslbm
