@@ -427,12 +427,12 @@ int sslbm_write(sslbm_handle* h, int scheme, int comp, const void* src, int src_
   const int own_dtype = h->g.precision == SSLBM_FP64 ? SSLBM_DT_F64 : SSLBM_DT_F32;
   const int n_comp = comp_planes(h);
   const int dev_S = h->g.precision == SSLBM_FP32_DEV ? 1 : 0;
-  if (!bgk && src_on_device && kernel_access(h, src, usize)) {  // every plane in one launch
+  if (!bgk && comp == SSLBM_ALL && src_on_device && kernel_access(h, src, usize)) {  // every plane in one launch
     cudaError_t e = sslbm::launch_planes_write(h->g.precision, h->gv, src, src_dtype, h->s_plane(h->s_cur, c0),
                                                n_comp ? h->s_plane(h->s_cur, 5 + c0) : nullptr, n_comp, c0, c1 - c0,
                                                dev_S, h->p.s_ref, h->stream);
     if (e != cudaSuccess) return cuda_fail(e, "write kernel");
-    if (comp == SSLBM_ALL) h->s_steps = 0;
+    h->s_steps = 0;
     return SSLBM_OK;
   }
   for (int c = c0; c < c1; ++c) {
@@ -542,7 +542,7 @@ int sslbm_read(sslbm_handle* h, int scheme, int comp, void* dst, int dst_dtype, 
   const int own_dtype = h->g.precision == SSLBM_FP64 ? SSLBM_DT_F64 : SSLBM_DT_F32;
   const int n_comp = comp_planes(h);
   const int dev_S = h->g.precision == SSLBM_FP32_DEV ? 1 : 0;
-  if (!bgk && dst_on_device && kernel_access(h, dst, usize)) {  // every plane in one launch
+  if (!bgk && comp == SSLBM_ALL && dst_on_device && kernel_access(h, dst, usize)) {  // every plane in one launch
     cudaError_t e = sslbm::launch_planes_read(h->g.precision, h->gv, h->s_plane(h->s_cur, c0),
                                               n_comp ? h->s_plane(h->s_cur, 5 + c0) : nullptr, n_comp, c0, c1 - c0,
                                               dev_S, h->p.s_ref, dst, dst_dtype, h->stream);

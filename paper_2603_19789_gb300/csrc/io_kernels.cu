@@ -22,115 +22,136 @@ namespace {
 // stored as given are copied.
 // Bound by HBM on large grids and by the launch on small ones: a launch per plane (or a strided
 // copy per plane) cost an ensemble of 32 scenarios 957 us to write and 1232 to read, now 186 and 524;
-// the strided device copies of an 8192^2 state took 1.33 ms each way, this 0.39.
+// the strided device copies of an 8192^2 state took 1.33 ms each way, this 0.39.  Conversions are bound
+// by the FP64 pipe; 3786 x 4055, us, the earlier launch per plane and this: double to Kahan 718 and 554,
+// FP64 to float 339 and 162, one plane of deviations to double 70 and 60; 64 x 20000, Kahan to double 72
+// and 38.
 // vec: nx is a multiple of 4 and the caller's planes are 16-byte aligned, so a thread moves four
-// cells at a time; else cells 128 apart, so that a warp's accesses stay contiguous.
-template <typename T>
-struct Vec4 {
-  T v[4];
+// cells at a time; else single cells.  A CTA is bx columns (cells or groups of four) by blockDim.x / bx
+// rows, so that narrow grids keep its lanes busy; on large grids a thread has the loads of four such
+// rows in flight before it stores the first, on small ones the FP64 arithmetic of the compensated
+// storages is spread over more and smaller CTAs.
+template <int N, typename T>
+__device__ __forceinline__ void ld_cells(T (&r)[N], const T* p) {
+  if constexpr (N == 1) {
+    r[0] = *p;
+  } else if constexpr (sizeof(T) == 4) {
+    *reinterpret_cast<float4*>(r) = *reinterpret_cast<const float4*>(p);
+  } else {
+    *reinterpret_cast<double2*>(r) = *reinterpret_cast<const double2*>(p);
+    *reinterpret_cast<double2*>(r + 2) = *reinterpret_cast<const double2*>(p + 2);
+  }
+}
+template <int N, typename T>
+__device__ __forceinline__ void st_cells(T* p, const T (&r)[N]) {
+  if constexpr (N == 1) {
+    *p = r[0];
+  } else if constexpr (sizeof(T) == 4) {
+    *reinterpret_cast<float4*>(p) = *reinterpret_cast<const float4*>(r);
+  } else {
+    *reinterpret_cast<double2*>(p) = *reinterpret_cast<const double2*>(r);
+    *reinterpret_cast<double2*>(p + 2) = *reinterpret_cast<const double2*>(r + 2);
+  }
+}
+
+constexpr int kIoThreads = 256;
+
+// What a stored value is: the value, value - compensation, or s_ref - the value.  Each kind is a loop of
+// its own, so that values stored as given see no FP64 arithmetic, of which this GPU has little.
+enum { IO_PLAIN, IO_COMP, IO_DEV };
+
+template <typename T, typename U, int N>
+struct IoCells {
+  alignas(16) T hi[N], lo[N];
+  alignas(16) U v[N];
 };
-template <typename T>
-__device__ __forceinline__ Vec4<T> ld_vec(const T* p) {
-  Vec4<T> r;
-  if constexpr (sizeof(T) == 4) {
-    *reinterpret_cast<float4*>(r.v) = *reinterpret_cast<const float4*>(p);
-  } else {
-    *reinterpret_cast<double2*>(r.v) = *reinterpret_cast<const double2*>(p);
-    *reinterpret_cast<double2*>(r.v + 2) = *reinterpret_cast<const double2*>(p + 2);
-  }
-  return r;
-}
-template <typename T>
-__device__ __forceinline__ void st_vec(T* p, const Vec4<T>& r) {
-  if constexpr (sizeof(T) == 4) {
-    *reinterpret_cast<float4*>(p) = *reinterpret_cast<const float4*>(r.v);
-  } else {
-    *reinterpret_cast<double2*>(p) = *reinterpret_cast<const double2*>(r.v);
-    *reinterpret_cast<double2*>(p + 2) = *reinterpret_cast<const double2*>(r.v + 2);
+
+template <typename T, typename U, bool WRITE, int KIND, int N, int ROWS>
+__device__ __forceinline__ void io_rows(const GridView& g, U* up, T* pp, T* cp, const double s_ref, const int bx) {
+  const int64_t x = (int64_t)N * ((int64_t)blockIdx.x * bx + ((int)threadIdx.x & (bx - 1)));
+  if (x >= g.nx) return;
+  const int by = (int)blockDim.x / bx;
+  for (int64_t y0 = (int64_t)blockIdx.y * ROWS * by + (int)threadIdx.x / bx; y0 < g.ny;
+       y0 += (int64_t)gridDim.y * ROWS * by) {
+    IoCells<T, U, N> q[ROWS];
+#pragma unroll
+    for (int r = 0; r < ROWS; ++r) {
+      const int64_t y = y0 + r * by;
+      if (y >= g.ny) continue;
+      if (WRITE) {
+        ld_cells<N>(q[r].v, up + y * g.nx + x);
+      } else {
+        ld_cells<N>(q[r].hi, pp + y * g.pitch + x);
+        if (KIND == IO_COMP) ld_cells<N>(q[r].lo, cp + y * g.pitch + x);
+      }
+    }
+#pragma unroll
+    for (int r = 0; r < ROWS; ++r) {
+      const int64_t y = y0 + r * by;
+      if (y >= g.ny) continue;
+#pragma unroll
+      for (int e = 0; e < N; ++e) {
+        if (WRITE) {
+          if (KIND == IO_PLAIN) {
+            q[r].hi[e] = (T)q[r].v[e];
+          } else {
+            const double v = KIND == IO_DEV ? s_ref - (double)q[r].v[e] : (double)q[r].v[e];
+            q[r].hi[e] = (T)v;
+            if (KIND == IO_COMP) q[r].lo[e] = (T)((double)q[r].hi[e] - v);
+          }
+        } else if (KIND == IO_PLAIN) {
+          q[r].v[e] = (U)q[r].hi[e];
+        } else {
+          q[r].v[e] = (U)(KIND == IO_DEV ? s_ref - (double)q[r].hi[e] : (double)q[r].hi[e] - (double)q[r].lo[e]);
+        }
+      }
+      if (WRITE) {
+        st_cells<N>(pp + y * g.pitch + x, q[r].hi);
+        if (KIND == IO_COMP) st_cells<N>(cp + y * g.pitch + x, q[r].lo);
+      } else {
+        st_cells<N>(up + y * g.nx + x, q[r].v);
+      }
+    }
   }
 }
 
-constexpr int kIoThreads = 128;
-
-template <typename T, typename U, bool WRITE>
+template <typename T, typename U, bool WRITE, int N, int ROWS>
 __global__ void __launch_bounds__(kIoThreads) planes_io_kernel(const GridView g, U* user, T* planes, T* comps,
                                                                const int n_comp, const int c0, const int dev_S,
-                                                               const double s_ref, const int vec) {
+                                                               const double s_ref, const int bx) {
   pdl_enter();
   const int c = c0 + (int)blockIdx.z;
   U* up = user + (int64_t)blockIdx.z * g.nx * g.ny;
   T* pp = planes + (int64_t)blockIdx.z * g.plane;
-  T* cp = comps != nullptr && c < n_comp ? comps + (int64_t)blockIdx.z * g.plane : nullptr;
-  const bool dev = dev_S && c == 0;
-  const bool plain = cp == nullptr && !dev;
-  auto put = [&](U a, T& hi, T& lo) {
-    if (plain) {
-      hi = (T)a;
-    } else {
-      double v = (double)a;
-      if (dev) v = s_ref - v;
-      hi = (T)v;
-      lo = (T)((double)hi - v);
-    }
-  };
-  auto get = [&](T hi, T lo) {
-    if (plain) return (U)hi;
-    double v = (double)hi;
-    if (cp) v -= (double)lo;
-    if (dev) v = s_ref - v;
-    return (U)v;
-  };
-  const int64_t xb = (int64_t)blockIdx.x * 4 * kIoThreads;
-  for (int64_t y = blockIdx.y; y < g.ny; y += gridDim.y) {
-    U* ur = up + y * g.nx;
-    T* pr = pp + y * g.pitch;
-    T* cr = cp + (cp ? y * g.pitch : 0);
-    if (vec) {
-      const int64_t x = xb + 4 * threadIdx.x;
-      if (x >= g.nx) continue;
-      if (WRITE) {
-        const Vec4<U> a = ld_vec(ur + x);
-        Vec4<T> hi, lo;
-#pragma unroll
-        for (int e = 0; e < 4; ++e) put(a.v[e], hi.v[e], lo.v[e]);
-        st_vec(pr + x, hi);
-        if (cp) st_vec(cr + x, lo);
-      } else {
-        const Vec4<T> hi = ld_vec(pr + x);
-        Vec4<T> lo = hi;
-        if (cp) lo = ld_vec(cr + x);
-        Vec4<U> a;
-#pragma unroll
-        for (int e = 0; e < 4; ++e) a.v[e] = get(hi.v[e], lo.v[e]);
-        st_vec(ur + x, a);
-      }
-    } else {
-#pragma unroll
-      for (int e = 0; e < 4; ++e) {
-        const int64_t x = xb + threadIdx.x + e * kIoThreads;
-        if (x >= g.nx) break;
-        if (WRITE) {
-          T hi, lo;
-          put(ur[x], hi, lo);
-          pr[x] = hi;
-          if (cp) cr[x] = lo;
-        } else {
-          const T hi = pr[x];
-          ur[x] = get(hi, cp ? cr[x] : hi);
-        }
-      }
-    }
-  }
+  if (comps != nullptr && c < n_comp)
+    io_rows<T, U, WRITE, IO_COMP, N, ROWS>(g, up, pp, comps + (int64_t)blockIdx.z * g.plane, s_ref, bx);
+  else if (dev_S && c == 0)
+    io_rows<T, U, WRITE, IO_DEV, N, ROWS>(g, up, pp, nullptr, s_ref, bx);
+  else
+    io_rows<T, U, WRITE, IO_PLAIN, N, ROWS>(g, up, pp, nullptr, s_ref, bx);
 }
 
 template <typename T, typename U, bool WRITE>
 cudaError_t planes_io_t(const GridView& g, void* user, void* planes, void* comps, int n_comp, int c0, int nplanes,
                         int dev_S, double s_ref, cudaStream_t s) {
-  const dim3 grid((unsigned)((g.nx + 4 * kIoThreads - 1) / (4 * kIoThreads)), (unsigned)(g.ny < 4096 ? g.ny : 4096),
-                  (unsigned)nplanes);
-  const int vec = g.nx % 4 == 0 && reinterpret_cast<uintptr_t>(user) % 16 == 0;
-  return launch_pdl(planes_io_kernel<T, U, WRITE>, grid, dim3(kIoThreads), 0, s, g, static_cast<U*>(user),
-                    static_cast<T*>(planes), static_cast<T*>(comps), n_comp, c0, dev_S, s_ref, vec);
+  const bool vec = g.nx % 4 == 0 && reinterpret_cast<uintptr_t>(user) % 16 == 0;
+  const int64_t cols = vec ? g.nx / 4 : g.nx;
+  // threads per CTA, columns (a power of two) and rows per thread: the largest CTAs of which there are
+  // enough for the GPU
+  int threads = 0, rows = 0, bx = 0;
+  int64_t gx = 0, gy = 0;
+  for (int t = 0; t < 3; ++t) {
+    threads = t < 2 ? kIoThreads : 64, rows = t == 0 ? 4 : 1;
+    for (bx = 8; bx < threads && bx < cols;) bx *= 2;
+    gx = (cols + bx - 1) / bx;
+    gy = (g.ny + (int64_t)rows * (threads / bx) - 1) / ((int64_t)rows * (threads / bx));
+    if (gx * gy * nplanes >= 1024) break;
+  }
+  const dim3 grid((unsigned)gx, (unsigned)(gy < 65535 ? gy : 65535), (unsigned)nplanes);
+  auto kern = vec ? (rows == 4 ? planes_io_kernel<T, U, WRITE, 4, 4> : planes_io_kernel<T, U, WRITE, 4, 1>)
+                  : (rows == 4 ? planes_io_kernel<T, U, WRITE, 1, 4> : planes_io_kernel<T, U, WRITE, 1, 1>);
+  return launch_pdl(kern, grid, dim3(threads), 0, s, g, static_cast<U*>(user), static_cast<T*>(planes),
+                    static_cast<T*>(comps), n_comp, c0, dev_S, s_ref, bx);
 }
 
 template <bool WRITE>
