@@ -162,13 +162,17 @@ __device__ __forceinline__ void diag_total(const double* __restrict__ partials, 
   }
 }
 
-// Blocks of a reduction over ny rows, at least four rows each: a block's FP64 reduction costs as much
-// as the sums of about four rows (a block per row: 533 us for an ensemble of 32 scenarios, now 186).  The
-// same for a grid alone and in an ensemble, so that both add in the same order.
-inline int64_t diag_blocks(int64_t ny) {
-  const int64_t b = (ny + 3) / 4;
+// Blocks of the reduction of a grid that an ensemble may hold (FP32, deviation and split storages): a
+// block's FP64 reduction costs as much as the sums of about 4096 cells, so a block takes up to four
+// rows, but no more than that many cells (a block per row: 533 us for an ensemble of 32 scenarios, now
+// 186; four rows each on 12000 x 300: 64 us, with a row each 42).  The same for a grid alone and in an
+// ensemble, so that both add in the same order.  FP64 and the compensated storages, whose cells
+// cost more, take a block per row.
+__host__ __device__ inline int64_t diag_blocks(int64_t nx, int64_t ny) {
+  const int64_t rows = nx >= 4096 ? 1 : nx >= 2048 ? 2 : 4, b = (ny + rows - 1) / rows;
   return b < 1 ? 1 : b < kDiagBlocks ? b : kDiagBlocks;
 }
+__host__ __device__ inline int64_t diag_blocks_by_row(int64_t ny) { return ny < kDiagBlocks ? ny : kDiagBlocks; }
 
 }  // namespace
 }  // namespace sslbm

@@ -49,8 +49,6 @@ struct EnsScenario {
   Coeffs<float> k;
   int64_t off;  // element offset of the scenario's planes in each buffer
   int nstrips, seg_rows, tiles, tile_base;
-  int64_t diag_base;  // first diagnostics partial
-  int diag_blocks;
 };
 
 struct EnsControl {
@@ -142,24 +140,27 @@ __global__ void __launch_bounds__(32 * K, 16 / K)
 
 // Diagnostics of the scenarios i0 + blockIdx.y, all in one launch: partials, the blocks of a scenario
 // as launch_diagnostics cuts them (so the totals are those of the grid alone, bit for bit), and their
-// totals (NCOMP = 1: plane 5 compensates S).  A reduction and a total per scenario, as before, took
-// 986 us for 32 scenarios of 256^2 to 1024^2, now 186.
+// totals (NCOMP = 1: plane 5 compensates S).  The partials (48 bytes per block, at most one per row of
+// 32 floats or more) lie in the scenario's planes of the spare buffer, which holds nothing between
+// calls.  A reduction and a total per scenario, as before, took 986 us for 32 scenarios of 256^2 to
+// 1024^2, now 186.
 template <int NCOMP>
 __global__ void __launch_bounds__(256) ens_diag_kernel(const EnsScenario* __restrict__ tab, const int i0,
-                                                       const float* __restrict__ buf, double* __restrict__ partials) {
+                                                       const float* __restrict__ buf, float* __restrict__ spare) {
   const EnsScenario& sc = tab[i0 + blockIdx.y];
-  if ((int)blockIdx.x >= sc.diag_blocks) return;
   const GridView g = sc.g;
+  const int blocks = (int)sslbm::diag_blocks(g.nx, g.ny);
+  if ((int)blockIdx.x >= blocks) return;
   const float* st = buf + sc.off;
-  sslbm::diag_rows_f32x4<0, NCOMP>(g, st, NCOMP ? st + 5 * g.plane : nullptr, (int)blockIdx.x, sc.diag_blocks,
-                                   partials + (sc.diag_base + blockIdx.x) * sslbm::kDiagSlots);
+  sslbm::diag_rows_f32x4<0, NCOMP>(g, st, NCOMP ? st + 5 * g.plane : nullptr, (int)blockIdx.x, blocks,
+                                   reinterpret_cast<double*>(spare + sc.off) + blockIdx.x * sslbm::kDiagSlots);
 }
 
 __global__ void __launch_bounds__(256) ens_diag_final_kernel(const EnsScenario* __restrict__ tab, const int i0,
-                                                             const double* __restrict__ partials,
+                                                             const float* __restrict__ spare,
                                                              double* __restrict__ results) {
   const int i = i0 + (int)blockIdx.x;
-  sslbm::diag_total(partials + tab[i].diag_base * sslbm::kDiagSlots, tab[i].diag_blocks,
+  sslbm::diag_total(reinterpret_cast<const double*>(spare + tab[i].off), (int)sslbm::diag_blocks(tab[i].g.nx, tab[i].g.ny),
                     results + (size_t)i * sslbm::kDiagSlots);
 }
 
@@ -202,7 +203,7 @@ constexpr size_t kAlign = 256;
 size_t round_up(size_t v, size_t a) { return (v + a - 1) / a * a; }
 
 struct EnsLayout {
-  size_t off_ctl, off_done, off_tab, off_partials, off_results, off_buf[2], total;
+  size_t off_ctl, off_done, off_tab, off_results, off_buf[2], total;
   std::vector<int64_t> pitch, plane, elem_off;
   int64_t buf_elems;
 };
@@ -229,10 +230,6 @@ int make_layout(int n, const sslbm_scenario* sc, int precision, EnsLayout* L) {
   off += round_up((size_t)n * sizeof(unsigned), kAlign);
   L->off_tab = off;
   off += round_up((size_t)n * sizeof(EnsScenario), kAlign);
-  L->off_partials = off;
-  int64_t blocks = 0;
-  for (int i = 0; i < n; ++i) blocks += sslbm::diag_blocks(sc[i].ny);
-  off += round_up((size_t)blocks * sslbm::kDiagSlots * sizeof(double), kAlign);
   L->off_results = off;
   off += round_up((size_t)n * sslbm::kDiagSlots * sizeof(double), kAlign);
   for (int b = 0; b < 2; ++b) {
@@ -303,7 +300,6 @@ namespace {
 int upload_table(sslbm_ensemble* e) {
   e->tab.resize(e->n);
   int base = 0;
-  int64_t diag_base = 0;
   for (int i = 0; i < e->n; ++i) {
     const sslbm_scenario& s = e->sc[i];
     EnsScenario& t = e->tab[i];
@@ -327,9 +323,6 @@ int upload_table(sslbm_ensemble* e) {
     t.tiles = t.nstrips * nsegs;
     t.tile_base = base;
     base += t.tiles;
-    t.diag_base = diag_base;
-    t.diag_blocks = (int)sslbm::diag_blocks(s.ny);
-    diag_base += t.diag_blocks;
   }
   e->total_tiles = base;
   cudaError_t ce = cudaMemcpyAsync(e->dtab(), e->tab.data(), sizeof(EnsScenario) * e->n,
@@ -629,17 +622,17 @@ int sslbm_ensemble_run(sslbm_ensemble* e, int64_t nsteps) {
 int sslbm_ensemble_diagnostics(sslbm_ensemble* e, double* totals, double* peak_I) {
   if (!e) return err(SSLBM_ERR_BAD_ARG, "ensemble is NULL");
   DevGuard dg(e->device);
-  double* partials = reinterpret_cast<double*>(e->ws + e->L.off_partials);
+  float* spare = e->buf(1 - e->cur);
   double* results = reinterpret_cast<double*>(e->ws + e->L.off_results);
   int most = 1;
-  for (const EnsScenario& t : e->tab) most = std::max(most, t.diag_blocks);
+  for (const sslbm_scenario& s : e->sc) most = std::max(most, (int)sslbm::diag_blocks(s.nx, s.ny));
   for (int i0 = 0; i0 < e->n; i0 += 65535) {  // a grid's limit in y
     const int nb = std::min(e->n - i0, 65535);
     if (e->precision == SSLBM_FP32_SPLIT)
-      ens_diag_kernel<1><<<dim3(most, nb), 256, 0, e->stream>>>(e->dtab(), i0, e->buf(e->cur), partials);
+      ens_diag_kernel<1><<<dim3(most, nb), 256, 0, e->stream>>>(e->dtab(), i0, e->buf(e->cur), spare);
     else
-      ens_diag_kernel<0><<<dim3(most, nb), 256, 0, e->stream>>>(e->dtab(), i0, e->buf(e->cur), partials);
-    ens_diag_final_kernel<<<nb, 256, 0, e->stream>>>(e->dtab(), i0, partials, results);
+      ens_diag_kernel<0><<<dim3(most, nb), 256, 0, e->stream>>>(e->dtab(), i0, e->buf(e->cur), spare);
+    ens_diag_final_kernel<<<nb, 256, 0, e->stream>>>(e->dtab(), i0, spare, results);
     cudaError_t ce = cudaGetLastError();
     if (ce != cudaSuccess) return cuda_err(ce, "diagnostics");
   }

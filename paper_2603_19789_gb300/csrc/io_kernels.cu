@@ -238,7 +238,8 @@ cudaError_t launch_diagnostics(int precision, int layout, const GridView& g, con
                                cudaStream_t s, int n_comp) {
   if (!comp_planes) n_comp = 0;
   if (n_comp != 0 && n_comp != 1 && n_comp != 5) return cudaErrorInvalidValue;
-  const int64_t blocks = diag_blocks(g.ny);
+  const int64_t blocks =
+      precision == SSLBM_FP64 || layout == 1 || n_comp == 5 ? diag_blocks_by_row(g.ny) : diag_blocks(g.nx, g.ny);
   if (precision == SSLBM_FP64) {
     if (layout == 0)
       diag_partial_kernel<double, 0><<<(unsigned)blocks, 256, 0, s>>>(
