@@ -467,6 +467,36 @@ __device__ __forceinline__ void two_sum_add(float& hi, float& lo, float x) {
   hi = s;
 }
 
+// A thread's sum: a TwoSum pair, renormalised by its owner every few values so that its low part keeps
+// FP32's unit roundoff squared, and beside it in FP64 what the pair cannot hold exactly -- terms that could
+// overflow it, infinities and NaN, and squares whose rounding error would underflow.
+struct PairSum {
+  float hi = 0.f, lo = 0.f;
+  double wide = 0.0;
+  __device__ __forceinline__ void add(float v) {
+    if (fabsf(v) <= 0x1p100f)
+      two_sum_add(hi, lo, v);
+    else
+      wide += (double)v;
+  }
+  __device__ __forceinline__ void add_square(float v) {
+    const float a = fabsf(v);
+    if (a <= 0x1p50f && (a >= 0x1p-50f || a == 0.f)) {
+      const float sq = __fmul_rn(v, v);
+      two_sum_add(hi, lo, sq);
+      lo = __fadd_rn(lo, __fmaf_rn(v, v, -sq));
+    } else {
+      wide += (double)v * (double)v;
+    }
+  }
+  __device__ __forceinline__ void renormalise() {
+    const float t = __fadd_rn(hi, lo), bp = __fsub_rn(t, hi);
+    lo = __fadd_rn(__fsub_rn(hi, __fsub_rn(t, bp)), __fsub_rn(lo, bp));
+    hi = t;
+  }
+  __device__ __forceinline__ double total() const { return ((double)hi + (double)lo) + wide; }
+};
+
 // per sample b = blockIdx.y: sums[3b] += sum (y - t), sums[3b+1] += sum t, sums[3b+2] += sum max(-y, 0).
 // Bound by its 8 bytes per value: every value added in FP64 took 84 us at B = 16, 256 x 256 (42 MB);
 // 21 us
@@ -475,12 +505,13 @@ __global__ void loss_sums_kernel(const float* __restrict__ y, const float* __res
                                  double* __restrict__ sums, int64_t P5) {
   __shared__ double sh[64];
   const int64_t b = blockIdx.y;
-  float eh = 0.f, el = 0.f, th = 0.f, tl = 0.f, nh = 0.f, nl = 0.f;
+  PairSum se, st, sn;
   auto take = [&](float yv, float tv) {
-    two_sum_add(eh, el, yv - tv);
-    two_sum_add(th, tl, tv);
-    if (yv < 0.f) two_sum_add(nh, nl, -yv);
+    se.add(yv - tv);
+    st.add(tv);
+    if (yv < 0.f) sn.add(-yv);
   };
+  auto renormalise = [&]() { se.renormalise(), st.renormalise(), sn.renormalise(); };
   const float* yb = y + b * P5;
   const float* tb = tgt + b * P5;
   const int64_t stride = (int64_t)gridDim.x * blockDim.x, i0 = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
@@ -488,13 +519,14 @@ __global__ void loss_sums_kernel(const float* __restrict__ y, const float* __res
     for (int64_t i = i0; i < P5 / 4; i += stride) {
       const float4 yv = reinterpret_cast<const float4*>(yb)[i], tv = reinterpret_cast<const float4*>(tb)[i];
       take(yv.x, tv.x), take(yv.y, tv.y), take(yv.z, tv.z), take(yv.w, tv.w);
+      renormalise();
     }
   } else {
-    for (int64_t i = i0; i < P5; i += stride) take(yb[i], tb[i]);
+    for (int64_t i = i0; i < P5; i += stride) take(yb[i], tb[i]), renormalise();
   }
-  block_add2((double)eh + (double)el, (double)th + (double)tl, sums + 3 * b, sh);
+  block_add2(se.total(), st.total(), sums + 3 * b, sh);
   __syncthreads();
-  block_add1((double)nh + (double)nl, sums + 3 * b + 2, sh);
+  block_add1(sn.total(), sums + 3 * b + 2, sh);
 }
 
 // The training loss (N = B * 5 * P):
@@ -519,7 +551,7 @@ __global__ void loss_kernel(const float* __restrict__ y, const float* __restrict
   }
   __syncthreads();
   const float gm = gsh[0], gn = gsh[1];
-  float hi = 0.f, lo = 0.f;
+  PairSum sum;
   const int64_t stride = (int64_t)gridDim.x * blockDim.x, i0 = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
   for (int c = 0; c < 5; ++c) {
     const float rs = (c == 1 || c == 2) ? rsg : 1.f;
@@ -528,9 +560,7 @@ __global__ void loss_kernel(const float* __restrict__ y, const float* __restrict
     float* db = dy + (b * 5 + c) * P;
     auto one = [&](float yv, float tv) {
       const float dn = (yv - tv) * rs;
-      const float sq = __fmul_rn(dn, dn);
-      two_sum_add(hi, lo, sq);
-      lo = __fadd_rn(lo, __fmaf_rn(dn, dn, -sq));
+      sum.add_square(dn);
       float g = 2.f * dn * rs * inv + gm;
       if (yv < 0.f) g -= gn;
       return g;
@@ -540,12 +570,13 @@ __global__ void loss_kernel(const float* __restrict__ y, const float* __restrict
       for (int64_t i = i0; i < P / 4; i += stride) {
         const float4 yv = reinterpret_cast<const float4*>(yb)[i], tv = reinterpret_cast<const float4*>(tb)[i];
         reinterpret_cast<float4*>(db)[i] = make_float4(one(yv.x, tv.x), one(yv.y, tv.y), one(yv.z, tv.z), one(yv.w, tv.w));
+        sum.renormalise();
       }
     } else {
-      for (int64_t i = i0; i < P; i += stride) db[i] = one(yb[i], tb[i]);
+      for (int64_t i = i0; i < P; i += stride) db[i] = one(yb[i], tb[i]), sum.renormalise();
     }
   }
-  block_add1(((double)hi + (double)lo) / (double)N, loss, sh);
+  block_add1(sum.total() / (double)N, loss, sh);
 }
 
 // Adam (decoupled weight decay), then refresh the BF16 copy used as GEMM operand
