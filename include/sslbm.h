@@ -232,9 +232,9 @@ int sslbm_set_diffusivity_scale(sslbm_handle* h, const void* kx, const void* ky,
  * Stream capture: a pass reads one of two state buffers and writes the other, so a captured call that is
  * replayed advances the state again only if the state is back in the buffer it was captured on.  Calls
  * of an even number of passes leave it there: n passes where the kernel takes one step each, else
- * ceil(n / depth) with the depth of sslbm_get_blocking.  Where the default blocking takes passes of its
- * own depths, a captured call of n >= 2 steps makes an even number of them, and calls between replays as
- * many as ceil(n / depth), or one more or less but of the same parity.
+ * ceil(n / depth) with the depth of sslbm_get_blocking.  Under the default blocking of a kernel that takes
+ * several steps a captured call of n >= 2 makes an even number of passes, and later calls a number of
+ * the parity of ceil(n / depth).
  * Enqueues on the handle's stream and returns. */
 int sslbm_step(sslbm_handle* h, int64_t n);
 

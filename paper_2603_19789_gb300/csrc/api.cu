@@ -606,15 +606,15 @@ int sslbm_step(sslbm_handle* h, int64_t n) {
   // under the default blocking, passes of this call's own choosing: the depth of most pipeline passes (a
   // tuned or set blocking has depth or segment of its own), and the register tiles of small grids
   const bool own_cut = blocked && h->auto_blocking && !h->fuse_diag;
-  const int deep = own_cut && h->depth > 1 && h->seg_rows == 0
-                       ? sslbm::default_pass_depth(h->g.lattice, h->g.precision)
-                       : h->depth;
+  const sslbm::PassCost* cost = own_cut ? sslbm::pass_cost(h->g.lattice, h->g.precision, h->g.bc) : nullptr;
+  const int sms = cost ? sslbm::sm_count() : 1;
+  const int pipe_depth = cost ? sslbm::default_pass_depth(*cost, h->g.nx, h->g.ny, sms) : h->depth;
+  const int deep = h->depth > 1 && h->seg_rows == 0 ? pipe_depth : h->depth;
   const bool captured = n > 0 && capturing(h);
   int parity = own_cut ? sslbm::pass_parity(n, h->depth, captured, h->s_captured) : sslbm::kAnyParity;
   h->s_captured |= captured;
   sslbm::TilePlan plan{0, 0};
-  const bool tiles = own_cut && n > 1 && sslbm::tile_plan(h->g.lattice, h->g.precision, h->gv, n, parity, &plan);
-  if (!tiles && deep == h->depth) parity = sslbm::kAnyParity;  // the plain cut
+  const bool tiles = cost && sslbm::tile_plan(*cost, h->g.nx, h->g.ny, n, pipe_depth, parity, sms, &plan);
   int64_t tile_passes = tiles ? sslbm::pass_count(n, plan.depth, parity) : 0;
   if (n > 0) h->diag_ready = false;
   h->last_pass = 0;
@@ -974,7 +974,11 @@ int sslbm_autotune(sslbm_handle* h, double budget_ms, int* depth_out, int* seg_o
     cand.push_back({1, 0});
     if (can_block(h)) {
       sslbm::TilePlan plan{0, 0};
-      if (sslbm::tile_plan(h->g.lattice, h->g.precision, h->gv, 1000, sslbm::kAnyParity, &plan)) cand.push_back({plan.depth, -plan.nr});
+      const sslbm::PassCost* cost = sslbm::pass_cost(h->g.lattice, h->g.precision, h->g.bc);
+      const int sms = sslbm::sm_count();
+      if (cost && sslbm::tile_plan(*cost, h->g.nx, h->g.ny, 1000,
+                                   sslbm::default_pass_depth(*cost, h->g.nx, h->g.ny, sms), sslbm::kAnyParity, sms, &plan))
+        cand.push_back({plan.depth, -plan.nr});
       for (int d = 2; d <= SSLBM_MAX_DEPTH; ++d) {
         const int base = default_seg(h, d);
         int segs[3] = {base, base / 2, base * 2};

@@ -9,6 +9,7 @@
 
 #include "bounds.cuh"
 #include "sslbm_internal.cuh"
+#include "pass_plan.cuh"
 #include "pdl.cuh"
 #include "sslbm_pipe.cuh"
 
@@ -23,6 +24,12 @@ constexpr size_t pipe_smem_bytes() {
   return sizeof(PipeSmem<K, mode_planes<MODE>()>) + (MODE == MODE_VARD ? sizeof(float) * kRingK * 2 * 128 : 0) +
          (DIAG ? sizeof(DiagSmem<mode_planes<MODE>()>) : 0);
 }
+// the planner's CTAs per SM follow from the same bytes
+static_assert(pipe_smem_bytes<MODE_VARD, 6>() == pipe_bytes(5, 6, true) &&
+                  pipe_smem_bytes<MODE_SPLIT, 8>() == pipe_bytes(6, 8, false) &&
+                  pipe_smem_bytes<MODE_KAHAN, 4>() == pipe_bytes(10, 4, false) &&
+                  pipe_smem_bytes<MODE_PLAIN, 3>() == pipe_bytes(5, 3, false),
+              "pass_plan.cuh: pipe_bytes");
 
 // kx, ky: the scale planes of the varying-diffusion lattice (MODE_VARD), else unused.
 // DIAG: also the diagnostics partial of the CTA's output cells into diag[6 blockIdx.x ...].

@@ -20,9 +20,7 @@
 // is resident and has its indices ready when the current one ends.
 #include <cuda_runtime.h>
 
-#include <algorithm>
 #include <atomic>
-#include <cmath>
 
 #include "bounds.cuh"
 #include "pdl.cuh"
@@ -34,8 +32,8 @@ SSLBM_OOB_ACCESSOR(tile)
 namespace sslbm {
 namespace {
 
-constexpr int kTW = 16;    // warps per CTA
-constexpr int kTCols = 64;  // region columns
+constexpr int kTW = kTileWarps;     // warps per CTA
+constexpr int kTCols = kTileCols;  // region columns
 
 // planes with neighbours: the exchanged ones
 constexpr int kTX = 4;
@@ -277,16 +275,7 @@ cudaError_t launch_nr(const GridView& g, const void* coeffs, const void* in, voi
   }
 }
 
-// Measured on a GB300 (us): one wave of tile passes takes fix + depth * step, by rows per warp; a
-// pass of the row pipeline takes pass + waves * iterations * (it + it_warp * warps per SM).
-struct TileCost {
-  double fix[3], step[3];  // 1, 2, 4 rows per warp
-  double pass, it, it_warp;
-};
-constexpr TileCost kCostD2q5{{2.1, 3.5, 4.5}, {0.38, 0.44, 0.77}, 6.4, 0.43, 0.053};
-constexpr TileCost kCostD2q9{{2.1, 3.5, 4.5}, {0.40, 0.50, 1.05}, 5.9, 0.54, 0.068};
-constexpr TileCost kCostD2q9Walls{{2.1, 2.8, 4.0}, {0.47, 0.85, 1.90}, 18.9, 0.21, 0.134};
-constexpr TileCost kCostVard{{2.1, 2.8, 4.3}, {0.42, 0.80, 1.90}, 7.25, 0.65, 0.083};
+}  // namespace
 
 int sm_count() {
   static std::atomic<int> cache[64];
@@ -296,56 +285,6 @@ int sm_count() {
   if (!v && cudaDeviceGetAttribute(&v, cudaDevAttrMultiProcessorCount, dev) == cudaSuccess)
     cache[dev & 63].store(v, std::memory_order_relaxed);
   return v > 0 ? v : 1;
-}
-
-}  // namespace
-
-// The cheaper of the two by the measured costs: tile passes recompute their halo but need no
-// pipeline fill, so they win where a pipeline would have only short segments to stream.  At the
-// shapes measured (14 grids from 128^2 to 4096^2, 12000 x 300 and 430 x 5304 among them, 2 to 24
-// steps) the side it picks is 0.3% slower on average than the faster one: at most 9% for D2Q5 (1300
-// x 1000, 2 steps: 8.2 and 8.9 us per step), 14% D2Q9, 7% with walls, 3% the varying diffusion.
-// The lines, in us per step of 24 (tile, pipeline): D2Q5 430 x 5304 9.2 and 8.7, 1300 x 1000 5.0
-// and 5.8; varying diffusion 1300 x 1000 8.4 and 8.2; D2Q9 walls 2048^2 27.6 and 31.4, 3000 x 2200
-// 43.7 and 37.1.
-bool tile_plan(int lattice, int precision, const GridView& g, int64_t n, int parity, TilePlan* plan) {
-  const bool d2q5 = lattice == SSLBM_LATTICE_D2Q5 && (precision == SSLBM_FP32 || precision == SSLBM_FP32_DEV);
-  const bool other = (lattice == SSLBM_LATTICE_D2Q9 || lattice == SSLBM_LATTICE_D2Q5_VARD) && precision == SSLBM_FP32;
-  // beyond 32 cells per column and SM the pipeline is ahead whatever the estimate's error
-  if ((!d2q5 && !other) || n < 2 || g.nx > (1 << 22) || g.ny > (1 << 22) || g.nx * g.ny > (int64_t)1 << 24) return false;
-  const TileCost& c = d2q5 ? kCostD2q5 : lattice == SSLBM_LATTICE_D2Q5_VARD ? kCostVard : g.bc == 0 ? kCostD2q9 : kCostD2q9Walls;
-  const double sms = sm_count();
-  double best = 1e300;
-  for (int i = 0; i < 3; ++i) {
-    const int nr = 1 << i, rows = kTW * nr;
-    for (int k = 2; k <= n && 2 * k < rows && k < 29; ++k) {
-      const int ke = (k + 1) & ~1;
-      const double ctas = std::ceil((double)g.nx / (kTCols - 2 * ke)) * std::ceil((double)g.ny / (rows - 2 * k));
-      const int64_t passes = pass_count(n, k, parity);  // of equal depth, as sslbm_step cuts them
-      const double t = std::ceil(ctas / sms) * (c.fix[i] * passes + c.step[i] * n) / n;
-      if (t < best) {
-        best = t;
-        *plan = TilePlan{nr, k};
-      }
-    }
-  }
-  // the pipeline's passes as sslbm_step cuts n steps (beyond 48 the pattern repeats): as many row
-  // segments as its automatic length makes
-  const int m = (int)std::min<int64_t>(n, 48), deep = default_pass_depth(lattice, precision);
-  double us[SSLBM_MAX_DEPTH + 1] = {0.0}, pipe = 0.0;
-  for (int left = m; left > 0;) {
-    const int k = next_pass_depth(left, 4, deep, kAnyParity);
-    if (us[k] == 0.0) {
-      const double res = sms * (16 / k), strips = std::ceil((double)g.nx / (128 - 8 * ((k + 3) / 4)));
-      const double segs = std::max(1.0, std::floor((&c == &kCostD2q9Walls ? 2 : 1) * res / strips));
-      const double rows = std::max(4.0 * k, std::ceil(g.ny / segs)), ctas = strips * std::ceil(g.ny / rows);
-      us[k] = c.pass + std::ceil(ctas / res) * (std::floor((rows + 4 * k - 3) / 2) + 1) *
-                           (c.it + c.it_warp * k * std::min((double)(16 / k), ctas / sms));
-    }
-    pipe += us[k] / m;
-    left -= k;
-  }
-  return best <= pipe;
 }
 
 cudaError_t launch_tile(int lattice, int precision, const GridView& g, const void* coeffs, const void* in, void* out,
