@@ -620,13 +620,14 @@ int sslbm_step(sslbm_handle* h, int64_t n) {
   h->last_pass = 0;
   while (n > 0) {
     cudaError_t e;
-    // a single step uses the one-step kernel, which produces the same bits
+    // a single step uses the one-step kernel, which produces the same bits (between tile passes, a tile
+    // pass of one: 800 x 600, three steps 12.4 us with the one-step kernel, 10.9)
     const int k = tiles                             ? (int)((n + tile_passes - 1) / tile_passes)
                   : blocked && h->depth > 1 && n > 1 ? sslbm::next_pass_depth(n, h->depth, deep, parity)
                                                      : 1;
     --tile_passes;
     parity = sslbm::flip_parity(parity);
-    if (k > 1 && tiles) {
+    if (tiles) {
       e = launch_tile_pass(h, plan.nr, k);
     } else if (k > 1) {
       int seg = h->seg_rows;

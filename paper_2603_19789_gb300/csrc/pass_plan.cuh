@@ -66,18 +66,19 @@ constexpr int pipe_ctas_per_sm(size_t bytes, int K) {
 // (1, 2, 4; no tile pass: 0).
 struct PassCost {
   int planes;      // of the pipeline's rows
-  bool whole;      // the fullest SM's CTAs count, not the average
+  bool whole;      // fitted with the CTAs that fit an SM, and those of the fullest SM; else 16 / K and the average
   int segments;    // row segments in units of what fits at once
   int deep;        // a default depth beside 4, or 4
   double pass, it, it_warp;
+  double shallow[2];  // factors of passes of two and three steps
   double fix[3], step[3];
 };
-constexpr PassCost kCostD2q5{5, false, 1, 4, 6.4, 0.43, 0.053, {2.1, 3.5, 4.5}, {0.38, 0.44, 0.77}};
-constexpr PassCost kCostD2q9{5, false, 1, 4, 5.9, 0.54, 0.068, {2.1, 3.5, 4.5}, {0.40, 0.50, 1.05}};
-constexpr PassCost kCostD2q9Walls{5, false, 2, 4, 18.9, 0.21, 0.134, {2.1, 2.8, 4.0}, {0.47, 0.85, 1.90}};
-constexpr PassCost kCostVard{5, true, 1, 6, 4.0, 0.64, 0.068, {2.1, 2.8, 4.3}, {0.42, 0.80, 1.90}};
-constexpr PassCost kCostSplit{6, true, 1, 8, 4.0, 0.52, 0.061, {0, 0, 0}, {0, 0, 0}};
-constexpr PassCost kCostKahan{10, true, 1, 8, 4.0, 0.70, 0.117, {0, 0, 0}, {0, 0, 0}};
+constexpr PassCost kCostD2q5{5, false, 1, 4, 6.4, 0.43, 0.053, {1.15, 1.0}, {2.1, 3.5, 4.5}, {0.38, 0.44, 0.77}};
+constexpr PassCost kCostD2q9{5, false, 1, 4, 5.9, 0.54, 0.068, {1.15, 1.0}, {2.1, 3.5, 4.5}, {0.40, 0.50, 1.05}};
+constexpr PassCost kCostD2q9Walls{5, false, 2, 4, 18.9, 0.21, 0.134, {1.1, 1.0}, {2.1, 2.8, 4.0}, {0.47, 0.85, 1.90}};
+constexpr PassCost kCostVard{5, true, 1, 6, 4.1, 0.66, 0.070, {1.3, 1.25}, {2.1, 2.8, 4.3}, {0.42, 0.80, 1.90}};
+constexpr PassCost kCostSplit{6, true, 1, 8, 4.0, 0.52, 0.061, {1.0, 1.0}, {0, 0, 0}, {0, 0, 0}};
+constexpr PassCost kCostKahan{10, true, 1, 8, 4.0, 0.70, 0.117, {1.0, 1.0}, {0, 0, 0}, {0, 0, 0}};
 
 inline const PassCost* pass_cost(int lattice, int precision, int bc) {
   if (lattice == SSLBM_LATTICE_D2Q5 && (precision == SSLBM_FP32 || precision == SSLBM_FP32_DEV)) return &kCostD2q5;
@@ -91,12 +92,13 @@ inline const PassCost* pass_cost(int lattice, int precision, int bc) {
 
 // A pipeline pass of depth k at its automatic segments.
 inline double pipe_pass_us(const PassCost& c, int64_t nx, int64_t ny, int k, int sms) {
-  const int per = pipe_ctas_per_sm(pipe_bytes(c.planes, k, &c == &kCostVard), k);
+  const int per = c.whole ? pipe_ctas_per_sm(pipe_bytes(c.planes, k, &c == &kCostVard), k) : 16 / k;
   const double res = (double)sms * per, strips = std::ceil((double)nx / (128 - 8 * ((k + 3) / 4)));
   const double segs = std::max(1.0, std::floor(c.segments * res / strips));
   const double rows = std::max(4.0 * k, std::ceil((double)ny / segs)), ctas = strips * std::ceil((double)ny / rows);
   const double load = std::min((double)per, c.whole ? std::ceil(ctas / sms) : ctas / sms);
-  return c.pass + std::ceil(ctas / res) * (std::floor((rows + 4 * k - 3) / 2) + 1) * (c.it + c.it_warp * k * load);
+  const double us = c.pass + std::ceil(ctas / res) * (std::floor((rows + 4 * k - 3) / 2) + 1) * (c.it + c.it_warp * k * load);
+  return k < 4 ? us * c.shallow[k - 2] : us;
 }
 
 // Depth of the pipeline passes that the default blocking takes where n allows: 4, or the update's deeper
@@ -117,6 +119,9 @@ constexpr int kTileCols = 64, kTileWarps = 16;  // a register tile's columns and
 // (passes of `deep` steps and the rest of up to 4) is expected to be faster or the update has no tile
 // pass: tile passes recompute their halo but need no pipeline fill, so they win where a pipeline would
 // have only short segments to stream.  parity: of the number of passes.
+// Of the choices measured (10 grids from 200^2 to 2048^2, 12000 x 300 and 430 x 5304, 2 to 20 steps) the one it
+// picks is 1.3% slower on average than the fastest for D2Q5, 0.8% D2Q9, 0.4% with walls, 2.3% the
+// varying diffusion; at most 19% (1500 x 1100 D2Q5, two steps).
 // The lines, in us per step of 24 (tile, pipeline): D2Q5 430 x 5304 9.2 and 8.7, 1300 x 1000 5.0 and
 // 5.8; D2Q9 walls 2048^2 27.6 and 31.4, 3000 x 2200 43.7 and 37.1.
 struct TilePlan {
