@@ -76,7 +76,7 @@ struct PassCost {
 constexpr PassCost kCostD2q5{5, false, 1, 4, 6.4, 0.43, 0.053, {1.15, 1.0}, {2.1, 3.5, 4.5}, {0.38, 0.44, 0.77}};
 constexpr PassCost kCostD2q9{5, false, 1, 4, 5.9, 0.54, 0.068, {1.15, 1.0}, {2.1, 3.5, 4.5}, {0.40, 0.50, 1.05}};
 constexpr PassCost kCostD2q9Walls{5, false, 2, 4, 18.9, 0.21, 0.134, {1.1, 1.0}, {2.1, 2.8, 4.0}, {0.47, 0.85, 1.90}};
-constexpr PassCost kCostVard{5, true, 1, 6, 4.1, 0.66, 0.070, {1.3, 1.25}, {2.1, 2.8, 4.3}, {0.42, 0.80, 1.90}};
+constexpr PassCost kCostVard{5, true, 1, 6, 4.1, 0.66, 0.070, {1.3, 1.25}, {2.1, 2.8, 6.0}, {0.42, 0.80, 1.55}};
 constexpr PassCost kCostSplit{6, true, 1, 8, 4.0, 0.52, 0.061, {1.0, 1.0}, {0, 0, 0}, {0, 0, 0}};
 constexpr PassCost kCostKahan{10, true, 1, 8, 4.0, 0.70, 0.117, {1.0, 1.0}, {0, 0, 0}, {0, 0, 0}};
 
@@ -120,7 +120,7 @@ constexpr int kTileCols = 64, kTileWarps = 16;  // a register tile's columns and
 // pass: tile passes recompute their halo but need no pipeline fill, so they win where a pipeline would
 // have only short segments to stream.  parity: of the number of passes.
 // Of the choices measured (10 grids from 200^2 to 2048^2, 12000 x 300 and 430 x 5304, 2 to 20 steps) the one it
-// picks is 1.3% slower on average than the fastest for D2Q5, 0.8% D2Q9, 0.4% with walls, 2.3% the
+// picks is 1.3% slower on average than the fastest for D2Q5, 0.8% D2Q9, 0.4% with walls, 0.8% the
 // varying diffusion; at most 19% (1500 x 1100 D2Q5, two steps).
 // The lines, in us per step of 24 (tile, pipeline): D2Q5 430 x 5304 9.2 and 8.7, 1300 x 1000 5.0 and
 // 5.8; D2Q9 walls 2048^2 27.6 and 31.4, 3000 x 2200 43.7 and 37.1.

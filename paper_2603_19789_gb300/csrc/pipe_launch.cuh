@@ -93,6 +93,14 @@ cudaError_t launch_blocked_t(const GridView& g, const void* coeffs, const void* 
   const int64_t blocks = nstrips * nseg;
   if (blocks > 0x7fffffffLL) return cudaErrorInvalidConfiguration;
   if (DIAG && (blocks > kDiagBlocks || diag == nullptr)) return cudaErrorInvalidConfiguration;
+  // A dependent launch lets the next pass's CTAs in beside this one's.  Where this one is on most SMs and
+  // leaves room, they settle two to an SM beside emptier ones, and stay so from pass to pass.  us per step
+  // of 40, dependent and ordinary: split 4096 x 100 at depth 8 (148 CTAs of 304 that fit) 5.3 and 4.4, FP32
+  // 800 x 600 at depth 4 (266 of 608) 4.7 and 4.2, split there (266 of 456) 5.5 and 5.2; but FP32 350^2 (66) 3.5
+  // and 3.9, 1500 x 1100 (598 of 608) 6.5 and 6.9.
+  const int sms = sm_count();
+  constexpr int64_t per = pipe_ctas_per_sm(pipe_smem_bytes<MODE, K, DIAG>(), K);
+  if (4 * blocks > 3 * sms && 10 * blocks < 9 * per * sms) chained = false;
   return launch_pdl_if(chained, pipe_kernel<MODE, K, DIAG>, dim3((unsigned)blocks), dim3(32 * K),
                        pipe_smem_bytes<MODE, K, DIAG>(), s, g, *static_cast<const Coeffs<float>*>(coeffs),
                        static_cast<const float*>(in), static_cast<float*>(out), seg_rows, (int)nstrips,

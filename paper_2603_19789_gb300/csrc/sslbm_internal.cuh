@@ -285,6 +285,9 @@ __device__ __forceinline__ void seird_cell2(const Coeffs<float>& k, float2 x0, f
   nD = fma2(splat2(k.ddt), I, D);
 }
 
+// Multiprocessors of the current device (at least 1).
+int sm_count();
+
 // ---- launchers (defined in the kernel translation units) --------------------------
 // SSLBM: one step per launch (every precision) and K fused steps per launch (FP32, FP32
 // deviation-S, FP32 split-S and FP32 Kahan).  seg_rows > 0 is the blocked kernel's row-segment

@@ -10,7 +10,4 @@ namespace sslbm {
 cudaError_t launch_tile(int lattice, int precision, const GridView& g, const void* coeffs, const void* in, void* out,
                         const void* kx, const void* ky, int nr, int K, cudaStream_t s);
 
-// Multiprocessors of the current device (at least 1).
-int sm_count();
-
 }  // namespace sslbm
