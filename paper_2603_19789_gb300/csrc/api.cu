@@ -667,6 +667,7 @@ int bgk_step(sslbm_handle* h, int64_t n) {
   // arithmetic rate bounds it, and a single step: one step per launch
   const bool fuse = h->g.precision == SSLBM_FP32 && n > 0, captured = fuse && capturing(h);
   int64_t passes = fuse ? sslbm::pass_count(n, sslbm::kBgkDepth, sslbm::pass_parity(n, 1, captured, h->b_captured)) : n;
+  if (fuse && n == 2 && passes == 1 && !sslbm::bgk_pair_pays(h->gv)) passes = 2;
   h->b_captured |= captured;
   while (n > 0) {
     const int64_t k = (n + passes - 1) / passes;

@@ -16,8 +16,6 @@
 // and 2.3; two steps 72.9 at 2048^2, three 58.3, six 57.1.
 #include <cuda_runtime.h>
 
-#include <atomic>
-
 #include "bounds.cuh"
 #include "pdl.cuh"
 #include "sslbm_internal.cuh"
@@ -168,23 +166,27 @@ cudaError_t launch_t(const GridView& g, const void* coeffs, const void* f_in, vo
 
 }  // namespace
 
+namespace {
+
+// regions of 2 NW rows that cover the grid with K steps per pass
+int64_t regions(const GridView& g, int K, int nw) {
+  const int ke = (K + 1) & ~1;
+  return (g.nx + kBCols - 2 * ke - 1) / (kBCols - 2 * ke) * ((g.ny + 2 * nw - 2 * K - 1) / (2 * nw - 2 * K));
+}
+
+}  // namespace
+
 cudaError_t launch_bgk_tile(const GridView& g, const void* coeffs, const void* f_in, void* f_out, int K, cudaStream_t s) {
   // regions of 16 rows (two CTAs per SM) while they make at most one wave, else of 32, whose halo is
   // relatively smaller: four steps per pass, us per step with 16 and 32 rows: 200^2 2.3 and 3.0,
   // 501 x 377 4.3 and 3.2, 2048^2 58.8 and 57.1, 4096^2 229 and 221
-  static std::atomic<int> sms_of[64];
-  int dev = 0;
-  cudaError_t e = cudaGetDevice(&dev);
-  if (e != cudaSuccess) return e;
-  int sms = sms_of[dev & 63].load(std::memory_order_relaxed);
-  if (!sms) {
-    if ((e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev)) != cudaSuccess) return e;
-    sms_of[dev & 63].store(sms, std::memory_order_relaxed);
-  }
-  const int ke = (K + 1) & ~1;
-  const int64_t small = (g.nx + kBCols - 2 * ke - 1) / (kBCols - 2 * ke) * ((g.ny + 15 - 2 * K) / (16 - 2 * K));
-  return small <= 2 * (int64_t)sms ? launch_t<8>(g, coeffs, f_in, f_out, K, s)
-                                   : launch_t<16>(g, coeffs, f_in, f_out, K, s);
+  return regions(g, K, 8) <= 2 * (int64_t)sm_count() ? launch_t<8>(g, coeffs, f_in, f_out, K, s)
+                                                     : launch_t<16>(g, coeffs, f_in, f_out, K, s);
+}
+
+bool bgk_pair_pays(const GridView& g) {
+  const int64_t sms = sm_count(), waves = (regions(g, 2, 16) + sms - 1) / sms;
+  return regions(g, 2, 8) <= 2 * sms || 8.6 * (double)waves < 2 * 168 / 5.6e6 * (double)g.nx * (double)g.ny;
 }
 
 }  // namespace sslbm

@@ -336,6 +336,10 @@ cudaError_t launch_bgk_step(int precision, const GridView& g, const void* coeffs
 constexpr int kBgkDepth = 4;
 cudaError_t launch_bgk_tile(const GridView& g, const void* coeffs, const void* f_in, void* f_out, int K,
                             cudaStream_t s);
+// Whether two steps are one such pass rather than two launches of one: a wave of its regions takes 8.6 us,
+// a step by itself 168 bytes per cell at 5.6 TB/s.  64 x 20000, whose regions are half outside the grid, 84 us
+// as a pass and 78 as two steps; 2048^2 162 and 213.
+bool bgk_pair_pays(const GridView& g);
 cudaError_t launch_bgk_init(int precision, const GridView& g, int comp, const void* rho,
                             int rho_dtype, void* f, cudaStream_t s);
 cudaError_t launch_bgk_density(int precision, const GridView& g, int comp, const void* f, void* rho,
