@@ -1422,9 +1422,10 @@ int sslbm_fno_make_input(sslbm_fno* f, int batch, const float* u, const float* r
   DevGuard dg(f->device);
   int* smax = f->at<int>(f->bu.smax);
   CK(cudaMemsetAsync(smax, 0, (size_t)batch * 4, f->stream), "zero scale");
-  // few blocks per sample: each thread has several loads in flight (64 blocks: 27 us
-  // at 64 x 256^2, 8 blocks: 10)
-  dim3 grid((unsigned)std::max<int64_t>(1, std::min<int64_t>(8, f->L.P / 2 / kThreads)), batch);
+  // enough blocks for the GPU and no more, so that each thread has several loads in flight (64 blocks
+  // per sample: 27 us at 64 x 256^2, 8: 10; 8 at 1 x 1024^2: 66, 64: 47)
+  const int64_t most = std::max<int64_t>(8, std::min<int64_t>(64, 608 / batch));
+  dim3 grid((unsigned)std::min<int64_t>(most, (2 * f->L.P + kThreads - 1) / kThreads), batch);
   infection_scale_kernel<<<grid, kThreads, 0, f->stream>>>(u, smax, f->L.P);
   CK(cudaGetLastError(), "infection scale");
   make_input_kernel<<<dim3(rows_grid(f->L.P), batch), kThreads, 0, f->stream>>>(u, r0, logd, smax, x, f->L.P);
