@@ -338,19 +338,6 @@ int upload_table(sslbm_ensemble* e) {
   return SSLBM_OK;
 }
 
-// Default segment length: the longest (least pipeline fill) that still gives every resident CTA a
-// tile of each step-block.  32 scenarios of 256^2 to 1024^2, 200 steps: 128 rows 4.9 ms (750 tiles
-// for 608 CTAs), 64 rows 5.5, 256 rows 7.1 (400 tiles).
-int default_seg_rows(const sslbm_ensemble* e, int ctas) {
-  const int hl = (e->depth + 3) / 4, wv = 128 - 8 * hl;
-  for (int seg : {256, 128, 64, 32}) {
-    int64_t tiles = 0;
-    for (const sslbm_scenario& s : e->sc) tiles += (s.nx + wv - 1) / wv * ((s.ny + seg - 1) / seg);
-    if (tiles >= ctas) return seg;
-  }
-  return 4 * e->depth;
-}
-
 int resident_ctas(EnsKernel kern, int depth, int precision, int* out) {
   int dev = 0, sms = 0, per = 0;
   cudaError_t ce = cudaGetDevice(&dev);
@@ -368,13 +355,37 @@ int resident_ctas(EnsKernel kern, int depth, int precision, int* out) {
   return SSLBM_OK;
 }
 
+EnsKernel ensemble_kernel_of(const sslbm_ensemble* e) {
+  return e->precision == SSLBM_FP32_DEV     ? pick_kernel<sslbm::MODE_DEV>(e->depth)
+         : e->precision == SSLBM_FP32_SPLIT ? pick_kernel<sslbm::MODE_SPLIT>(e->depth)
+                                            : pick_kernel<sslbm::MODE_PLAIN>(e->depth);
+}
+
+// Default segment length, by the tiles it makes and the CTAs resident at once: 64 rows, longer (less
+// pipeline fill) while every resident CTA still gets a tile of each step-block, shorter where the tiles
+// would take half of the CTAs.  us for 40 steps at 64 rows and at the length chosen, FP32 (608 CTAs): 32
+// scenarios of 256^2 to 1024^2 1133 and 1032 (128 rows), 2 x 4096^2 2939 and 2530 (256), 300 x 64^2 369 and 291
+// (32), 2 x 512^2 435 and 195 (16); 64 rows stay for 2048^2 (463; 32: 550), 4 x 1024^2 (469; 32: 492), 8 x 1000^2 (772;
+// 128: 815); split (456 CTAs): 8 x 1000^2 1067 and 984 (128), 300 x 64^2 428 (32: 401, 16: 550).
+int default_seg_rows(const sslbm_ensemble* e, int ctas) {
+  const int hl = (e->depth + 3) / 4, wv = 128 - 8 * hl;
+  auto tiles = [&](int seg) {
+    int64_t t = 0;
+    for (const sslbm_scenario& s : e->sc) t += (s.nx + wv - 1) / wv * ((s.ny + seg - 1) / seg);
+    return t;
+  };
+  if (tiles(256) >= ctas) return 256;
+  if (tiles(128) >= ctas) return 128;
+  int seg = 64;
+  while (seg > 4 * e->depth && 2 * tiles(seg) <= ctas) seg /= 2;
+  return seg;
+}
+
 // Enqueue nblocks step-blocks of depth e->depth (counters reset first), captured once in a
 // CUDA graph and replayed.
 int launch_blocks(sslbm_ensemble* e, int nblocks) {
   if (nblocks <= 0) return SSLBM_OK;
-  EnsKernel kern = e->precision == SSLBM_FP32_DEV     ? pick_kernel<sslbm::MODE_DEV>(e->depth)
-                    : e->precision == SSLBM_FP32_SPLIT ? pick_kernel<sslbm::MODE_SPLIT>(e->depth)
-                                                       : pick_kernel<sslbm::MODE_PLAIN>(e->depth);
+  EnsKernel kern = ensemble_kernel_of(e);
   if (!kern) return err(SSLBM_ERR_BAD_ARG, "depth %d has no ensemble kernel", e->depth);
   if (!(e->exec && e->exec_blocks == nblocks && e->exec_cur == e->cur && e->exec_depth == e->depth)) {
     if (e->exec) {
@@ -480,14 +491,12 @@ int sslbm_ensemble_create(int n, const sslbm_scenario* sc, int precision, void* 
     delete e;
     return cuda_err(ce, "cudaMemsetAsync(workspace)");
   }
-  int sms = 0;
-  ce = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, e->device);
-  if (ce != cudaSuccess) {
-    delete e;
-    return cuda_err(ce, "cudaDeviceGetAttribute");
+  int ctas = 0;
+  st = resident_ctas(ensemble_kernel_of(e), e->depth, e->precision, &ctas);
+  if (st == SSLBM_OK) {
+    e->seg_rows = default_seg_rows(e, ctas);
+    st = upload_table(e);
   }
-  e->seg_rows = default_seg_rows(e, 4 * sms);
-  st = upload_table(e);
   if (st) {
     delete e;
     return st;
