@@ -233,7 +233,7 @@ int sslbm_set_diffusivity_scale(sslbm_handle* h, const void* kx, const void* ky,
  * replayed advances the state again only if the state is back in the buffer it was captured on.  Calls
  * of an even number of passes leave it there: n passes where the kernel takes one step each, else
  * ceil(n / depth) with the depth of sslbm_get_blocking.  Under the default blocking of a kernel that takes
- * several steps a captured call of n >= 2 makes an even number of passes, and later calls a number of
+ * several steps (or the autotuner's choice of its tile passes) a captured call of n >= 2 makes an even number of passes, and later calls a number of
  * the parity of ceil(n / depth).
  * Enqueues on the handle's stream and returns. */
 int sslbm_step(sslbm_handle* h, int64_t n);
@@ -368,7 +368,10 @@ int sslbm_set_blocking(sslbm_handle* h, int k, int seg_rows);
  * and write the spare buffer, so the state is left unchanged.  budget_ms bounds the search
  * (0 = 300 ms).  The choice is cached per (device, nx, ny, precision, lattice, boundary)
  * for the life of the process, applied to the
- * handle, and returned through depth, seg_rows and ms_per_step (each may be NULL).
+ * handle, and returned through depth, seg_rows and ms_per_step (each may be NULL): one configuration
+ * and its time, which sslbm_set_blocking(depth, seg_rows) reproduces and sslbm_get_blocking returns.
+ * Where the register-tile passes of the default blocking measured faster still, sslbm_step on
+ * this handle takes those wherever it would by default (the same bits).
  * Synchronises the stream.  Not part of the paper (which gives no implementation). */
 int sslbm_autotune(sslbm_handle* h, double budget_ms, int* depth, int* seg_rows,
                    double* ms_per_step);

@@ -940,7 +940,7 @@ struct TuneKey {
 struct TuneResult {
   int depth, seg_rows;
   double ms_per_step;
-  bool tiles;  // the tile passes of the default blocking
+  bool tiles;  // the tile passes of the default blocking were faster still
 };
 std::mutex g_tune_mu;
 std::map<TuneKey, TuneResult> g_tune_cache;
@@ -1036,10 +1036,9 @@ int sslbm_autotune(sslbm_handle* h, double budget_ms, int* depth_out, int* seg_o
     }
     cudaEventDestroy(e0);
     cudaEventDestroy(e1);
-    if (tile_ms < best.ms_per_step) {  // depth and segment stay the pipeline's best, for steps that take no tiles
-      best.ms_per_step = tile_ms;
-      best.tiles = true;
-    }
+    // depth, segment and time stay the pipeline's best, one configuration that sslbm_set_blocking
+    // reproduces; sslbm_step takes the tile passes where they are faster still
+    best.tiles = tile_ms < best.ms_per_step;
     std::lock_guard<std::mutex> lock(g_tune_mu);
     g_tune_cache[key] = best;
   }
