@@ -506,10 +506,10 @@ int sslbm_fd4_set_order(sslbm_fd4* f, int order);
  * {R_l[W][W][2m][m][2], B_l[W][W], b_l[W]}_{l=1..L}, Q1[H][W], q1[H], Q2[5][H], q2[5].
  * Dense contractions run on BF16 tensor cores with FP32 accumulation; activations are
  * BF16, parameters, gradients and Adam moments FP32.  For (W, m, H) = (32, 12, 64) or
- * (16, 8, 32) and n in {64, 128, 256} the forward pass runs as fused per-row kernels
+ * (16, 8, 32) and n in {64, 128, 256} the forward and the backward pass run as fused per-row kernels
  * (sslbm_fno_fused() says which); other shapes use one product per contraction.  All
  * tensors passed in are device pointers, FP32, laid out [batch][channel][n][n], 16-byte
- * aligned. */
+ * aligned (an x that is not returns SSLBM_ERR_BAD_ARG where n is even). */
 typedef struct sslbm_fno_config {
   int32_t n;          /* grid side (periodic), 2 * modes <= n */
   int32_t width;      /* W: channels of the hidden layers (<= 64) */
@@ -540,7 +540,7 @@ int sslbm_fno_forward(sslbm_fno* f, int batch, const float* x, float* y);
 /* The same y without keeping the activations (the rollout's call; a following backward
  * pass returns SSLBM_ERR_STATE). */
 int sslbm_fno_infer(sslbm_fno* f, int batch, const float* x, float* y);
-/* 1 when this configuration runs the fused forward kernels, 0 otherwise, < 0 on error. */
+/* 1 when this configuration runs the fused forward and backward kernels, 0 otherwise, < 0 on error. */
 int sslbm_fno_fused(const sslbm_fno* f);
 /* Parameter gradients of a scalar loss with dL/dy = dy, after sslbm_fno_forward on x with
  * the same batch (SSLBM_ERR_STATE otherwise). */
@@ -559,7 +559,9 @@ int sslbm_fno_set_loss_weights(sslbm_fno* f, float mass_weight, float neg_weight
  * issue neither their MMAs nor the completion signal, so every wait runs out with no
  * tensor-core work in flight, the products write NaN and sslbm_fno_train_step returns
  * SSLBM_ERR_TIMEOUT instead of hanging.  The paper has no counterpart.  A product whose
- * wait runs out drains its MMAs (one more bounded wait) before it frees its tensor memory. */
+ * wait runs out drains its MMAs (one more bounded wait) before it frees its tensor memory.
+ * The fused kernels have no such waits, so polls matters only where sslbm_fno_fused() is 0; with
+ * stall != 0 the backward pass of every configuration takes the products. */
 int sslbm_fno_set_wait_limit(sslbm_fno* f, long long polls, int stall);
 /* One training step on the loss of sslbm_fno_set_loss_weights: forward, loss, backward,
  * Adam with learning rate lr.  y_scratch and dy_scratch are [batch][5][n][n] device
