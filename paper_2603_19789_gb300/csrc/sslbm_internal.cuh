@@ -10,6 +10,7 @@
 #include <cuda_runtime.h>
 #include <stdint.h>
 
+#include "quot_range.cuh"
 #include "sslbm.h"
 
 namespace sslbm {
@@ -111,13 +112,11 @@ __device__ __forceinline__ float force_quot(float num, float Nc) {
 }
 __device__ __forceinline__ double force_quot(double num, double Nc) {
   const int hi = __double2hiint(Nc);
-  // sign bit clear and 2^-99 <= Nc < 2^99 (NaN, infinities, zero and negative values fail it)
-  if ((unsigned)(hi - ((1023 - 99) << 20)) >= (unsigned)(198 << 20))
-    return __ddiv_rn(num, fmax(Nc, 2.2250738585072014e-308));
+  if (!quot_in_range(hi)) return __ddiv_rn(num, fmax(Nc, 2.2250738585072014e-308));
   // the float with Nc's exponent and its leading 23 fraction bits, and back
   const float f = __int_as_float(__funnelshift_l(__double2loint(Nc), hi - ((1023 - 127) << 20), 3));
   const int rb = __float_as_int(rcp_approx(f));
-  double r = __hiloint2double((rb >> 3) + ((1023 - 127) << 20), rb << 29);
+  double r = __hiloint2double(quot_hi(rb), quot_lo(rb));
   r = __fma_rn(r, __fma_rn(-Nc, r, 1.0), r);
   const double q = __dmul_rn(num, r);
   return __fma_rn(r, __fma_rn(-Nc, q, num), q);
