@@ -10,10 +10,12 @@
 // are never read.  The operations and their order are those of bgk_step_kernel, so a pass gives
 // the bits of K of its launches.
 //
-// What bounds it: HBM.  One step per launch moves 168 bytes per cell and step (39.5 GLUPS is 99% of
-// HBM); a pass moves the same once for K steps, plus the halo's reads from L2.  Per step, one
-// step per launch and four per pass: 2048^2 107.6 and 57.1 us, 4096^2 419 and 221 (76 GLUPS), 200^2 4.3
-// and 2.3; two steps 72.9 at 2048^2, three 58.3, six 57.1.
+// What bounds it: one step per launch moves 168 bytes per cell and step (39.5 GLUPS is 99% of HBM); a
+// pass moves the same once for K steps, 42 bytes per cell and step at four, which is 46% of HBM at
+// 2048^2.  The rest is instruction issue (170 operations per cell and step, half of them on packed
+// pairs, on a third more cells than are written) and the exchange of each step, so deeper passes gain
+// nothing.  Per step, one step per launch and four per pass: 2048^2 107.6 and 57.1 us, 4096^2 419 and 221 (76
+// GLUPS), 200^2 4.3 and 2.3; two steps 72.9 at 2048^2, three 58.3, six 57.1.
 #include <cuda_runtime.h>
 
 #include "bounds.cuh"

@@ -82,10 +82,12 @@ __global__ void __launch_bounds__(kStep1Threads) step1_kernel(const GridView g, 
 }
 
 // Small grids (at most kStep1Threads cells per SM): one CTA per SM with an equal share of the cells,
-// and enough shared memory reserved that an SM holds two, one of this launch and one of the next:
-// with small CTAs the dependent launch's go where there is room and some SMs get twice the work
-// (200^2, us per step: 10.3 with 64 x 8 blocks of two cells, 8.2 with 64-thread CTAs, 10.6 with
-// those and dependent launches, 5.2 with even shares).  Only a step after a step is a dependent
+// and enough shared memory reserved that an SM holds no more than two, one of this launch and one of
+// the next: with small CTAs the dependent launch's go where there is room and some SMs get twice the
+// work (200^2, us per step: 10.3 with 64 x 8 blocks of two cells, 8.2 with 64-thread CTAs, 10.6 with
+// those and dependent launches, 5.2 with even shares).  Above 576 cells per SM (about 296^2) the
+// registers, 56 per thread, leave room for one CTA, and the next launch starts when it ends; even
+// shares stay ahead of 64-thread CTAs to the limit: 350^2 11.1 and 14.4, 394^2 13.3 and 14.5.  Only a step after a step is a dependent
 // launch: after another kernel, two CTAs may go to one SM, and stay together from step to step (8.0).
 // Larger grids: 64-thread CTAs.
 cudaError_t launch_step1_fp64(const GridView& g, const void* coeffs, const void* in, void* out, bool chained,
