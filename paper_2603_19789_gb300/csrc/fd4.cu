@@ -177,7 +177,8 @@ __global__ void __launch_bounds__(kTX * kTY) fd4_stage_kernel(int64_t nx, int64_
 // evaluations per cell (TY = 16), and latency; the separate stages moved 85 planes a step through
 // HBM or L2 (340 bytes per cell), this moves 32.
 // Four separate stages and these, us per step: 200^2 25.7 and 19.0, 1000^2 79.7 and 58.5, 2048^2 314
-// and 176, 8192^2 4476 and 2462 (27.3 GLUPS; issue 59% busy, 200 instructions per cell and stage).
+// and 176, 8192^2 4476 and 2462 (27.3 GLUPS; issue 59% busy, 200 instructions per cell and stage); widths
+// that are no multiple of four, moved cell by cell: 1023 x 1025 78 and 73, 2047 x 2049 375 and 244.
 // The loads of u and acc wait for HBM if issued where they are used (8192^2 3117); they are
 // requested before the right-hand sides.
 // ghost2 in 32-bit arithmetic, the wrap by one fold without a division on all but tiny grids (with

@@ -29,8 +29,8 @@ namespace sslbm {
 
 // Rows and columns inside a tile (a side is at most 2^30).  In 32 bits, the index arithmetic of
 // warp 0, which also copies the level-0 rows and which the other warps wait for, is shorter:
-// us per step at 8192^2, varying diffusion 315 -> 279 at depth 6, Kahan 437 -> 414 at depth 8,
-// D2Q9 no-flux 245 -> 222 at depth 4.  The plain, deviation and split storages keep 64 bits: the
+// us per step at 8192^2, with the dependent launches that came beside it, varying diffusion 319 -> 247 at
+// depth 6, Kahan 437 -> 410 at depth 8, D2Q9 no-flux 246 -> 224 at depth 4.  The plain, deviation and split storages keep 64 bits: the
 // compiler's schedule of their lighter rows came out slower with 32 (plain 153 -> 162 at depth 4,
 // split 191 -> 202 at depth 8).
 template <int MODE>

@@ -14,9 +14,9 @@
 // per step the FP32 arithmetic of the region's rows, halo included (0.38 us for 16 rows, 0.44 for
 // 32, 0.77 for 64; 0.35 at 100% of the FP32 pipes for 64).  The row pipeline needs one barrier per
 // two rows and 12 rows of fill whatever the grid, so a 128^2 pass of 4 steps takes 16.5 us there;
-// here 14 steps take 9.7.  Per step, pipeline (default depth) and tiles: 128^2 4.1 and 0.69 us,
-// 512 x 640 4.6 and 1.55, 1001 x 777 5.1 and 2.9, 1201^2 6.7 and 5.5, 2048^2 12.8 and 16.7; D2Q9
-// with walls 1500 x 1100 19.8 and 10.7.  Passes use programmatic dependent launch: the next one
+// here 14 steps take 9.7.  us per step of 40, pipeline (depth 4, without dependent launches) and tiles:
+// 128^2 4.1 and 0.64, 512^2 4.6 and 1.2, 1000^2 5.9 and 3.7; 2048^2, where the pipeline stays ahead, 12.8 and
+// 16.7; D2Q9 with walls 1500 x 1100 19.8 and 10.7; varying diffusion 1000^2 9.2 and 6.6.  Passes use programmatic dependent launch: the next one
 // is resident and has its indices ready when the current one ends.
 #include <cuda_runtime.h>
 
