@@ -467,34 +467,48 @@ __device__ __forceinline__ void two_sum_add(float& hi, float& lo, float x) {
   hi = s;
 }
 
-// A thread's sum: a TwoSum pair, renormalised by its owner every few values so that its low part keeps
-// FP32's unit roundoff squared, and beside it in FP64 what the pair cannot hold exactly -- terms that could
-// overflow it, infinities and NaN, and squares whose rounding error would underflow.
+// A thread's sum, four terms at a time: a TwoSum pair, renormalised after them so that its low part keeps
+// FP32's unit roundoff squared, and beside it in FP64 the groups that the pair cannot hold exactly -- with
+// terms that could overflow it, infinities, NaN, or squares whose rounding error would underflow.
 struct PairSum {
   float hi = 0.f, lo = 0.f;
   double wide = 0.0;
-  __device__ __forceinline__ void add(float v) {
-    if (fabsf(v) <= 0x1p100f)
-      two_sum_add(hi, lo, v);
-    else
-      wide += (double)v;
-  }
-  __device__ __forceinline__ void add_square(float v) {
-    const float a = fabsf(v);
-    if (a <= 0x1p50f && (a >= 0x1p-50f || a == 0.f)) {
-      const float sq = __fmul_rn(v, v);
-      two_sum_add(hi, lo, sq);
-      lo = __fadd_rn(lo, __fmaf_rn(v, v, -sq));
+  __device__ __forceinline__ void add4(float a, float b, float c, float d) {
+    const float m = fmaxf(fmaxf(fabsf(a), fabsf(b)), fmaxf(fabsf(c), fabsf(d)));
+    // a NaN hides from the maxima, but not from the sum of the magnitudes' zeros
+    if (m <= 0x1p100f && 0.f * a + 0.f * b + 0.f * c + 0.f * d == 0.f) {
+      two_sum_add(hi, lo, a), two_sum_add(hi, lo, b), two_sum_add(hi, lo, c), two_sum_add(hi, lo, d);
+      renormalise();
     } else {
-      wide += (double)v * (double)v;
+      wide += ((double)a + (double)b) + ((double)c + (double)d);
     }
+  }
+  __device__ __forceinline__ void add_squares4(float a, float b, float c, float d) {
+    if (square_ok(a) && square_ok(b) && square_ok(c) && square_ok(d)) {
+      square(a), square(b), square(c), square(d);
+      renormalise();
+    } else {
+      wide += ((double)a * a + (double)b * b) + ((double)c * c + (double)d * d);
+    }
+  }
+  __device__ __forceinline__ double total() const { return ((double)hi + (double)lo) + wide; }
+
+ private:
+  // 0 or 2^-50 <= |v| <= 2^50: the square and its rounding error are exact in a pair
+  static __device__ __forceinline__ bool square_ok(float v) {
+    const unsigned m = __float_as_uint(v) & 0x7fffffffu;
+    return m == 0u || m - ((127u - 50u) << 23) <= (100u << 23);
+  }
+  __device__ __forceinline__ void square(float v) {
+    const float sq = __fmul_rn(v, v);
+    two_sum_add(hi, lo, sq);
+    lo = __fadd_rn(lo, __fmaf_rn(v, v, -sq));
   }
   __device__ __forceinline__ void renormalise() {
     const float t = __fadd_rn(hi, lo), bp = __fsub_rn(t, hi);
     lo = __fadd_rn(__fsub_rn(hi, __fsub_rn(t, bp)), __fsub_rn(lo, bp));
     hi = t;
   }
-  __device__ __forceinline__ double total() const { return ((double)hi + (double)lo) + wide; }
 };
 
 // per sample b = blockIdx.y: sums[3b] += sum (y - t), sums[3b+1] += sum t, sums[3b+2] += sum max(-y, 0).
@@ -506,23 +520,21 @@ __global__ void loss_sums_kernel(const float* __restrict__ y, const float* __res
   __shared__ double sh[64];
   const int64_t b = blockIdx.y;
   PairSum se, st, sn;
-  auto take = [&](float yv, float tv) {
-    se.add(yv - tv);
-    st.add(tv);
-    if (yv < 0.f) sn.add(-yv);
+  auto take = [&](float4 y, float4 t) {
+    se.add4(y.x - t.x, y.y - t.y, y.z - t.z, y.w - t.w);
+    st.add4(t.x, t.y, t.z, t.w);
+    if (y.x < 0.f || y.y < 0.f || y.z < 0.f || y.w < 0.f)
+      sn.add4(y.x < 0.f ? -y.x : 0.f, y.y < 0.f ? -y.y : 0.f, y.z < 0.f ? -y.z : 0.f, y.w < 0.f ? -y.w : 0.f);
   };
-  auto renormalise = [&]() { se.renormalise(), st.renormalise(), sn.renormalise(); };
   const float* yb = y + b * P5;
   const float* tb = tgt + b * P5;
   const int64_t stride = (int64_t)gridDim.x * blockDim.x, i0 = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
   if ((P5 & 3) == 0 && ((reinterpret_cast<uintptr_t>(yb) | reinterpret_cast<uintptr_t>(tb)) & 15) == 0) {
     for (int64_t i = i0; i < P5 / 4; i += stride) {
-      const float4 yv = reinterpret_cast<const float4*>(yb)[i], tv = reinterpret_cast<const float4*>(tb)[i];
-      take(yv.x, tv.x), take(yv.y, tv.y), take(yv.z, tv.z), take(yv.w, tv.w);
-      renormalise();
+      take(reinterpret_cast<const float4*>(yb)[i], reinterpret_cast<const float4*>(tb)[i]);
     }
   } else {
-    for (int64_t i = i0; i < P5; i += stride) take(yb[i], tb[i]), renormalise();
+    for (int64_t i = i0; i < P5; i += stride) take(make_float4(yb[i], 0.f, 0.f, 0.f), make_float4(tb[i], 0.f, 0.f, 0.f));
   }
   block_add2(se.total(), st.total(), sums + 3 * b, sh);
   __syncthreads();
@@ -558,9 +570,8 @@ __global__ void loss_kernel(const float* __restrict__ y, const float* __restrict
     const float* yb = y + (b * 5 + c) * P;
     const float* tb = tgt + (b * 5 + c) * P;
     float* db = dy + (b * 5 + c) * P;
-    auto one = [&](float yv, float tv) {
-      const float dn = (yv - tv) * rs;
-      sum.add_square(dn);
+    auto one = [&](float yv, float tv, float& dn) {
+      dn = (yv - tv) * rs;
       float g = 2.f * dn * rs * inv + gm;
       if (yv < 0.f) g -= gn;
       return g;
@@ -569,11 +580,17 @@ __global__ void loss_kernel(const float* __restrict__ y, const float* __restrict
                           reinterpret_cast<uintptr_t>(db)) & 15) == 0) {
       for (int64_t i = i0; i < P / 4; i += stride) {
         const float4 yv = reinterpret_cast<const float4*>(yb)[i], tv = reinterpret_cast<const float4*>(tb)[i];
-        reinterpret_cast<float4*>(db)[i] = make_float4(one(yv.x, tv.x), one(yv.y, tv.y), one(yv.z, tv.z), one(yv.w, tv.w));
-        sum.renormalise();
+        float4 d;
+        reinterpret_cast<float4*>(db)[i] =
+            make_float4(one(yv.x, tv.x, d.x), one(yv.y, tv.y, d.y), one(yv.z, tv.z, d.z), one(yv.w, tv.w, d.w));
+        sum.add_squares4(d.x, d.y, d.z, d.w);
       }
     } else {
-      for (int64_t i = i0; i < P; i += stride) db[i] = one(yb[i], tb[i]), sum.renormalise();
+      for (int64_t i = i0; i < P; i += stride) {
+        float d;
+        db[i] = one(yb[i], tb[i], d);
+        sum.add_squares4(d, 0.f, 0.f, 0.f);
+      }
     }
   }
   block_add1(sum.total() / (double)N, loss, sh);
