@@ -269,8 +269,8 @@ int64_t sslbm_steps_done(const sslbm_handle* h, int scheme);
 
 /* Not part of the paper's method; a checking facility of this library.
  * Compiled with SSLBM_BOUNDS_CHECK (libsslbm_check.so, built by build.py --checked), the
- * hot-path kernels -- the fused pipeline tile of sslbm_step and the ensemble, the one-step
- * kernel, the BGK step and the diagnostics -- test the row and column indices of their
+ * hot-path kernels -- the fused pipeline tile of sslbm_step and the ensemble, the register
+ * tiles, the one-step kernel, the BGK step and the diagnostics -- test the row and column indices of their
  * global loads and stores against the grid before each access, skip an access whose index
  * is out of range and record it.  sslbm_debug_bounds synchronises the current device,
  * returns the number of such indices since the last call, the first one, the limit it
@@ -409,7 +409,7 @@ void sslbm_ensemble_destroy(sslbm_ensemble* e);
 
 /* Tile shape of the persistent launch: steps fused per pass (depth in {2..6, 8}) and the
  * row-segment length of a tile (>= 4 * depth); the tile width is one 128-column strip.  Without
- * this call: depth 4 and a segment length by the scenarios' sizes. */
+ * this call: depth 4 and a segment length by the scenarios' sizes and the CTAs resident at once. */
 int sslbm_ensemble_set_tiling(sslbm_ensemble* e, int depth, int seg_rows);
 int sslbm_ensemble_get_tiling(const sslbm_ensemble* e, int* depth, int* seg_rows);
 
@@ -479,7 +479,9 @@ void sslbm_fd4_destroy(sslbm_fd4* f);
 /* The whole state, [5][ny][nx] FP64 or FP32, host or device; host transfers synchronise. */
 int sslbm_fd4_write(sslbm_fd4* f, const void* src, int src_dtype, int src_on_device);
 int sslbm_fd4_read(sslbm_fd4* f, void* dst, int dst_dtype, int dst_on_device);
-/* n RK4 steps of dt (four stage launches each, in FP32 two launches of two stages), stream-ordered. */
+/* n RK4 steps of dt, stream-ordered: four stage launches each, in FP32 two launches of two stages on grids
+ * where those are faster.  The state is the workspace's first five planes after every call, so a captured
+ * call can be replayed for any n. */
 int sslbm_fd4_step(sslbm_fd4* f, int64_t n);
 int64_t sslbm_fd4_steps_done(const sslbm_fd4* f);
 /* Order of the Laplacian: 4 (default, the reference) or 2, the second-order centred
