@@ -31,6 +31,9 @@ static_assert(pipe_smem_bytes<MODE_VARD, 6>() == pipe_bytes(5, 6, true) &&
                   pipe_smem_bytes<MODE_PLAIN, 3>() == pipe_bytes(5, 3, false),
               "pass_plan.cuh: pipe_bytes");
 
+// Columns written per strip at depth K (128 computed, K of halo on each side rounded up to lanes).
+__host__ __device__ constexpr int64_t pipe_strip_cols(int K) { return 128 - 8 * ((K + 3) / 4); }
+
 // kx, ky: the scale planes of the varying-diffusion lattice (MODE_VARD), else unused.
 // DIAG: also the diagnostics partial of the CTA's output cells into diag[6 blockIdx.x ...].
 template <int MODE, int K, bool DIAG = false>
@@ -53,8 +56,11 @@ __global__ void __launch_bounds__(32 * K, MODE == MODE_KAHAN ? 1 : 16 / K) pipe_
     DiagSmem<NF>* dsm = reinterpret_cast<DiagSmem<NF>*>(pipe_smem + sizeof(PipeSmem<K, NF>));
     pipe_tile<MODE, K, false, true, true>(sm, g, k, in, out, strip, y0, y1, nullptr, nullptr, nullptr, dsm, diag,
                                           (int)blockIdx.x);
-  } else if ((MODE == MODE_D2Q9_NOFLUX || MODE == MODE_D2Q9_NOFLUX4) && strip != 0 && strip != nstrips - 1) {
-    pipe_tile<MODE, K, false, false>(sm, g, k, in, out, strip, y0, y1);  // no wall column in this strip
+  } else if ((MODE == MODE_D2Q9_NOFLUX || MODE == MODE_D2Q9_NOFLUX4) && strip != 0 &&
+             (int64_t)(strip + 1) * pipe_strip_cols(K) <= g.nx - K) {
+    // K steps carry neither wall column to a column that this strip writes.  (The strip before the last
+    // needs the wall code too where the last is narrower than K columns.)
+    pipe_tile<MODE, K, false, false>(sm, g, k, in, out, strip, y0, y1);
   } else {
     pipe_tile<MODE, K>(sm, g, k, in, out, strip, y0, y1, kx, ky, rk);
   }
@@ -75,9 +81,6 @@ void prefer_shared() {
                        (int)pipe_smem_bytes<MODE, K, DIAG>());
   done.fetch_or(bit, std::memory_order_release);
 }
-
-// Columns written per strip at depth K (128 computed, K of halo on each side rounded up to lanes).
-constexpr int64_t pipe_strip_cols(int K) { return 128 - 8 * ((K + 3) / 4); }
 
 // DIAG: diag receives one 6-double partial per CTA (at most kDiagBlocks CTAs).
 template <int MODE, int K, bool DIAG = false>

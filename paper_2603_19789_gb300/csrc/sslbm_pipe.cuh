@@ -447,8 +447,8 @@ __device__ __forceinline__ void pipe_pair(PipeSmem<K, NF>& sm, const GridView& g
 // included, are one contiguous 16-byte group at the wrapped position, so all loads are
 // L2-only cp.async.cg (required when other CTAs of the same launch wrote the input, since
 // L1 is not coherent).
-// COLW = false: the strip holds neither x = 0 nor x = nx - 1 (D2Q9 no-flux: no column wall
-// code in its rows).
+// COLW = false: neither x = 0 nor x = nx - 1 is within K columns of the strip's output (D2Q9 no-flux:
+// no column wall code in its rows).
 // DIAG (five planes): also the totals of the five output planes over the tile's output cells
 // and their largest I, written as FP64 partial `diag_slot` of diag (6 doubles: the totals,
 // then the peak), with dsm as the diagnostics' shared memory.
